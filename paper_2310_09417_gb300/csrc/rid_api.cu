@@ -95,12 +95,13 @@ struct Plan {
   size_t wsz = 0;        // bytes per Omega element
   size_t off_state = 0, off_omega = 0, off_G = 0, off_Gpart = 0, off_S = 0, off_Spart = 0, off_N = 0,
          off_Linv = 0, off_act0 = 0, off_act1 = 0, off_pivmark = 0, off_perm32 = 0, off_piv = 0,
-         off_pivorig = 0, off_pivdiag = 0, off_cand_v = 0, off_cand_i = 0, off_cand_rows = 0, off_e2 = 0,
+         off_pivorig = 0, off_pivdiag = 0, off_xchg = 0, off_e2 = 0,
          off_normp = 0, off_trace = 0, off_digits = 0, off_colexp = 0, total = 0;
   // condition of L1 / FP64 solve for X (opts->x_solve_f64)
   int64_t ldl = 0;
   size_t off_L = 0, off_L1 = 0, off_T64 = 0, off_Linv64 = 0, off_iota = 0, off_csum = 0;
   // path 65: digit slices of N and T(piv, old) for the tensor-core block update
+  size_t xchg_bytes = 0;  // the panel's exchange words
   size_t off_ndig = 0, off_nexp = 0, off_pdig = 0, off_pexp = 0;
   // path 65: digit slices of T(act, 0:tb) and G(perm, cols) for the tensor-core Schur GEMM
   size_t off_adig = 0, off_aexp = 0, off_bdig = 0, off_bexp = 0, off_colmax = 0;
@@ -265,9 +266,8 @@ int make_plan(const id_matrix* A, const id_opts* o, int64_t k, int64_t l, Plan* 
   p->off_piv = take((size_t)kMaxBlock * 4);
   p->off_pivorig = take((size_t)kMaxBlock * 4);
   p->off_pivdiag = take((size_t)kMaxBlock * 8);
-  p->off_cand_v = take((size_t)2 * p->maxg * 8);
-  p->off_cand_i = take((size_t)2 * p->maxg * 4);
-  p->off_cand_rows = take((size_t)2 * p->maxg * p->wmax * e);
+  p->xchg_bytes = align_up(panel_xchg_bytes(p->maxg, p->wmax, e));
+  p->off_xchg = take(p->xchg_bytes);
   p->off_e2 = take((size_t)p->nparts * 8);
   p->off_normp = take((size_t)p->nparts * 8);
   p->off_trace = take((size_t)p->max_rounds * 8);
@@ -348,9 +348,7 @@ class Engine {
     piv_ = reinterpret_cast<int32_t*>(w + p.off_piv);
     pivorig_ = reinterpret_cast<int32_t*>(w + p.off_pivorig);
     pivdiag_ = reinterpret_cast<double*>(w + p.off_pivdiag);
-    cand_v_ = reinterpret_cast<double*>(w + p.off_cand_v);
-    cand_i_ = reinterpret_cast<int32_t*>(w + p.off_cand_i);
-    cand_rows_ = reinterpret_cast<T*>(w + p.off_cand_rows);
+    xchg_ = w + p.off_xchg;
     e2_ = reinterpret_cast<double*>(w + p.off_e2);
     normp_ = reinterpret_cast<double*>(w + p.off_normp);
     trace_ = reinterpret_cast<double*>(w + p.off_trace);
@@ -470,9 +468,8 @@ class Engine {
     // the fixed-rank estimate set the stop flag; the extra steps must run
     RID_TRY(cuda(cudaMemsetAsync(&st_->done, 0, sizeof(int32_t), s_)));
     PanelCfg cfg = panel_config<T>((int)na, (int)p, p_.maxg);
-    RID_TRY(cuda(panel_lupp<T>(cfg, (int)na, (int)p, (int)p, panel_par_, S_, p_.wmax, piv_, pivmark_, pivdiag_,
-                               cand_v_, cand_i_, cand_rows_, st_, s_)));
-    panel_par_ ^= 1;
+    RID_TRY(cuda(panel_lupp<T>(cfg, (int)na, (int)p, (int)p, panel_seq_++, S_, p_.wmax, piv_, pivmark_, pivdiag_,
+                               xchg_, st_, s_)));
     RID_TRY(cuda(ur_extract<T>((int)p, (int)na, S_, p_.wmax, piv_, act_[cur_], U, ldu, Jx, e2_, s_)));
     RID_TRY(tend(2));
     RID_TRY(cuda(cudaMemcpyAsync(stats, e2_, 2 * sizeof(double), cudaMemcpyDeviceToHost, s_)));
@@ -487,8 +484,8 @@ class Engine {
   // pivoted for k steps, and the interpolation coefficients land in the X buffer.
   int run_panel(const T* src, int64_t m_src, int64_t n_src, int64_t ld_src, const int64_t* J) {
     RID_TRY(tbegin(ID_PHASE_OTHER));
-    RID_TRY(cuda(init_state(st_, act_[0], pivmark_, p_.n, s_)));
-    panel_par_ = 0;  // both barrier counters were cleared
+    RID_TRY(cuda(init_state(st_, act_[0], pivmark_, p_.n, xchg_, p_.xchg_bytes, s_)));
+    panel_seq_ = 0;  // the exchange words were cleared
     RID_TRY(cuda(gather_panel<T>(src, ld_src, m_src, n_src, J, p_.k, G_, st_, s_)));
     RID_TRY(tend(2));
     int64_t tb = 0, na = p_.n;
@@ -542,8 +539,8 @@ class Engine {
 
   int start() {
     RID_TRY(tbegin(ID_PHASE_OTHER));
-    RID_TRY(cuda(init_state(st_, act_[0], pivmark_, p_.n, s_)));
-    panel_par_ = 0;  // both barrier counters were cleared
+    RID_TRY(cuda(init_state(st_, act_[0], pivmark_, p_.n, xchg_, p_.xchg_bytes, s_)));
+    panel_seq_ = 0;  // the exchange words were cleared
     if (p_.path == 8)
       RID_TRY(cuda(norm2_fp8(p_.m, p_.n, Araw_, lda_, scale_, normp_, p_.nparts, st_, s_)));
     else if (p_.path == 16)
@@ -814,9 +811,8 @@ class Engine {
     const int64_t lds = p_.wmax;
     RID_TRY(tbegin(ID_PHASE_LU));
     PanelCfg cfg = panel_config<T>((int)na, (int)w, p_.maxg);
-    RID_TRY(cuda(panel_lupp<T>(cfg, (int)na, (int)w, (int)bt, panel_par_, S_, lds, piv_, pivmark_, pivdiag_,
-                               cand_v_, cand_i_, cand_rows_, st_, s_)));
-    panel_par_ ^= 1;
+    RID_TRY(cuda(panel_lupp<T>(cfg, (int)na, (int)w, (int)bt, panel_seq_++, S_, lds, piv_, pivmark_, pivdiag_,
+                               xchg_, st_, s_)));
     RID_TRY(tend(1));
     RID_TRY(tbegin(ID_PHASE_UPDATE));
     int nl = 3;
@@ -924,9 +920,9 @@ class Engine {
   int64_t lda_;
   DevState* st_;
   DevState h_{};
-  T *omega_, *G_, *Gpart_, *S_, *Spart_, *N_, *Linv_, *cand_rows_, *X_;
-  int32_t *act_[2], *pivmark_, *perm32_, *piv_, *pivorig_, *cand_i_;
-  double *pivdiag_, *cand_v_, *e2_, *normp_, *trace_;
+  T *omega_, *G_, *Gpart_, *S_, *Spart_, *N_, *Linv_, *X_;
+  int32_t *act_[2], *pivmark_, *perm32_, *piv_, *pivorig_;
+  double *pivdiag_, *e2_, *normp_, *trace_;
   void* digits_;       // path 65: digit slices of A
   int32_t* colexp_;    // path 65: column exponents of A
   T* L_;               // x_solve_f64: LUPP multipliers by original row (null otherwise)
@@ -952,7 +948,8 @@ class Engine {
   int32_t x_f64_ = 0;
   int64_t predicted_ = 0;
   int32_t passes_ = 0;
-  int panel_par_ = 0;  // barrier counter of the next panel launch (alternates)
+  void* xchg_;              // candidate words of the panel
+  unsigned panel_seq_ = 0;  // panel launches of this call
   int64_t launches_ = 0;
   double phase_ms_[kNumPhases];
   int64_t phase_launches_[kNumPhases];
@@ -1219,7 +1216,7 @@ cudaError_t run_sketch(const id_matrix* A, const void* omega, int64_t ld_omega, 
                        void* G, int64_t ldg, void* ws, cudaStream_t s) {
   DevState* st = static_cast<DevState*>(ws);
   void* part = static_cast<unsigned char*>(ws) + 256;
-  cudaError_t e0 = init_state(st, nullptr, nullptr, 0, s);
+  cudaError_t e0 = init_state(st, nullptr, nullptr, 0, nullptr, 0, s);
   if (e0 != cudaSuccess) return e0;
   cudaError_t e = cudaSuccess;
   // split-K partials: row stride rows (what the workspace holds), reduced into G (row stride ldg)
@@ -1501,7 +1498,7 @@ int id_certificate(const id_matrix* A, const int64_t* J, const void* X, int64_t 
   unsigned char* w = static_cast<unsigned char*>(ws);
   DevState* st = reinterpret_cast<DevState*>(w + c.off_st);
   const int64_t m = A->m, n = A->n;
-  cudaError_t e = init_state(st, nullptr, nullptr, 0, s);
+  cudaError_t e = init_state(st, nullptr, nullptr, 0, nullptr, 0, s);
   const void* Om = omega;
   int64_t ldo = ld_omega;
   if (e == cudaSuccess && omega == nullptr) {  // Omega' rows [row0, row0 + q) of the generator `seed`

@@ -28,8 +28,6 @@ struct DevState {
   uint32_t err;           // kErr* bits
   uint32_t zero_pivots;   // exactly zero pivot columns met
   uint32_t bar[2];        // grid-barrier arrival counters, one per launch parity
-  uint32_t pad[5];
-  unsigned long long pkey[2][3][2];  // LUPP panel: pivot-key maxima, [launch parity][step mod 3][key]
 };
 static_assert(sizeof(DevState) <= 256, "DevState must fit its 256-byte slot");
 
@@ -56,8 +54,21 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 // Upper bound on any single device-side wait (nanoseconds).
 constexpr uint64_t kWaitLimitNs = 4000000000ull;
 
-__device__ __forceinline__ void red_max_u64(unsigned long long* p, unsigned long long v) {
-  asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+// Relaxed 64-bit words: a word is read or written as a whole (of a pair, each word by itself).
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void ld_relaxed_v2(const unsigned long long* p, unsigned long long& a,
+                                              unsigned long long& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed_v2(unsigned long long* p, unsigned long long a, unsigned long long b) {
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
 }
 __device__ __forceinline__ void red_release_add_u32(unsigned* p, unsigned v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");

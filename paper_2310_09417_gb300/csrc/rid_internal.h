@@ -120,10 +120,12 @@ PanelCfg panel_config(int na, int w, int num_sms);
 // Rows per block and shared memory of the panel kernel for a given block count.
 template <typename T>
 PanelCfg panel_layout(int na, int w, int grid);
+// `xchg`: panel_xchg_bytes() of words through which the blocks exchange candidates,
+// cleared before the first launch of a call; `seq` numbers the call's launches.
+size_t panel_xchg_bytes(int maxg, int64_t wmax, size_t esz);
 template <typename T>
-cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, int par, T* S, int64_t lds,
-                       int32_t* piv, int32_t* pivmark, double* pivdiag, double* cand_v,
-                       int32_t* cand_i, T* cand_rows, DevState* st, cudaStream_t s);
+cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, unsigned seq, T* S, int64_t lds,
+                       int32_t* piv, int32_t* pivmark, double* pivdiag, void* xchg, DevState* st, cudaStream_t s);
 
 // Inverse of the unit-lower block L-hat(piv, 0:bt) (bt x bt, row-major).
 template <typename T>
@@ -145,7 +147,9 @@ cudaError_t compact(int na, int bt, const int32_t* act_in, int32_t* act_out, int
 template <typename T>
 cudaError_t finalize_x(int64_t k, const int32_t* perm32, T* X, int64_t ldx, cudaStream_t s);
 
-cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, cudaStream_t s);
+// Clears the state, lists every column as active and zeroes `clear` (16-byte words).
+cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, void* clear, size_t clear_bytes,
+                       cudaStream_t s);
 
 // G (m x k row-major) = A(:, J); W (m x k column-major) = X^T.
 template <typename T>

@@ -637,259 +637,359 @@ cudaError_t decide(const double* e2part, int nparts, int w, double tol, int tol_
 // ============================================================ LUPP panel
 // One cooperative launch factors S (na x w) for `steps` pivots.  Block b owns
 // rows [b*chunk, min(na, (b+1)*chunk)), staged in shared memory (row stride
-// w + 1: column reads hit distinct banks) when they fit.  Each pivot step:
-// block-local argmax of |S(i,c)| over unselected rows (ties to the smallest row
-// index = smallest column index of A, since `act` is ascending), publication of
-// the block's candidate, one bounded grid barrier, the global pivot and its
-// row, then division by the pivot and the rank-1 update (Eq. lupps) of the
-// block's unselected rows.  Rows are marked, never swapped.  Look-ahead: column
-// c+1 of the update, the candidate for pivot c+1 and the arrival at the next
-// barrier come first; the remaining columns are updated while the barrier fills.
-// Every entry receives the same single FMA per pivot as without look-ahead.
+// w + 1: column reads hit distinct banks) when they fit.  Rows are marked, never
+// swapped.  Each pivot step: the global argmax of |S(i,c)| over unselected rows
+// (ties to the smallest row index = smallest column index of A, since `act` is
+// ascending), division by the pivot and the rank-1 update (Eq. lupps).  Every
+// entry receives one division and one FMA per pivot, whatever the schedule.
 //
-// The global pivot comes from two 64-bit atomic maxima that every block adds
-// before the barrier: (top, ~row) and (top, row), top = the leading 32 bits of
-// |S(i,c)|'s pattern.  The first names the smallest row among the candidates of
-// largest top; when the second names the same row no other candidate shares
-// that top, and the row is the exact argmax.  Otherwise (FP64 candidates equal
-// in their leading 32 bits) every block compares the published full patterns.
-// For FP32 the top is the whole pattern and the first key is exact.  A step thus
-// costs the barrier and two L2 round trips on one or two lines, whatever the
-// number of blocks.  Key slots rotate over three steps (block 0 clears the next
-// one before it arrives at a barrier: every block has read the slot two steps
-// back) and alternate between launches like the barrier counter (block 0 clears
-// the other launch's slots).
+// What bounds it: the chain from one pivot to the next (the blocks learn the
+// winner, fetch its row, divide, update one column, find their next candidate),
+// 64 times per launch; the update itself is 0.2 - 0.6 us per pivot.  So the
+// exchange is built for the fewest trips to L2 and no fence:
+//  - a block publishes its candidate's magnitude and row as 64-bit words that
+//    carry 32 bits of data and a 32-bit tag (launch and step).  A word is stored
+//    and loaded as a whole, so a reader that finds the tag has the data; no release,
+//    no barrier counter, no atomics.  Tags never repeat within a call and the words
+//    are cleared when it starts.
+//  - warp 0 alone polls every block's magnitude words (a lane reads up to five
+//    blocks at once), picks the winner by integer maxima, and reads its row: one
+//    trip for the candidates, one for the row, which was stored at the same time
+//    and is normally there.  The larger magnitude wins; block b's rows come before
+//    block b+1's, so ties go to the smaller block.
+//  - the other warps run the rank-1 update of the previous pivot meanwhile.  Column
+//    c+1 and the candidate's row are updated before (look-ahead), so the bulk of the
+//    update is never waited for unless it is longer than the exchange.
+// A step has two block barriers.  Two word buffers alternate between steps: a block
+// stores step c+2's words only after it has seen every block's word of step c+1,
+// and each block stored that after it had read step c's.
+// Measured on GB300 per pivot (w = 64): FP64 3.1 us (n = 10000; 4.2 with a
+// counter barrier and atomic keys), FP32 2.0 us (n = 3000; 2.9) and 2.3 us (n = 20000; 3.6).
 constexpr int kPanelThreads = 256;
 constexpr int kPanelMaxW = 128;
+constexpr int kPanelPoll = 5;  // candidates a lane of the polling warp reads at once
 
-// Pivot search key: |S(i,c)| by its IEEE bit pattern (sign cleared; the order of
-// the patterns is the order of the values), then the smaller row index: the
-// largest key wins.  lo = ~row (never 0 for a row), so {0, 0} is "no candidate".
-// Integer comparisons only (GB300 issues about two FP64 instructions per clock
-// per SM).
-struct PivKey {
-  unsigned long long hi;
-  unsigned lo;
-};
-__device__ __forceinline__ PivKey key_pick(PivKey a, PivKey b) {
-  return (b.hi > a.hi || (b.hi == a.hi && b.lo > a.lo)) ? b : a;
-}
-__device__ __forceinline__ PivKey warp_key_max(PivKey a) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    PivKey o;
-    o.hi = __shfl_xor_sync(0xffffffffu, a.hi, off);
-    o.lo = __shfl_xor_sync(0xffffffffu, a.lo, off);
-    a = key_pick(a, o);
-  }
-  return a;
-}
-// Block-wide key maximum (every thread gets it); blockDim.x a multiple of 32.
-__device__ __forceinline__ PivKey block_key_max(PivKey a) {
-  __shared__ unsigned long long s_hi[32];
-  __shared__ unsigned s_lo[32];
-  a = warp_key_max(a);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_hi[wid] = a.hi;
-    s_lo[wid] = a.lo;
-  }
-  __syncthreads();
-  const int nw = blockDim.x >> 5;
-  PivKey b;
-  b.hi = lane < nw ? s_hi[lane] : 0ull;
-  b.lo = lane < nw ? s_lo[lane] : 0u;
-  b = warp_key_max(b);  // every warp reduces the same values
-  __syncthreads();      // s_hi / s_lo are reused by the next call
-  return b;
-}
 __device__ __forceinline__ unsigned long long mag_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
 }
 __device__ __forceinline__ unsigned long long mag_bits(float x) {
-  return (unsigned long long)((unsigned)__float_as_int(x) & 0x7FFFFFFFu);
+  return (unsigned long long)((unsigned)__float_as_int(x) & 0x7FFFFFFFu) << 32;
 }
-__device__ __forceinline__ unsigned mag_top(unsigned long long hi, double) { return (unsigned)(hi >> 31); }
-__device__ __forceinline__ unsigned mag_top(unsigned long long hi, float) { return (unsigned)hi; }
 
-// Grid barrier in two halves: every block adds its arrival (after its publications,
-// ordered by the block barrier and the release), works on, then waits for the k-th
-// barrier's (k+1) nblocks arrivals.  The wait is bounded as in grid_barrier.
-__device__ __forceinline__ void grid_arrive(unsigned* ctr) {
-  __syncthreads();
-  if (threadIdx.x == 0) red_release_add_u32(ctr, 1u);
-}
-__device__ __forceinline__ bool grid_wait(unsigned* ctr, unsigned target, DevState* st) {
-  __shared__ int s_ok;
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    if ((int)(ld_acquire_u32(ctr) - target) < 0) {
-      const uint64_t t0 = globaltimer_ns();
-      unsigned spins = 0;
-      while ((int)(ld_acquire_u32(ctr) - target) < 0) {
-        if ((++spins & 255u) == 0u) {
-          if (ld_acquire_u32(&st->err) & kErrTimeout) { ok = 0; break; }
-          if (globaltimer_ns() - t0 > kWaitLimitNs) {
-            atomicOr(&st->err, kErrTimeout);
-            ok = 0;
-            break;
-          }
-        }
-      }
-    }
-    s_ok = ok;
+// Largest magnitude of a warp, by its IEEE bit pattern (the order of the patterns
+// is the order of the values; integer comparisons only: GB300 issues about two FP64
+// instructions per clock per SM).  Lanes with `have` false take no part.  Returns
+// the lowest lane that holds the maximum, -1 when no lane takes part.
+template <typename T>
+__device__ __forceinline__ int warp_mag_argmax(bool have, unsigned long long mag, unsigned long long& best) {
+  const unsigned hi = (unsigned)(mag >> 32);
+  const unsigned top = __reduce_max_sync(0xffffffffu, have ? hi + 1u : 0u);  // hi <= 0x7FFFFFFF
+  if (top == 0u) return -1;
+  bool in = have && hi + 1u == top;
+  best = (unsigned long long)(top - 1u) << 32;
+  if (sizeof(T) == 8) {
+    const unsigned lo = __reduce_max_sync(0xffffffffu, in ? (unsigned)mag : 0u);
+    in = in && (unsigned)mag == lo;
+    best |= (unsigned long long)lo;
   }
-  __syncthreads();
-  return s_ok != 0;
+  return __ffs(__ballot_sync(0xffffffffu, in)) - 1;
+}
+
+// 64-bit words of one block's publication: the magnitude (kMagWords), then the row
+// index, then the row's entries (kValWords each).  A block without a candidate
+// stores kNoCand.
+template <typename T>
+struct PanelWords {
+  static constexpr int kMag = 2;                  // magnitude words (16-byte stride; FP32 uses the first)
+  static constexpr int kVal = (int)sizeof(T) / 4;  // words per entry
+  __host__ __device__ static constexpr int row_words(int w) { return 2 + kVal * ((w + 1) & ~1); }
+  __host__ __device__ static constexpr int slot_words(int w) { return kMag + row_words(w); }
+};
+constexpr unsigned kNoCand = 0xFFFFFFFFu;
+
+size_t panel_xchg_bytes(int maxg, int64_t wmax, size_t esz) {
+  const int w = wmax > kPanelMaxW ? kPanelMaxW : (int)wmax;
+  const int words = esz == 8 ? PanelWords<double>::slot_words(w) : PanelWords<float>::slot_words(w);
+  return (size_t)2 * maxg * words * sizeof(unsigned long long);
+}
+
+__device__ __forceinline__ unsigned long long tagged(unsigned data, unsigned tag) {
+  return ((unsigned long long)tag << 32) | data;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kPanelThreads)
-    k_panel_lupp(int na, int w, int steps, T* __restrict__ S, int64_t lds, int chunk, int use_smem, int par,
-                 int32_t* piv, int32_t* pivmark, double* pivdiag, double* cand_v, int32_t* cand_i,
-                 T* cand_rows, DevState* st) {
+    k_panel_lupp(int na, int w, int steps, T* __restrict__ S, int64_t lds, int chunk, int use_smem, unsigned tag0,
+                 int32_t* piv, int32_t* pivmark, double* pivdiag, unsigned long long* xchg, DevState* st) {
+  using PW = PanelWords<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ T prow[kPanelMaxW];
-  __shared__ int s_piv;
+  __shared__ T prow[2][kPanelMaxW];
+  __shared__ int s_piv[2];
+  __shared__ unsigned long long s_mag[kPanelThreads / 32];
+  __shared__ int s_row[kPanelThreads / 32];
   const int nb = gridDim.x, bid = blockIdx.x, tid = threadIdx.x;
-  if (bid == 0 && tid < 6) (&st->pkey[par ^ 1][0][0])[tid] = 0ull;  // the previous launch has ended
-  if (bid == 0 && tid == 0) st->bar[par ^ 1] = 0u;
   if (st->done) return;  // set before the launch or never during it: uniform over the grid
-  unsigned* ctr = &st->bar[par];
-  unsigned long long* cand_k = reinterpret_cast<unsigned long long*>(cand_v);
-  const int lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int lane = tid & 31, wid = tid >> 5;
+  constexpr int nw = kPanelThreads / 32;
   const int r0 = bid * chunk;
   const int nr = max(0, min(na, r0 + chunk) - r0);
   T* Ss = use_smem ? reinterpret_cast<T*>(smem_raw) : S + (int64_t)r0 * lds;
   const int64_t ldl = use_smem ? w + 1 : lds;
   unsigned char* sel = smem_raw + (use_smem ? (size_t)chunk * (w + 1) * sizeof(T) : 0);
+  // magnitude words of both buffers, then the row words of both
+  const int rwords = PW::row_words(w);
+  unsigned long long* const rows = xchg + (size_t)2 * nb * PW::kMag;
 
   if (use_smem)
-    for (int e = tid; e < nr * w; e += blockDim.x) {
+    for (int e = tid; e < nr * w; e += kPanelThreads) {
       const int r = e / w, c = e - r * w;
       Ss[(int64_t)r * ldl + c] = S[(int64_t)(r0 + r) * lds + c];
     }
-  for (int r = tid; r < chunk; r += blockDim.x) sel[r] = 0;
+  for (int r = tid; r < chunk; r += kPanelThreads) sel[r] = 0;
   __syncthreads();
 
-  // Publish this block's candidate for pivot c (its row complete in every column)
-  // and add the arrival at barrier c.
-  auto publish = [&](int c, PivKey loc) {
-    const int lidx = loc.lo == 0u ? -1 : (int)~loc.lo;
-    const int base = (c & 1) * nb;
-    unsigned long long* key = &st->pkey[par][c % 3][0];
-    if (tid == 0) {
-      if (bid == 0) {
-        unsigned long long* next = &st->pkey[par][(c + 1) % 3][0];
-        next[0] = 0ull;
-        next[1] = 0ull;
-      }
-      if (lidx >= 0) {
-        const unsigned long long top = mag_top(loc.hi, T(0));
-        red_max_u64(&key[0], (top << 32) | (unsigned long long)loc.lo);
-        red_max_u64(&key[1], (top << 32) | (unsigned long long)(unsigned)lidx);
-      }
-      __stcg(&cand_k[base + bid], loc.hi);
-      __stcg(&cand_i[base + bid], lidx);
+  // This block's candidate for pivot c from the warps' maxima (every warp finds the
+  // same one): its local row, or -1.
+  auto block_cand = [&](unsigned long long& mag) {
+    const int r = lane < nw ? s_row[lane] : -1;
+    const unsigned long long v = lane < nw ? s_mag[lane] : 0ull;
+    // a warp's rows are not contiguous: equal magnitudes go to the smallest row
+    if (warp_mag_argmax<T>(r >= 0, v, mag) < 0) return -1;
+    return (int)__reduce_min_sync(0xffffffffu, r >= 0 && v == mag ? (unsigned)r : 0x7FFFFFFFu);
+  };
+  // Column c's maximum over this warp's rows into s_mag / s_row.
+  auto warp_cand = [&](bool have, unsigned long long mag, int r) {
+    unsigned long long best = 0ull;
+    const int src = warp_mag_argmax<T>(have, mag, best);
+    // (a lane may hold a later row than its neighbours: equal magnitudes go to the smallest)
+    const unsigned br = __reduce_min_sync(0xffffffffu, have && mag == best ? (unsigned)r : 0x7FFFFFFFu);
+    if (lane == 0) {
+      s_mag[wid] = best;
+      s_row[wid] = src < 0 ? -1 : (int)br;
     }
-    if (lidx >= 0) {
-      const T* src = Ss + (int64_t)(lidx - r0) * ldl;
-      for (int cc = tid; cc < w; cc += blockDim.x) __stcg(&cand_rows[(int64_t)(base + bid) * w + cc], src[cc]);
+  };
+  // Warp 0: store the candidate's magnitude and row; the entries from column c on are
+  // updated for pivot c-1 on the way when `l` says so.
+  auto publish = [&](int c, int cand, unsigned long long mag, const T* p, T l, bool upd) {
+    const unsigned tag = tag0 + (unsigned)c;
+    unsigned long long* mw = xchg + ((size_t)(c & 1) * nb + bid) * PW::kMag;
+    unsigned long long* rw = rows + ((size_t)(c & 1) * nb + bid) * rwords;
+    if (lane == 0) {
+      const unsigned hi = cand < 0 ? kNoCand : (unsigned)(mag >> 32);
+      if (sizeof(T) == 8)
+        st_relaxed_v2(mw, tagged(hi, tag), tagged((unsigned)mag, tag));
+      else
+        st_relaxed(mw, tagged(hi, tag));
     }
-    grid_arrive(ctr);
+    if (cand < 0) return;
+    if (lane == 0) st_relaxed(rw, tagged((unsigned)(r0 + cand), tag));
+    T* row = Ss + (int64_t)cand * ldl;
+    for (int cc = c + lane; cc < w; cc += 32) {
+      T v = row[cc];
+      if (upd && cc > c) {  // column c itself was updated with the whole column
+        v = fma(-l, p[cc], v);
+        row[cc] = v;
+      }
+      if constexpr (sizeof(T) == 8) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+        st_relaxed_v2(rw + 2 + 2 * cc, tagged((unsigned)(b >> 32), tag), tagged((unsigned)b, tag));
+      } else {
+        st_relaxed(rw + 2 + cc, tagged(__float_as_uint(v), tag));
+      }
+    }
+  };
+  // Warp 0: wait until every block's magnitude for pivot c is there, pick the winner
+  // and bring its row into prow[c & 1], its index into s_piv[c & 1] (-1: no
+  // candidate anywhere, -2: the wait ran out).
+  auto collect = [&](int c) {
+    const unsigned tag = tag0 + (unsigned)c;
+    const unsigned long long* mw = xchg + (size_t)(c & 1) * nb * PW::kMag;
+    bool have = false;
+    unsigned long long bmag = 0ull;
+    int bq = 0;
+    unsigned spins = 0;
+    uint64_t t0 = 0;
+    auto gave_up = [&]() {  // uniform over the warp
+      if ((++spins & 255u) != 0u) return false;
+      int bad = 0;
+      if (lane == 0) {
+        const uint64_t now = globaltimer_ns();
+        if (t0 == 0) t0 = now;
+        if (ld_acquire_u32(&st->err) & kErrTimeout) {
+          bad = 1;
+        } else if (now - t0 > kWaitLimitNs) {
+          atomicOr(&st->err, kErrTimeout);
+          bad = 1;
+        }
+      }
+      return __shfl_sync(0xffffffffu, bad, 0) != 0;
+    };
+    for (int q0 = 0; q0 < nb; q0 += 32 * kPanelPoll) {
+      unsigned long long v[kPanelPoll], u[kPanelPoll];
+      for (;;) {
+        bool all = true;
+#pragma unroll
+        for (int i = 0; i < kPanelPoll; ++i) {
+          const int q = q0 + lane + 32 * i;
+          v[i] = u[i] = tagged(kNoCand, tag);
+          if (q < nb) {
+            if (sizeof(T) == 8)
+              ld_relaxed_v2(mw + (size_t)q * PW::kMag, v[i], u[i]);
+            else
+              v[i] = ld_relaxed(mw + (size_t)q * PW::kMag);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < kPanelPoll; ++i)
+          all = all && (unsigned)(v[i] >> 32) == tag && (sizeof(T) == 4 || (unsigned)(u[i] >> 32) == tag);
+        if (__all_sync(0xffffffffu, all)) break;
+        if (gave_up()) {
+          if (lane == 0) s_piv[c & 1] = -2;
+          return;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < kPanelPoll; ++i) {
+        const unsigned hi = (unsigned)v[i];
+        const unsigned long long mag = ((unsigned long long)hi << 32) | (sizeof(T) == 8 ? (unsigned)u[i] : 0u);
+        if (hi != kNoCand && (!have || mag > bmag)) {  // ascending blocks: ties keep the smaller
+          have = true;
+          bmag = mag;
+          bq = q0 + lane + 32 * i;
+        }
+      }
+    }
+    unsigned long long best = 0ull;
+    if (warp_mag_argmax<T>(have, bmag, best) < 0) {
+      if (lane == 0) s_piv[c & 1] = -1;
+      return;
+    }
+    const int q = (int)__reduce_min_sync(0xffffffffu, have && bmag == best ? (unsigned)bq : 0x7FFFFFFFu);
+    const unsigned long long* rw = rows + ((size_t)(c & 1) * nb + q) * rwords;
+    for (;;) {
+      const unsigned long long g = ld_relaxed(rw);
+      bool all = (unsigned)(g >> 32) == tag;
+#pragma unroll
+      for (int j = 0; j < kPanelMaxW / 32; ++j) {
+        const int cc = c + lane + 32 * j;
+        if (cc < w) {
+          if constexpr (sizeof(T) == 8) {
+            unsigned long long h, l;
+            ld_relaxed_v2(rw + 2 + 2 * cc, h, l);
+            all = all && (unsigned)(h >> 32) == tag && (unsigned)(l >> 32) == tag;
+            prow[c & 1][cc] = __longlong_as_double((long long)((h << 32) | (l & 0xFFFFFFFFull)));
+          } else {
+            const unsigned long long h = ld_relaxed(rw + 2 + cc);
+            all = all && (unsigned)(h >> 32) == tag;
+            prow[c & 1][cc] = __uint_as_float((unsigned)h);
+          }
+        }
+      }
+      if (__all_sync(0xffffffffu, all)) {
+        if (lane == 0) s_piv[c & 1] = (int)(unsigned)g;
+        return;
+      }
+      if (gave_up()) {
+        if (lane == 0) s_piv[c & 1] = -2;
+        return;
+      }
+    }
   };
 
   // pivot 0's candidate
-  if (steps > 0) {
-    PivKey loc{0ull, 0u};
-    for (int r = tid; r < nr; r += blockDim.x)
-      loc = key_pick(loc, PivKey{mag_bits(Ss[(int64_t)r * ldl]), ~(unsigned)(r0 + r)});
-    publish(0, block_key_max(loc));
+  {
+    bool have = false;
+    unsigned long long mag = 0ull;
+    int row = 0;
+    for (int r = tid; r < nr; r += kPanelThreads) {
+      const unsigned long long v = mag_bits(Ss[(int64_t)r * ldl]);
+      if (!have || v > mag) {
+        have = true;
+        mag = v;
+        row = r;
+      }
+    }
+    if (steps > 0) warp_cand(have, mag, row);
+    __syncthreads();
+    if (steps > 0 && wid == 0) {
+      const int cand = block_cand(mag);
+      publish(0, cand, mag, nullptr, T(0), false);
+    }
   }
 
   for (int c = 0; c < steps; ++c) {
-    // 1. every block's candidate for pivot c is published
-    if (!grid_wait(ctr, (unsigned)(c + 1) * (unsigned)nb, st)) return;
-    const int base = (c & 1) * nb;
-    const unsigned long long* key = &st->pkey[par][c % 3][0];
-    // 2. global pivot (warp 0 of every block, identically) and its row
-    if (wid == 0) {
-      const unsigned long long k0 = __ldcg(&key[0]), k1 = __ldcg(&key[1]);
-      int gi = k0 == 0ull ? -1 : (int)~(unsigned)k0;
-      if (gi >= 0 && sizeof(T) == 8 && (int)(unsigned)k1 != gi) {
-        // candidates tie in their leading 32 bits: compare the full patterns
-        PivKey g{0ull, 0u};
-        for (int q = lane; q < nb; q += 32) {
-          const int i = __ldcg(&cand_i[base + q]);
-          const unsigned long long h = __ldcg(&cand_k[base + q]);
-          if (i >= 0) g = key_pick(g, PivKey{h, ~(unsigned)i});
-        }
-        g = warp_key_max(g);
-        gi = (int)~g.lo;
-      }
-      if (gi >= 0) {
-        const int pblk = gi / chunk;  // the block that published row gi
-        for (int cc = lane; cc < w; cc += 32) prow[cc] = __ldcg(&cand_rows[(int64_t)(base + pblk) * w + cc]);
-      }
-      __syncwarp();
-      if (lane == 0) {
-        s_piv = gi;
-        const T pv = gi >= 0 ? prow[c] : T(0);
-        if (gi >= r0 && gi < r0 + nr) sel[gi - r0] = (unsigned char)1;
-        if (bid == 0) {
-          piv[c] = gi;
-          if (pivdiag != nullptr) pivdiag[c] = (double)tabs(pv);
-          if (pv == T(0)) atomicAdd(&st->zero_pivots, 1u);
-        }
-      }
-    }
+    // 1. warp 0: the global pivot and its row; the other warps arrive here when the
+    //    rank-1 update of pivot c-1 is done
+    if (wid == 0) collect(c);
     __syncthreads();
-    const T pv = s_piv >= 0 ? prow[c] : T(0);
+    const int gi = s_piv[c & 1];
+    if (gi == -2) return;
+    const T* pr = prow[c & 1];
+    const T pv = gi >= 0 ? pr[c] : T(0);
     const bool elim = pv != T(0);  // a zero column below: nothing to eliminate
-    // 3. multipliers l(i) = S(i,c) / pivot
-    if (elim)
-      for (int r = tid; r < nr; r += blockDim.x)
-        if (!sel[r]) Ss[(int64_t)r * ldl + c] = Ss[(int64_t)r * ldl + c] / pv;
-    __syncthreads();
-    // 4. look-ahead: column c+1 of the rank-1 update (Eq. lupps), the candidate for
-    //    pivot c+1 and its row's remaining columns, then the arrival at barrier c+1
-    int cand = -1;  // local row of the published candidate (updated already)
-    if (c + 1 < steps) {
-      const T p1 = prow[c + 1];
-      PivKey loc{0ull, 0u};
-      for (int r = tid; r < nr; r += blockDim.x)
-        if (!sel[r]) {
+    const bool more = c + 1 < steps;
+    // 2. multipliers l(i) = S(i,c) / pivot, column c+1 of the update and its maximum
+    {
+      const T p1 = more ? pr[c + 1] : T(0);
+      bool have = false;
+      unsigned long long mag = 0ull;
+      int brow = 0;
+      for (int r = tid; r < nr; r += kPanelThreads) {
+        if (r0 + r == gi) {
+          sel[r] = (unsigned char)1;
+        } else if (!sel[r]) {
           T* row = Ss + (int64_t)r * ldl;
-          if (elim) row[c + 1] = fma(-row[c], p1, row[c + 1]);
-          loc = key_pick(loc, PivKey{mag_bits(row[c + 1]), ~(unsigned)(r0 + r)});
+          T v = more ? row[c + 1] : T(0);
+          if (elim) {
+            const T l = row[c] / pv;
+            row[c] = l;
+            if (more) row[c + 1] = v = fma(-l, p1, v);
+          }
+          const unsigned long long m = mag_bits(v);
+          if (!have || m > mag) {
+            have = true;
+            mag = m;
+            brow = r;
+          }
         }
-      loc = block_key_max(loc);
-      cand = loc.lo == 0u ? -1 : (int)~loc.lo - r0;
-      if (elim && cand >= 0 && wid == 0) {
-        T* row = Ss + (int64_t)cand * ldl;
-        const T l = row[c];
-        for (int cc = c + 2 + lane; cc < w; cc += 32) row[cc] = fma(-l, prow[cc], row[cc]);
       }
-      __syncthreads();      // the candidate row is complete before it is published
-      publish(c + 1, loc);
+      if (more) warp_cand(have, mag, brow);
     }
-    // 5. the rest of the rank-1 update while the barrier fills: a warp per row,
-    //    lanes along the row, four rows at a time with their loads ahead of the stores
-    const int cfirst = c + 1 < steps ? c + 2 : c + 1;
-    if (elim && cfirst < w) {
+    if (bid == 0 && tid == 0) {
+      piv[c] = gi;
+      if (pivdiag != nullptr) pivdiag[c] = (double)tabs(pv);
+      if (pv == T(0)) atomicAdd(&st->zero_pivots, 1u);
+    }
+    __syncthreads();
+    // 3. warp 0 completes the candidate's row and publishes it
+    int cand = -1;
+    if (more) {
+      unsigned long long mag = 0ull;
+      cand = block_cand(mag);
+      if (wid == 0) {
+        const T l = cand >= 0 ? Ss[(int64_t)cand * ldl + c] : T(0);
+        publish(c + 1, cand, mag, pr, l, elim);
+      }
+    }
+    // 4. the rest of the rank-1 update: a warp per row, lanes along the row, four rows
+    //    at a time with their loads ahead of the stores (warp 0 is exchanging, except
+    //    after the last pivot, where it works too)
+    const int cfirst = more ? c + 2 : c + 1;
+    if (elim && cfirst < w && (wid > 0 || !more)) {
+      const int nwork = more ? nw - 1 : nw;
       T p[kPanelMaxW / 32];
 #pragma unroll
       for (int j = 0; j < kPanelMaxW / 32; ++j) {
         const int cc = cfirst + lane + 32 * j;
-        p[j] = cc < w ? prow[cc] : T(0);
+        p[j] = cc < w ? pr[cc] : T(0);
       }
-      for (int r = wid; r < nr; r += 4 * nw) {
+      for (int r = more ? wid - 1 : wid; r < nr; r += 4 * nwork) {
         T* rp[4];
         T l[4];
         bool live[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int rr = r + u * nw;
+          const int rr = r + u * nwork;
           live[u] = rr < nr && !sel[rr] && rr != cand;
           rp[u] = Ss + (int64_t)(live[u] ? rr : 0) * ldl;
           l[u] = live[u] ? rp[u][c] : T(0);
@@ -908,21 +1008,20 @@ __global__ void __launch_bounds__(kPanelThreads)
         }
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
   if (use_smem)
-    for (int e = tid; e < nr * w; e += blockDim.x) {
+    for (int e = tid; e < nr * w; e += kPanelThreads) {
       const int r = e / w, c = e - r * w;
       S[(int64_t)(r0 + r) * lds + c] = Ss[(int64_t)r * ldl + c];
     }
-  for (int r = tid; r < nr; r += blockDim.x) pivmark[r0 + r] = sel[r];
+  for (int r = tid; r < nr; r += kPanelThreads) pivmark[r0 + r] = sel[r];
 }
 
 // Blocks of the panel: one per SM, at least 32 rows each, and enough for the
-// rows of a block to fit in shared memory.  With the key exchange a step's
-// barrier and round trips cost about the same for any number of blocks (measured
-// on GB300: 3.2 - 5.3 us per pivot for 4000 - 20000 rows, FP32 and FP64 alike,
-// fastest with the most blocks), so the rows are spread as thin as possible.
+// rows of a block to fit in shared memory.  A step's exchange costs about the same
+// for any number of blocks, while the update of a block's rows shrinks with them,
+// so the rows are spread as thin as possible.
 // RANDID_PANEL_BLOCKS fixes the count (tuning).
 static int panel_blocks_env() {
   static int blocks = -1;
@@ -976,11 +1075,10 @@ PanelCfg panel_layout(int na, int w, int grid) {
 }
 
 template <typename T>
-cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, int par, T* S, int64_t lds, int32_t* piv,
-                       int32_t* pivmark, double* pivdiag, double* cand_v, int32_t* cand_i, T* cand_rows,
-                       DevState* st, cudaStream_t s) {
+cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, unsigned seq, T* S, int64_t lds, int32_t* piv,
+                       int32_t* pivmark, double* pivdiag, void* xchg, DevState* st, cudaStream_t s) {
   static SmemLimit lim;
-  if (w > kPanelMaxW || (par != 0 && par != 1)) return cudaErrorInvalidValue;
+  if (w > kPanelMaxW || steps > w) return cudaErrorInvalidValue;
   // the kernel addresses chunk rows at stride w + 1 and the selection bytes after them
   if (cfg.chunk < 1 || (int64_t)cfg.chunk * cfg.grid < na ||
       cfg.smem < panel_smem_bytes(cfg.chunk, w, sizeof(T), cfg.use_smem != 0))
@@ -988,8 +1086,10 @@ cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, int par, T
   cudaError_t e = raise_smem(k_panel_lupp<T>, cfg.smem, lim);
   if (e != cudaSuccess) return e;
   int chunk = cfg.chunk, use_smem = cfg.use_smem;
-  void* args[] = {&na, &w, &steps, &S, &lds, &chunk, &use_smem, &par, &piv, &pivmark,
-                  &pivdiag, &cand_v, &cand_i, &cand_rows, &st};
+  // tags of this launch's steps: never 0 (the cleared words) and new to the call
+  unsigned tag0 = seq * (unsigned)kPanelMaxW + 1u;
+  unsigned long long* words = static_cast<unsigned long long*>(xchg);
+  void* args[] = {&na, &w, &steps, &S, &lds, &chunk, &use_smem, &tag0, &piv, &pivmark, &pivdiag, &words, &st};
   return cudaLaunchCooperativeKernel((const void*)k_panel_lupp<T>, dim3(cfg.grid), dim3(kPanelThreads), args,
                                      cfg.smem, s);
 }
@@ -1256,7 +1356,7 @@ cudaError_t transpose_w(const T* X, int64_t ldx, int64_t m, int64_t k, T* W, int
   return cudaGetLastError();
 }
 
-__global__ void k_init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n) {
+__global__ void k_init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, uint4* clear, int64_t nclear) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i == 0) {
     st->norm2_A = 0.0;
@@ -1271,17 +1371,20 @@ __global__ void k_init_state(DevState* st, int32_t* act, int32_t* pivmark, int64
     st->zero_pivots = 0u;
     st->bar[0] = 0u;
     st->bar[1] = 0u;
-    for (int q = 0; q < 12; ++q) (&st->pkey[0][0][0])[q] = 0ull;
   }
   if (i < n) {
     act[i] = (int32_t)i;
     pivmark[i] = 0;
   }
+  for (int64_t e = i; e < nclear; e += (int64_t)gridDim.x * blockDim.x) clear[e] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, cudaStream_t s) {
-  const int64_t blocks = (n + 255) / 256;
-  k_init_state<<<(int)(blocks < 1 ? 1 : blocks), 256, 0, s>>>(st, act, pivmark, n);
+cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, void* clear, size_t clear_bytes,
+                       cudaStream_t s) {
+  const int64_t nclear = (int64_t)(clear_bytes / 16);
+  int64_t blocks = ((n > nclear ? n : nclear) + 255) / 256;
+  if (blocks < 1) blocks = 1;
+  k_init_state<<<(int)blocks, 256, 0, s>>>(st, act, pivmark, n, static_cast<uint4*>(clear), nclear);
   return cudaGetLastError();
 }
 
@@ -1301,8 +1404,8 @@ cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, 
                                        const T*, T*, int64_t, double*, int, const int32_t*, cudaStream_t);  \
   template PanelCfg panel_config<T>(int, int, int);                                                         \
   template PanelCfg panel_layout<T>(int, int, int);                                                         \
-  template cudaError_t panel_lupp<T>(const PanelCfg&, int, int, int, int, T*, int64_t, int32_t*, int32_t*,       \
-                                     double*, double*, int32_t*, T*, DevState*, cudaStream_t);              \
+  template cudaError_t panel_lupp<T>(const PanelCfg&, int, int, int, unsigned, T*, int64_t, int32_t*, int32_t*,  \
+                                     double*, void*, DevState*, cudaStream_t);                              \
   template cudaError_t linv<T>(int, const T*, int64_t, const int32_t*, T*, const int32_t*, cudaStream_t);   \
   template cudaError_t make_n<T>(int, int, const T*, int64_t, const T*, const int32_t*, const int32_t*, T*, \
                                  T*, int64_t, int64_t, const int32_t*, int32_t*, const int32_t*,            \

@@ -545,7 +545,7 @@ cudaError_t stable_x_run(const T* A, int64_t lda, int64_t m, int64_t n, const in
   T* R = reinterpret_cast<T*>(ws + p.off_R);
   T* Ri = reinterpret_cast<T*>(ws + p.off_Ri);
   unsigned char* qws = ws + p.off_qr;
-  cudaError_t e = init_state(st, nullptr, nullptr, 0, s);
+  cudaError_t e = init_state(st, nullptr, nullptr, 0, nullptr, 0, s);
   if (e != cudaSuccess) return e;
   k_gather2<T><<<grid1(m * k), 256, 0, s>>>(m, k, A, lda, m, n, nullptr, J, 0, F, m, st);  // C = A(:, J)
   e = cudaGetLastError();
@@ -621,7 +621,7 @@ cudaError_t cur_run(const T* A, int64_t lda, int64_t m, int64_t n, const int64_t
   T* Z = reinterpret_cast<T*>(ws + p.off_Z);
   T* R = reinterpret_cast<T*>(ws + p.off_R);
   T* Ri = reinterpret_cast<T*>(ws + p.off_Ri);
-  cudaError_t e = init_state(st, nullptr, nullptr, 0, s);
+  cudaError_t e = init_state(st, nullptr, nullptr, 0, nullptr, 0, s);
   dim3 tg((unsigned)std::min<int64_t>(cdv(k, 32), 1024), (unsigned)std::min<int64_t>(cdv(k, 32), 1024));
   if (kind == 0) {
     // U = C^+ A R^+ = Rc^{-1} (Qc^T A Qr) Rr^{-T} with C = Qc Rc, R^T = Qr Rr
