@@ -546,6 +546,9 @@ class Engine {
     else if (p_.path == 16)
       RID_TRY(cuda(norm2_partial<__nv_bfloat16>(p_.m, p_.n, static_cast<const __nv_bfloat16*>(Araw_), lda_, normp_,
                                                 p_.nparts, st_, s_)));
+    else if (p_.path == 65 && !p_.sparse)  // the column exponents of the digit slices come with the norm
+      RID_TRY(cuda(norm2_f64(p_.m, p_.n, reinterpret_cast<const double*>(Araw_), lda_, normp_, p_.nparts, colexp_, st_,
+                             s_)));
     else
       RID_TRY(cuda(norm2_partial<T>(p_.m, p_.n, A_, lda_, normp_, p_.nparts, st_, s_)));
     RID_TRY(cuda(norm2_final(normp_, p_.nparts, st_, s_)));
@@ -564,10 +567,10 @@ class Engine {
                                         sfix_, s_)));
       RID_TRY(tend(2));
     }
-    if (p_.path == 65 && !p_.sparse) {  // column exponents and digit slices of A, once per call
+    if (p_.path == 65 && !p_.sparse) {  // digit slices of A, once per call
       RID_TRY(tbegin(ID_PHASE_SKETCH));
-      RID_TRY(cuda(f64emu_prepare(reinterpret_cast<const double*>(Araw_), lda_, p_.m, p_.n, colexp_, digits_, s_)));
-      RID_TRY(tend(2));
+      RID_TRY(cuda(f64emu_split(reinterpret_cast<const double*>(Araw_), lda_, p_.m, p_.n, colexp_, digits_, s_)));
+      RID_TRY(tend(1));
     }
     return 0;
   }

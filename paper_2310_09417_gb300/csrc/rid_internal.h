@@ -87,6 +87,9 @@ cudaError_t gaussian_rows(uint64_t seed, int64_t row0, int64_t rows, int64_t m, 
 template <typename T>
 cudaError_t norm2_partial(int64_t m, int64_t n, const T* A, int64_t lda, double* part, int nparts,
                           DevState* st, cudaStream_t s);
+// FP64, and with `colexp` also every column's exponent E_j (max_i |A_ij| < 2^E_j).
+cudaError_t norm2_f64(int64_t m, int64_t n, const double* A, int64_t lda, double* part, int nparts, int32_t* colexp,
+                      DevState* st, cudaStream_t s);
 cudaError_t norm2_final(const double* part, int nparts, DevState* st, cudaStream_t s);
 
 // G[j*ldg + c] = sum_z P[z*zs + j*ldg + c]
@@ -189,6 +192,9 @@ cudaError_t mlp_predict_rank(const float* params, const double* piv, int npiv, i
 int64_t f64emu_pad(int64_t m);
 size_t f64emu_digit_bytes(int64_t m, int64_t n);
 int f64emu_splits(int64_t m, int64_t n, int sms);
+cudaError_t f64emu_split(const double* A, int64_t lda, int64_t m, int64_t n, const int32_t* colexp, void* digits,
+                         cudaStream_t s);
+// the column exponents first, then the split
 cudaError_t f64emu_prepare(const double* A, int64_t lda, int64_t m, int64_t n, int32_t* colexp, void* digits,
                            cudaStream_t s);
 cudaError_t f64emu_omega(uint64_t seed, int64_t row0, int64_t rows, int64_t m, int64_t rows_alloc,

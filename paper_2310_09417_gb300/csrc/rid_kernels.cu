@@ -119,132 +119,6 @@ cudaError_t gaussian_rows(uint64_t seed, int64_t row0, int64_t rows, int64_t m, 
   return cudaGetLastError();
 }
 
-// ============================================================ ||A||_F and finiteness
-template <typename T>
-__global__ void k_norm2_partial(int64_t m, int64_t n, const T* __restrict__ A, int64_t lda,
-                                double* part, DevState* st) {
-  double acc = 0.0;
-  bool finite = true;
-  for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
-    const T* a = A + j * lda;
-    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
-      const double v = to_double(a[i]);
-      // finiteness from the exponent bits (integer pipe): one FP64 instruction per element
-      finite = finite && ((__double_as_longlong(v) >> 52) & 0x7FF) != 0x7FF;
-      acc += v * v;
-    }
-  }
-  if (!finite) atomicOr(&st->err, kErrNonFinite);
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-// BF16 columns 16-byte aligned (lda a multiple of 8): eight elements per load, the
-// squares summed exactly in FP32 and in float-float groups of 64 (sq_add_bits),
-// folded into FP64 -- no per-element FP64 work, which on GB300 (about two FP64
-// instructions per clock per SM) made this pass take ~20x its HBM time.
-__global__ void k_norm2_bf16(int64_t m, int64_t n, const __nv_bfloat16* __restrict__ A, int64_t lda, double* part,
-                             DevState* st) {
-  double acc = 0.0;
-  bool finite = true;
-  const int64_t nv = m / 8;
-  for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
-    const uint4* a = reinterpret_cast<const uint4*>(A + j * lda);
-    float hi = 0.f, lo = 0.f;
-    int grp = 0;
-    for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
-      const uint4 w = __ldg(a + v);
-      const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        sq_add_bits(ws[q] << 16, hi, lo, acc, finite);
-        sq_add_bits(ws[q] & 0xFFFF0000u, hi, lo, acc, finite);
-      }
-      if (++grp == 8) {
-        acc += (double)hi + (double)lo;
-        hi = lo = 0.f;
-        grp = 0;
-      }
-    }
-    const uint16_t* r = reinterpret_cast<const uint16_t*>(A + j * lda);
-    for (int64_t i = nv * 8 + threadIdx.x; i < m; i += blockDim.x) sq_add_bits((uint32_t)r[i] << 16, hi, lo, acc, finite);
-    acc += (double)hi + (double)lo;
-  }
-  if (!finite) atomicOr(&st->err, kErrNonFinite);
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-// FP32 columns: four elements per load when 16-byte aligned, each square's rounding
-// error recovered exactly by an FMA and summed in float-float groups of 64
-// (sq_add_f32), folded into FP64.
-__global__ void k_norm2_f32(int64_t m, int64_t n, const float* __restrict__ A, int64_t lda, double* part,
-                            DevState* st) {
-  double acc = 0.0;
-  bool finite = true;
-  const bool vec = (lda % 4) == 0 && (reinterpret_cast<uintptr_t>(A) % 16) == 0;
-  const int64_t nv = vec ? m / 4 : 0;
-  float hi = 0.f, lo = 0.f;
-  int grp = 0;
-  for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
-    const float* a = A + j * lda;
-    const float4* a4 = reinterpret_cast<const float4*>(a);
-    for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
-      const float4 w = __ldg(a4 + v);
-      sq_add_f32(w.x, hi, lo, acc, finite);
-      sq_add_f32(w.y, hi, lo, acc, finite);
-      sq_add_f32(w.z, hi, lo, acc, finite);
-      sq_add_f32(w.w, hi, lo, acc, finite);
-      if (++grp == 16) {
-        acc += (double)hi + (double)lo;
-        hi = lo = 0.f;
-        grp = 0;
-      }
-    }
-    for (int64_t i = nv * 4 + threadIdx.x; i < m; i += blockDim.x) {
-      sq_add_f32(a[i], hi, lo, acc, finite);
-      if (++grp == 16) {
-        acc += (double)hi + (double)lo;
-        hi = lo = 0.f;
-        grp = 0;
-      }
-    }
-  }
-  acc += (double)hi + (double)lo;
-  if (!finite) atomicOr(&st->err, kErrNonFinite);
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-template <typename T>
-cudaError_t norm2_partial(int64_t m, int64_t n, const T* A, int64_t lda, double* part, int nparts,
-                          DevState* st, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {
-    k_norm2_f32<<<nparts, 256, 0, s>>>(m, n, A, lda, part, st);
-    return cudaGetLastError();
-  }
-  if constexpr (sizeof(T) == 2) {
-    if ((lda % 8) == 0 && (reinterpret_cast<uintptr_t>(A) % 16) == 0) {
-      k_norm2_bf16<<<nparts, 256, 0, s>>>(m, n, A, lda, part, st);
-      return cudaGetLastError();
-    }
-  }
-  k_norm2_partial<T><<<nparts, 256, 0, s>>>(m, n, A, lda, part, st);
-  return cudaGetLastError();
-}
-
-__global__ void k_norm2_final(const double* part, int nparts, DevState* st) {
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[i];
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) st->norm2_A = tot;
-}
-
-cudaError_t norm2_final(const double* part, int nparts, DevState* st, cudaStream_t s) {
-  k_norm2_final<<<1, 256, 0, s>>>(part, nparts, st);
-  return cudaGetLastError();
-}
-
 // ============================================================ gather-GEMM
 // 64 x 64 output tile per block, K step 16, 256 threads each owning a 4 x 4
 // sub-tile strided by 16 (rows ty + 16 i, columns tx + 16 j), so that shared
@@ -1394,8 +1268,6 @@ cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, 
                                       const int32_t*, cudaStream_t);                                        \
   template cudaError_t gaussian_rows<T>(uint64_t, int64_t, int64_t, int64_t, T*, int64_t, const int32_t*,   \
                                         cudaStream_t);                                                      \
-  template cudaError_t norm2_partial<T>(int64_t, int64_t, const T*, int64_t, double*, int, DevState*,       \
-                                        cudaStream_t);                                                      \
   template cudaError_t splitk_reduce<T>(int64_t, int, int64_t, int, int64_t, const T*, T*, const int32_t*,  \
                                         cudaStream_t);                                                      \
   template cudaError_t splitk_reduce_ld<T>(int64_t, int, int64_t, int64_t, int, int64_t, const T*, T*,       \
@@ -1421,7 +1293,5 @@ template cudaError_t gaussian_rows<__nv_bfloat16>(uint64_t, int64_t, int64_t, in
                                                   const int32_t*, cudaStream_t);
 template cudaError_t gaussian_rows<__nv_fp8_e4m3>(uint64_t, int64_t, int64_t, int64_t, __nv_fp8_e4m3*, int64_t,
                                                   const int32_t*, cudaStream_t);
-template cudaError_t norm2_partial<__nv_bfloat16>(int64_t, int64_t, const __nv_bfloat16*, int64_t, double*, int,
-                                                  DevState*, cudaStream_t);
 
 }  // namespace rid

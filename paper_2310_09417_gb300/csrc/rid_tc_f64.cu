@@ -505,17 +505,20 @@ int f64emu_splits(int64_t m, int64_t n, int sms) {
   return best;
 }
 
-cudaError_t f64emu_prepare(const double* A, int64_t lda, int64_t m, int64_t n, int32_t* colexp, void* digits,
-                           cudaStream_t s) {
-  tc64::k_colexp<<<(int)(n < 4096 ? n : 4096), 256, 0, s>>>(A, lda, m, n, colexp);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+cudaError_t f64emu_split(const double* A, int64_t lda, int64_t m, int64_t n, const int32_t* colexp, void* digits,
+                         cudaStream_t s) {
   const int64_t nkb = digit_kblocks(m), ntl = digit_tiles(n);
   int64_t blocks = nkb * ntl;  // tiles
   if (blocks > 8192) blocks = 8192;
   tc64::k_split_digits<<<(int)blocks, 256, 0, s>>>(A, lda, m, n, nkb, ntl, colexp,
                                                    static_cast<__nv_bfloat16*>(digits));
   return cudaGetLastError();
+}
+
+cudaError_t f64emu_prepare(const double* A, int64_t lda, int64_t m, int64_t n, int32_t* colexp, void* digits,
+                           cudaStream_t s) {
+  cudaError_t e = f64_colexp(A, lda, m, n, colexp, s);
+  return e == cudaSuccess ? f64emu_split(A, lda, m, n, colexp, digits, s) : e;
 }
 
 cudaError_t f64_colexp(const double* A, int64_t lda, int64_t m, int64_t n, int32_t* E, cudaStream_t s) {

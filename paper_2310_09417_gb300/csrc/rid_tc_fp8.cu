@@ -184,75 +184,6 @@ __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
   }
 }
 
-// ------------------------------------------------------------------ ||A||_F^2 and finiteness
-// One block per column at a time: sum of (fp8(i,j) * scale(i/128, j))^2 in FP64.
-__global__ void k_norm2_fp8(int64_t m, int64_t n, const uint8_t* __restrict__ A, int64_t lda,
-                            const float* __restrict__ scale, int64_t nbs, double* part, DevState* st) {
-  double acc = 0.0;
-  bool finite = true;
-  for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
-    const uint8_t* a = A + j * lda;
-    for (int64_t i = threadIdx.x; i < m; i += blockDim.x) {
-      __nv_fp8_e4m3 q;
-      q.__x = a[i];
-      const double s = (double)scale[j * nbs + i / kBK];
-      const double v = (double)static_cast<float>(q) * s;
-      finite = finite && isfinite(v);
-      acc += v * v;
-    }
-  }
-  if (!finite) atomicOr(&st->err, kErrNonFinite);
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
-// ||A||_F^2 with 16 E4M3 values per load (columns 16-byte aligned: lda a multiple of
-// 16).  A vector's 16 values share one block scale; their squares are exact in
-// FP32 (at most 8 significant bits, between 2^-18 and 448^2) and are summed in
-// float-float (sq_twosum), then scaled by scale^2 and added in FP64: a few FP64
-// operations per 16 values instead of several per value.
-__global__ void k_norm2_fp8v(int64_t m, int64_t n, const uint8_t* __restrict__ A, int64_t lda,
-                             const float* __restrict__ scale, int64_t nbs, double* part, DevState* st) {
-  double acc = 0.0;
-  bool finite = true;
-  const int64_t nv = (m + 15) / 16;
-  for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
-    const uint4* a = reinterpret_cast<const uint4*>(A + j * lda);
-    for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
-      const uint4 w = __ldg(a + v);
-      uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-      const int64_t left = m - 16 * v;
-      if (left < 16) {  // the last vector of the column: rows past m are ignored
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (4 * q + k >= left) ws[q] &= ~(0xFFu << (8 * k));
-      }
-      const float sc = scale[j * nbs + (16 * v) / kBK];
-      if (!isfinite(sc)) finite = false;
-      float hi = 0.f, lo = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (__vcmpeq4(ws[q] & 0x7F7F7F7Fu, 0x7F7F7F7Fu) != 0u) finite = false;  // E4M3 NaN
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const __half2_raw hr =
-              __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((ws[q] >> (16 * h)) & 0xFFFFu), __NV_E4M3);
-          const float2 f = __half22float2(__half2(hr));
-          sq_twosum(__fmul_rn(f.x, f.x), hi, lo);
-          sq_twosum(__fmul_rn(f.y, f.y), hi, lo);
-        }
-      }
-      const double sd = (double)sc;
-      acc += ((double)hi + (double)lo) * (sd * sd);
-    }
-  }
-  if (!finite) atomicOr(&st->err, kErrNonFinite);
-  const double tot = block_sum(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = tot;
-}
-
 // ------------------------------------------------------------------ quantisation
 template <typename T>
 __device__ __forceinline__ float as_float(T x) {
@@ -374,16 +305,6 @@ cudaError_t tc_sketch_fp8(const void* A, int64_t lda, int64_t m, int64_t n, cons
   const int64_t nbs = (m + tc8::kBK - 1) / tc8::kBK;
   if (nt == 4) return launch_fp8<4>(ma, mw, scale, nbs, m, n, rows, kchunk, nz, out, out_ld, zstride, st, done, s);
   return launch_fp8<1>(ma, mw, scale, nbs, m, n, rows, kchunk, nz, out, out_ld, zstride, st, done, s);
-}
-
-cudaError_t norm2_fp8(int64_t m, int64_t n, const void* A, int64_t lda, const float* scale, double* part, int nparts,
-                      DevState* st, cudaStream_t s) {
-  const int64_t nbs = (m + tc8::kBK - 1) / tc8::kBK;
-  if ((lda % 16) == 0 && (reinterpret_cast<uintptr_t>(A) % 16) == 0)
-    tc8::k_norm2_fp8v<<<nparts, 256, 0, s>>>(m, n, static_cast<const uint8_t*>(A), lda, scale, nbs, part, st);
-  else
-    tc8::k_norm2_fp8<<<nparts, 256, 0, s>>>(m, n, static_cast<const uint8_t*>(A), lda, scale, nbs, part, st);
-  return cudaGetLastError();
 }
 
 cudaError_t quantize_fp8(int dtype, int64_t m, int64_t n, const void* A, int64_t lda, void* Q, int64_t ldq,
