@@ -48,8 +48,9 @@ int num_sms() {
   return cache[dev];
 }
 
-// Split-K factor of the 64 x 64 gather-GEMM (FP64 Schur products): enough blocks
-// for about four waves, at least 256 K per split.
+// Split-K factor of the FP64 Schur products: by 64 x 64 tiles, at least 256 K per split.
+// It fixes the order in which an entry is summed, and with it the bits of X, whose late
+// columns are sensitive to the last bit; the kernel's tiles are chosen apart from it.
 int choose_splits_gather(int64_t M, int64_t N, int64_t K, int sms, int cap) {
   const int64_t tiles = cdiv(M, 64) * cdiv(N, 64);
   int64_t s = cdiv(4 * (int64_t)sms, tiles);
@@ -58,8 +59,8 @@ int choose_splits_gather(int64_t M, int64_t N, int64_t K, int sms, int cap) {
   return (int)imax(1, s);
 }
 
-// Split-K factor for the store GEMM (k_sgemm_gather: 128 x 64 tiles, two blocks per
-// SM in FP32, one in FP64): the count (at most cap, at least 128 K per split)
+// Split-K factor of the FP32 store GEMM (k_sgemm_gather: 128 x 64 tiles, two blocks per
+// SM) and of the FP64 sketch (per_sm 1: the count fixes its order of summation): the count (at most cap, at least 128 K per split)
 // minimising waves x (K per split + a fixed cost).
 int choose_splits_sgemm(int64_t M, int64_t N, int64_t K, int sms, int cap, int per_sm) {
   const int64_t tiles = cdiv(M, 128) * cdiv(N, 64);
@@ -784,7 +785,6 @@ class Engine {
         }
       }
       if (!done_tc) {
-        // FP64 Schur products run on the 64 x 64 kernel: about four blocks per SM
         nz = gemm_splits((int)tb, sizeof(T) == 4 ? choose_splits_sgemm(na, w, tb, p_.sms, p_.s2max, 2)
                                                  : choose_splits_gather(na, w, tb, p_.sms, p_.s2max));
         Operand<T> a{X_, ldx_, act_[cur_], 0};

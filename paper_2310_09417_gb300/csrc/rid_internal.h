@@ -75,6 +75,8 @@ struct EpiArgs {
 // along N).  The K range is split across gridDim.z in chunks of `kchunk`.
 // The split count actually used (<= requested) is what gemm_splits() returns.
 int gemm_splits(int K, int splits);
+// Split count of an FP64 product with a free summation order (already in the sense of gemm_splits).
+int dgemm_splits(int64_t M, int64_t N, int64_t K, int sms, int cap);
 template <typename T>
 cudaError_t gemm_gather(int M, int N, int K, int splits, bool b_kmajor, Operand<T> a, Operand<T> b,
                         int epi, EpiArgs<T> ep, const int32_t* done, cudaStream_t s);

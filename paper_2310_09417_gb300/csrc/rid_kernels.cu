@@ -120,64 +120,166 @@ cudaError_t gaussian_rows(uint64_t seed, int64_t row0, int64_t rows, int64_t m, 
 }
 
 // ============================================================ gather-GEMM
-// 64 x 64 output tile per block, K step 16, 256 threads each owning a 4 x 4
-// sub-tile strided by 16 (rows ty + 16 i, columns tx + 16 j), so that shared
-// reads of a warp hit consecutive words and global writes are coalesced.
-constexpr int kGM = 64, kGN = 64, kGK = 16;
+// FP64, every product: a DM x DN output tile per block, each thread owning 2 x (DN / 8)
+// entries strided by DM / 2 and 8 (shared reads of a warp hit consecutive words, global
+// writes are coalesced), K steps of 16 double-buffered through registers and shared
+// memory.  The bound is the FP64 pipe, about two FMAs per clock per SM: a warp
+// instruction occupies it for sixteen clocks, so shared memory and L2 are idle
+// whatever the tile, and the tile only has to give every SM the same share: 32 x 32
+// with many tiles, 16 x 16 with few (dgemm_small_tiles).  64 x 64 and 128 x 64 tiles
+// left most SMs without work where the products are small or narrow.  Measured: the
+// sketch of 600 x 400 with 56 rows 326 -> 34 us, of 4000 x 1000 with 64 rows 519 -> 401
+// (the rate of the FP64 pipe), the Schur product of 1000
+// rows and up to 384 pivots 271 -> 42, the QR's V^T C (4000 x 96 by 32) 570 -> 12.
+// Every entry is summed over k in increasing order, one FMA per term, within its split:
+// the tile does not change a bit.
+constexpr int kDK = 16;
 
-template <typename T, bool BK, int EPI>
-__global__ void __launch_bounds__(256)
-    k_gemm_gather(int M, int N, int K, int kchunk, Operand<T> a, Operand<T> b, EpiArgs<T> ep,
-                  const int32_t* done) {
+template <int DM, int DN, bool BK, int EPI>
+__global__ void __launch_bounds__(DM * 4)
+    k_dgemm(int M, int N, int K, int kchunk, Operand<double> a, Operand<double> b, EpiArgs<double> ep,
+            const int32_t* done) {
+  constexpr int NT = DM * 4, TN = DN / 8;
+  constexpr int NA = DM * kDK / NT, NB = DN * kDK / NT;  // loads of a K step per thread
+  static_assert(DM == DN, "the loaders of both operands cover the same rows");
   if (done != nullptr && *done) return;
-  __shared__ T As[kGK][kGM + 1];
-  __shared__ T Bs[kGK][kGN + 1];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.x * kGM, n0 = blockIdx.y * kGN;
+  __shared__ double As[2][kDK][DM + 1];
+  __shared__ double Bs[2][kDK][DN + 1];
+  const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+  const unsigned mt = ((unsigned)M + DM - 1) / DM;  // tiles in one grid dimension, M fastest
+  const int m0 = (int)(blockIdx.x % mt) * DM, n0 = (int)(blockIdx.x / mt) * DN;
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
+  // K-major loader: k = tid % 16 of rows tid / 16 + i NT / 16 (128-byte runs); N-major
+  // loader: column tid % DN of k rows tid / DN + i NT / DN
+  const int lk = tid & 15, lr = tid >> 4;
+  const int lc = tid % DN, lq = tid / DN;
+  const double* ap[NA];
+  const double* bp[NB];
+#pragma unroll
+  for (int i = 0; i < NA; ++i) {
+    const int m = m0 + lr + NT / 16 * i, n = n0 + lr + NT / 16 * i;
+    ap[i] = m < M ? a.base + (int64_t)(a.idx ? a.idx[m] : m) * a.ld + a.off : nullptr;
+    bp[i] = (BK && n < N) ? b.base + (int64_t)(b.idx ? b.idx[n] : n) * b.ld + b.off : nullptr;
+  }
+  double ra[NA], rb[NB];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) ra[i] = (ap[i] != nullptr && k0 + lk < kend) ? ap[i][k0 + lk] : 0.0;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      if (BK) {
+        rb[i] = (bp[i] != nullptr && k0 + lk < kend) ? bp[i][k0 + lk] : 0.0;
+      } else {
+        const int k = k0 + lq + NT / DN * i;
+        rb[i] = (k < kend && n0 + lc < N) ? b.base[(int64_t)(b.idx ? b.idx[k] : k) * b.ld + b.off + n0 + lc] : 0.0;
+      }
+    }
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int i = 0; i < NA; ++i) As[buf][lk][lr + NT / 16 * i] = ra[i];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      if (BK)
+        Bs[buf][lk][lr + NT / 16 * i] = rb[i];
+      else
+        Bs[buf][lq + NT / DN * i][lc] = rb[i];
+    }
+  };
+  double acc[2][TN];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
+  int buf = 0;
+  if (kbeg < kend) {
+    load(kbeg);
+    store(0);
+  }
+  __syncthreads();
+  for (int k0 = kbeg; k0 < kend; k0 += kDK, buf ^= 1) {
+    if (k0 + kDK < kend) load(k0 + kDK);
+#pragma unroll
+    for (int kk = 0; kk < kDK; ++kk) {
+      double av[2], bv[TN];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) av[i] = As[buf][kk][ty + DM / 2 * i];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) bv[j] = Bs[buf][kk][tx + 8 * j];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+    }
+    if (k0 + kDK < kend) store(buf ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int r = m0 + ty + DM / 2 * i;
+    if (r >= M) continue;
+    double* o;
+    if (EPI == kEpiStore) {
+      o = ep.out + blockIdx.z * ep.zstride + (int64_t)r * ep.out_ld;
+    } else {
+      if (ep.skip != nullptr && ep.skip[r] != 0) continue;
+      o = ep.out + (int64_t)(ep.out_idx ? ep.out_idx[r] : r) * ep.out_ld;
+    }
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int c = n0 + tx + 8 * j;
+      if (c >= N) continue;
+      if (EPI == kEpiStore)
+        o[c] = acc[i][j];
+      else
+        o[c] -= acc[i][j];
+    }
+  }
+}
 
-  // K-major loaders: row lr, four consecutive k starting at lk
+// FP32 rank-bt subtraction (blocks wider than the tensor-core update takes, and the
+// QR): 64 x 64 output tile per block, K step 16, 256 threads each owning a 4 x 4
+// sub-tile strided by 16 (rows ty + 16 i, columns tx + 16 j), so that shared reads of
+// a warp hit consecutive words and global writes are coalesced.  B is N-major.
+constexpr int kGM = 64, kGN = 64, kGK = 16;
+
+__global__ void __launch_bounds__(256)
+    k_gemm_sub(int M, int N, int K, Operand<float> a, Operand<float> b, EpiArgs<float> ep, const int32_t* done) {
+  if (done != nullptr && *done) return;
+  __shared__ float As[kGK][kGM + 1];
+  __shared__ float Bs[kGK][kGN + 1];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int m0 = blockIdx.x * kGM, n0 = blockIdx.y * kGN;
+  // K-major loader: row lr, four consecutive k starting at lk
   const int lr = tid >> 2, lk = (tid & 3) * 4;
-  const T* arow = nullptr;
+  const float* arow = nullptr;
   if (m0 + lr < M) arow = a.base + (int64_t)(a.idx ? a.idx[m0 + lr] : m0 + lr) * a.ld + a.off;
-  const T* brow_k = nullptr;
-  if (BK && n0 + lr < N) brow_k = b.base + (int64_t)(b.idx ? b.idx[n0 + lr] : n0 + lr) * b.ld + b.off;
   // N-major loader: k row lq, four consecutive columns starting at lc
   const int lq = tid >> 4, lc = (tid & 15) * 4;
-
-  T acc[4][4];
+  float acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-
-  for (int k0 = kbeg; k0 < kend; k0 += kGK) {
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  for (int k0 = 0; k0 < K; k0 += kGK) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int k = k0 + lk + u;
-      As[lk + u][lr] = (arow != nullptr && k < kend) ? arow[k] : T(0);
+      As[lk + u][lr] = (arow != nullptr && k < K) ? arow[k] : 0.f;
     }
-    if (BK) {
+    const int q = k0 + lq;
+    const float* br = nullptr;
+    if (q < K) br = b.base + (int64_t)(b.idx ? b.idx[q] : q) * b.ld + b.off;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int k = k0 + lk + u;
-        Bs[lk + u][lr] = (brow_k != nullptr && k < kend) ? brow_k[k] : T(0);
-      }
-    } else {
-      const int q = k0 + lq;
-      const T* br = nullptr;
-      if (q < kend) br = b.base + (int64_t)(b.idx ? b.idx[q] : q) * b.ld + b.off;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int c = n0 + lc + u;
-        Bs[lq][lc + u] = (br != nullptr && c < N) ? br[c] : T(0);
-      }
+    for (int u = 0; u < 4; ++u) {
+      const int c = n0 + lc + u;
+      Bs[lq][lc + u] = (br != nullptr && c < N) ? br[c] : 0.f;
     }
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < kGK; ++kk) {
-      T av[4], bv[4];
+      float av[4], bv[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) av[i] = As[kk][ty + 16 * i];
 #pragma unroll
@@ -185,35 +287,24 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
     __syncthreads();
   }
-
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int r = m0 + ty + 16 * i;
-    if (r >= M) continue;
-    if (EPI == kEpiStore) {
-      T* o = ep.out + blockIdx.z * ep.zstride + (int64_t)r * ep.out_ld;
+    if (r >= M || (ep.skip != nullptr && ep.skip[r] != 0)) continue;
+    float* o = ep.out + (int64_t)(ep.out_idx ? ep.out_idx[r] : r) * ep.out_ld;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = n0 + tx + 16 * j;
-        if (c < N) o[c] = acc[i][j];
-      }
-    } else {
-      if (ep.skip != nullptr && ep.skip[r] != 0) continue;
-      T* o = ep.out + (int64_t)(ep.out_idx ? ep.out_idx[r] : r) * ep.out_ld;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = n0 + tx + 16 * j;
-        if (c < N) o[c] -= acc[i][j];
-      }
+    for (int j = 0; j < 4; ++j) {
+      const int c = n0 + tx + 16 * j;
+      if (c < N) o[c] -= acc[i][j];
     }
   }
 }
 
-// Gather-GEMM for the store epilogue (the sketch and Schur products, FP32 and FP64):
+// FP32 gather-GEMM for the store epilogue (the sketch and Schur products):
 // 128 x 64 tile, 256 threads each owning 8 rows x 4 columns (thread (ty, tx) =
 // (tid / 16, tid % 16): a warp reads two A fragments and sixteen B fragments of
 // shared memory per k, broadcast across its lanes), K steps of 32 double-buffered
@@ -222,28 +313,14 @@ __global__ void __launch_bounds__(256)
 // in 32 distinct banks and the 16-byte fragment reads stay aligned.
 constexpr int kSM = 128, kSN = 64, kSK = 32;
 constexpr int kSAld = kSM + 4, kSBld = kSN + 4;
-template <typename T>
-constexpr size_t sgemm_smem() {
-  return (size_t)2 * kSK * (kSAld + kSBld) * sizeof(T);
-}
+constexpr size_t kSgemmSmem = (size_t)2 * kSK * (kSAld + kSBld) * sizeof(float);
 
-// Vector of four for the fragment reads.
-template <typename T>
-struct Vec4;
-template <>
-struct Vec4<float> {
-  using type = float4;
-};
-template <>
-struct Vec4<double> {
-  using type = double4_32a;
-};
-
-template <typename T, bool BK>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
-    k_sgemm_gather(int M, int N, int K, int kchunk, Operand<T> a, Operand<T> b, EpiArgs<T> ep,
+template <bool BK>
+__global__ void __launch_bounds__(256, 2)
+    k_sgemm_gather(int M, int N, int K, int kchunk, Operand<float> a, Operand<float> b, EpiArgs<float> ep,
                    const int32_t* done) {
-  using V4 = typename Vec4<T>::type;
+  using T = float;
+  using V4 = float4;
   if (done != nullptr && *done) return;
   extern __shared__ __align__(32) unsigned char sg_raw[];
   T* As = reinterpret_cast<T*>(sg_raw);  // [2][kSK][kSAld]
@@ -366,39 +443,86 @@ int gemm_splits(int K, int splits) {
   return (K + kchunk - 1) / kchunk;
 }
 
-template <typename T>
-cudaError_t gemm_gather(int M, int N, int K, int splits, bool b_kmajor, Operand<T> a, Operand<T> b,
-                        int epi, EpiArgs<T> ep, const int32_t* done, cudaStream_t s) {
+static int64_t tiles_of(int64_t M, int64_t N, int64_t d) { return ((M + d - 1) / d) * ((N + d - 1) / d); }
+
+// Split-K count of an FP64 product whose summation order is free (the QR's): the count
+// (at most cap, at least 32 K per split) that minimises an SM's share, 32 x 32 tiles per
+// SM x (K per split + a fixed cost of about 24 K for a tile's prologue and its partial's
+// store and re-read).
+int dgemm_splits(int64_t M, int64_t N, int64_t K, int sms, int cap) {
+  const int64_t tiles = tiles_of(M, N, 32);
+  int best = 1;
+  double best_t = 1e300;
+  for (int64_t s = 1; s <= cap && (s == 1 || K / s >= 32); ++s) {
+    const double t = (double)((tiles * s + sms - 1) / sms) * ((double)((K + s - 1) / s) + 24.0);
+    if (t < best_t * (1.0 - 1e-9)) {
+      best_t = t;
+      best = (int)s;
+    }
+  }
+  return gemm_splits((int)K, best);
+}
+
+// 16 x 16 tiles when they make the busiest SM's share of the product smaller by more
+// than the tenth that their prologues and loads cost.
+static bool dgemm_small_tiles(int64_t M, int64_t N, int64_t nz, int sms) {
+  const int64_t t32 = (tiles_of(M, N, 32) * nz + sms - 1) / sms * 4, t16 = (tiles_of(M, N, 16) * nz + sms - 1) / sms;
+  return (double)t16 * 1.1 < (double)t32;
+}
+
+template <int D>
+static cudaError_t dgemm(int M, int N, int K, int kchunk, bool b_kmajor, const Operand<double>& a,
+                         const Operand<double>& b, int epi, const EpiArgs<double>& ep, const int32_t* done,
+                         cudaStream_t s) {
+  const int64_t tiles = tiles_of(M, N, D);
+  if (tiles > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)tiles, 1, (K + kchunk - 1) / kchunk);
+  if (epi == kEpiStore) {
+    if (b_kmajor)
+      k_dgemm<D, D, true, kEpiStore><<<grid, D * 4, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
+    else
+      k_dgemm<D, D, false, kEpiStore><<<grid, D * 4, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
+  } else {
+    if (b_kmajor || grid.z != 1) return cudaErrorInvalidValue;
+    k_dgemm<D, D, false, kEpiSubRows><<<grid, D * 4, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
+  }
+  return cudaGetLastError();
+}
+
+template <>
+cudaError_t gemm_gather<double>(int M, int N, int K, int splits, bool b_kmajor, Operand<double> a, Operand<double> b,
+                                int epi, EpiArgs<double> ep, const int32_t* done, cudaStream_t s) {
+  if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
+  const int kchunk = split_chunk(K, splits), nz = (K + kchunk - 1) / kchunk;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  return dgemm_small_tiles(M, N, nz, sms) ? dgemm<16>(M, N, K, kchunk, b_kmajor, a, b, epi, ep, done, s)
+                                          : dgemm<32>(M, N, K, kchunk, b_kmajor, a, b, epi, ep, done, s);
+}
+
+template <>
+cudaError_t gemm_gather<float>(int M, int N, int K, int splits, bool b_kmajor, Operand<float> a, Operand<float> b,
+                               int epi, EpiArgs<float> ep, const int32_t* done, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   const int kchunk = split_chunk(K, splits);
   splits = (K + kchunk - 1) / kchunk;
-  // the double-buffered kernel for stores; in FP64 only for the sketch (K-major B):
-  // its one block per SM measured slower than the 64 x 64 kernel on the Schur shapes
-  if (epi == kEpiStore && (sizeof(T) == 4 || b_kmajor)) {
-    constexpr size_t smem = sgemm_smem<T>();
+  if (epi == kEpiStore) {
     static SmemLimit lim_kmajor, lim_nmajor;
-    cudaError_t e = raise_smem(k_sgemm_gather<T, true>, smem, lim_kmajor);
-    if (e == cudaSuccess) e = raise_smem(k_sgemm_gather<T, false>, smem, lim_nmajor);
+    cudaError_t e = raise_smem(k_sgemm_gather<true>, kSgemmSmem, lim_kmajor);
+    if (e == cudaSuccess) e = raise_smem(k_sgemm_gather<false>, kSgemmSmem, lim_nmajor);
     if (e != cudaSuccess) return e;
     dim3 g((M + kSM - 1) / kSM, (N + kSN - 1) / kSN, splits);
     if (b_kmajor)
-      k_sgemm_gather<T, true><<<g, 256, smem, s>>>(M, N, K, kchunk, a, b, ep, done);
+      k_sgemm_gather<true><<<g, 256, kSgemmSmem, s>>>(M, N, K, kchunk, a, b, ep, done);
     else
-      k_sgemm_gather<T, false><<<g, 256, smem, s>>>(M, N, K, kchunk, a, b, ep, done);
+      k_sgemm_gather<false><<<g, 256, kSgemmSmem, s>>>(M, N, K, kchunk, a, b, ep, done);
     return cudaGetLastError();
   }
-  dim3 grid((M + kGM - 1) / kGM, (N + kGN - 1) / kGN, splits);
-  if (b_kmajor) {
-    if (epi == kEpiStore)
-      k_gemm_gather<T, true, kEpiStore><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
-    else
-      k_gemm_gather<T, true, kEpiSubRows><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
-  } else {
-    if (epi == kEpiStore)
-      k_gemm_gather<T, false, kEpiStore><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
-    else
-      k_gemm_gather<T, false, kEpiSubRows><<<grid, 256, 0, s>>>(M, N, K, kchunk, a, b, ep, done);
-  }
+  if (b_kmajor || splits != 1) return cudaErrorInvalidValue;
+  dim3 grid((M + kGM - 1) / kGM, (N + kGN - 1) / kGN);
+  k_gemm_sub<<<grid, 256, 0, s>>>(M, N, K, a, b, ep, done);
   return cudaGetLastError();
 }
 
@@ -1264,8 +1388,6 @@ cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, 
 
 // ============================================================ instantiations
 #define RID_INST(T)                                                                                         \
-  template cudaError_t gemm_gather<T>(int, int, int, int, bool, Operand<T>, Operand<T>, int, EpiArgs<T>,    \
-                                      const int32_t*, cudaStream_t);                                        \
   template cudaError_t gaussian_rows<T>(uint64_t, int64_t, int64_t, int64_t, T*, int64_t, const int32_t*,   \
                                         cudaStream_t);                                                      \
   template cudaError_t splitk_reduce<T>(int64_t, int, int64_t, int, int64_t, const T*, T*, const int32_t*,  \

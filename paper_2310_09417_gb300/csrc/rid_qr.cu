@@ -6,9 +6,9 @@
 // QR (LAPACK dgeqrf's convention): H_j = I - tau_j v_j v_j^T with v_j(j) = 1,
 // R on and above the diagonal, v_j below it.  Panels of 32 columns:
 //   * k_qr_panel: one cooperative launch over the panel's rows (staged in shared
-//     memory), two bounded grid barriers per column (the column's sum of squares,
-//     then the dot products with the later columns of the panel), every
-//     reduction summed in block order (deterministic), then V^T V and the
+//     memory), one bounded grid barrier per column (the column's sum of squares and
+//     its products with the later columns of the panel), every reduction summed in
+//     a fixed order (deterministic), then V^T V and the
 //     compact-WY factor T with H_1 ... H_w = I - V T V^T (Schreiber and Van Loan).
 //   * the trailing columns: C2 := C2 - V T^T (V^T C2) through the gather-GEMM
 //     (split-K product, reduction times T, rank-32 subtract).
@@ -42,101 +42,113 @@ struct PanelRows {
   __device__ __forceinline__ T& operator()(int r, int c) const { return base[r * rs + c * cs]; }
 };
 
+// One column costs one grid barrier: the sum of squares below the diagonal and the
+// products of that part of column j with the later columns are one reduction, taken
+// before the reflector is known (v = scale x below the diagonal, 1 on it), and
+// w_c = v^T S(:, c) = S(j, c) + scale sum_{r > j} S(r, j) S(r, c) follows from it.
+// What bounds it is the barrier and the FP64 pipe (two per clock per SM) on the
+// block's own products, on the sum over blocks that every block repeats, and on the
+// update; kQrRows rows per block balance them.  Lanes run along the columns, so no
+// product is spent on shuffles.
+constexpr int kQrRows = 64;
+
 template <typename T>
 __global__ void __launch_bounds__(kQrThreads)
-    k_qr_panel(int mr, int w, T* __restrict__ P, int64_t ld, int chunk, int use_smem, double* __restrict__ pssq,
-               double* __restrict__ pdot, double* __restrict__ pgram, T* __restrict__ tau, T* __restrict__ Vc,
+    k_qr_panel(int mr, int w, T* __restrict__ P, int64_t ld, int chunk, int use_smem, double* __restrict__ pdot,
+               double* __restrict__ prow, double* __restrict__ pgram, T* __restrict__ tau, T* __restrict__ Vc,
                int64_t ldv, T* __restrict__ Tm, unsigned* ctr, DevState* st) {
   extern __shared__ __align__(16) unsigned char qr_raw[];
-  __shared__ double s_w[kQrW];
-  __shared__ double s_par[3];  // tau, beta, scale
+  constexpr int nw = kQrThreads / 32;
+  __shared__ double s_part[nw][kQrW];  // per warp, per column
+  __shared__ double s_row[kQrW];       // row j of the panel
+  __shared__ double s_tw[kQrW];        // tau_j w_c
+  __shared__ double s_par[3];          // tau, beta, scale
   const int nb = gridDim.x, bid = blockIdx.x, tid = threadIdx.x;
-  const int lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int lane = tid & 31, wid = tid >> 5;
   const int r0 = bid * chunk;
   const int nr = max(0, min(mr, r0 + chunk) - r0);
   PanelRows<T> S = use_smem ? PanelRows<T>{reinterpret_cast<T*>(qr_raw), (int64_t)(w + 1), 1}
                             : PanelRows<T>{P + r0, 1, ld};
   if (use_smem)
-    for (int e = tid; e < nr * w; e += blockDim.x) {
+    for (int e = tid; e < nr * w; e += kQrThreads) {
       const int r = e % nr, c = e / nr;
       S(r, c) = P[(int64_t)(r0 + r) + (int64_t)c * ld];
     }
   __syncthreads();
   unsigned nbar = 0;
   for (int j = 0; j < w; ++j) {
-    // 1. the sum of squares of column j below the diagonal over this block's rows
-    double acc = 0.0;
-    for (int r = tid; r < nr; r += blockDim.x)
-      if (r0 + r > j) {
-        const double x = (double)S(r, j);
-        acc += x * x;
-      }
-    acc = block_sum(acc);
-    if (tid == 0) {
-      pssq[((j & 1) * nb + bid) * 2] = acc;
-      if (bid == 0) pssq[((j & 1) * nb) * 2 + 1] = (double)S(j, j);  // block 0 owns rows 0 .. w-1
+    // 1. this block's sums over its rows below the diagonal (block 0 owns rows 0 .. w-1)
+    const bool mine = lane >= j && lane < w;
+    const int rb = max(0, j + 1 - r0);  // first local row below the diagonal
+    double d = 0.0;
+    for (int r = rb + wid; r < nr; r += nw)
+      if (mine) d += (double)S(r, j) * (double)S(r, lane);
+    s_part[wid][lane] = d;
+    __syncthreads();
+    if (wid == 0 && mine) {
+      double t = 0.0;
+#pragma unroll
+      for (int q = 0; q < nw; ++q) t += s_part[q][lane];
+      pdot[((int64_t)(j & 1) * nb + bid) * kQrW + lane] = t;
+      if (bid == 0) prow[(j & 1) * kQrW + lane] = (double)S(j, lane);
     }
     if (!grid_barrier(ctr, ++nbar * (unsigned)nb, st)) return;
-    // 2. the reflector (every block, identically)
-    if (tid == 0) {
-      double s2 = 0.0;
-      for (int b = 0; b < nb; ++b) s2 += __ldcg(&pssq[((j & 1) * nb + b) * 2]);
-      const double x0 = __ldcg(&pssq[((j & 1) * nb) * 2 + 1]);
-      double t = 0.0, beta = x0, scale = 0.0;
+    // 2. the sums over all blocks and the reflector (every block, identically)
+    {
+      const double* src = pdot + (int64_t)(j & 1) * nb * kQrW + lane;
+      double t = 0.0;
+      for (int q0 = wid; q0 < nb; q0 += 8 * nw) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = (mine && q0 + u * nw < nb) ? __ldcg(src + (int64_t)(q0 + u * nw) * kQrW) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t += v[u];
+      }
+      if (wid == 0 && mine) s_row[lane] = __ldcg(&prow[(j & 1) * kQrW + lane]);
+      s_part[wid][lane] = t;
+    }
+    __syncthreads();
+    if (wid == 0) {
+      double t = 0.0;
+#pragma unroll
+      for (int q = 0; q < nw; ++q) t += s_part[q][lane];
+      const double s2 = __shfl_sync(0xffffffffu, t, j), x0 = s_row[j];
+      double tj = 0.0, beta = x0, scale = 0.0;
       if (s2 > 0.0) {
         const double nrm = sqrt(x0 * x0 + s2);
         beta = x0 >= 0.0 ? -nrm : nrm;
-        t = (beta - x0) / beta;
+        tj = (beta - x0) / beta;
         scale = 1.0 / (x0 - beta);
       }
-      s_par[0] = t;
-      s_par[1] = beta;
-      s_par[2] = scale;
+      if (lane > j && lane < w) s_tw[lane] = tj * (s_row[lane] + scale * t);
+      if (lane == 0) {
+        s_par[0] = tj;
+        s_par[1] = beta;
+        s_par[2] = scale;
+        if (bid == 0) tau[j] = (T)tj;
+      }
     }
     __syncthreads();
-    const double t = s_par[0];
-    for (int r = tid; r < nr; r += blockDim.x)
-      if (r0 + r > j) S(r, j) = (T)((double)S(r, j) * s_par[2]);
-    if (bid == 0 && tid == 0) tau[j] = (T)t;
-    __syncthreads();
-    // 3. the later columns of the panel: w_c = v^T S(:, c), then S(:, c) -= tau v w_c
-    if (j + 1 < w && t != 0.0) {
-      for (int c = j + 1 + wid; c < w; c += nw) {
-        double d = 0.0;
-        for (int r = lane; r < nr; r += 32) {
-          const int gi = r0 + r;
-          if (gi >= j) d += (gi == j ? 1.0 : (double)S(r, j)) * (double)S(r, c);
-        }
-        d = warp_sum(d);
-        if (lane == 0) pdot[((j & 1) * nb + bid) * kQrW + c] = d;
-      }
-      if (!grid_barrier(ctr, ++nbar * (unsigned)nb, st)) return;
-      for (int c = j + 1 + tid; c < w; c += blockDim.x) {
-        double d = 0.0;
-        for (int b = 0; b < nb; ++b) d += __ldcg(&pdot[((j & 1) * nb + b) * kQrW + c]);
-        s_w[c] = d;
-      }
-      __syncthreads();
-      const int ncol = w - j - 1;
-      for (int e = tid; e < nr * ncol; e += blockDim.x) {
-        const int r = e % nr, c = j + 1 + e / nr;
-        const int gi = r0 + r;
-        if (gi >= j) {
-          const double v = gi == j ? 1.0 : (double)S(r, j);
-          S(r, c) = (T)((double)S(r, c) - t * v * s_w[c]);
-        }
-      }
-      __syncthreads();
+    // 3. v below the diagonal, S(:, c) -= tau v w_c for the later columns
+    const double tj = s_par[0], scale = s_par[2];
+    for (int r = rb + wid; r < nr; r += nw) {
+      const T v = (T)((double)S(r, j) * scale);
+      __syncwarp();
+      if (lane == j) S(r, j) = v;
+      if (lane > j && lane < w && tj != 0.0) S(r, lane) = (T)((double)S(r, lane) - (double)v * s_tw[lane]);
     }
-    if (bid == 0 && tid == 0) S(j, j) = (T)s_par[1];  // R(j, j)
+    if (bid == 0 && wid == 0) {
+      if (lane == j) S(j, j) = (T)s_par[1];  // R(j, j)
+      if (lane > j && lane < w && tj != 0.0) S(j, lane) = (T)((double)S(j, lane) - s_tw[lane]);
+    }
     __syncthreads();
   }
   // 4. V (unit diagonal, zero above) for the GEMMs, V^T V partials, the rows back
-  for (int e = tid; e < nr * w; e += blockDim.x) {
+  for (int e = tid; e < nr * w; e += kQrThreads) {
     const int r = e % nr, c = e / nr, gi = r0 + r;
     Vc[(int64_t)gi + (int64_t)c * ldv] = gi > c ? S(r, c) : (gi == c ? T(1) : T(0));
   }
-  for (int e = tid; e < w * w; e += blockDim.x) {
+  for (int e = tid; e < w * w; e += kQrThreads) {
     const int a = e / w, c = e % w;
     double g = 0.0;
     if (a <= c)
@@ -149,7 +161,7 @@ __global__ void __launch_bounds__(kQrThreads)
     pgram[(int64_t)bid * kQrW * kQrW + e] = g;
   }
   if (use_smem)
-    for (int e = tid; e < nr * w; e += blockDim.x) {
+    for (int e = tid; e < nr * w; e += kQrThreads) {
       const int r = e % nr, c = e / nr;
       P[(int64_t)(r0 + r) + (int64_t)c * ld] = S(r, c);
     }
@@ -158,46 +170,71 @@ __global__ void __launch_bounds__(kQrThreads)
   // 5. T (w x w upper, row-major): T(j,j) = tau_j, T(0:j, j) = -tau_j T(0:j,0:j) V(:,0:j)^T v_j
   __shared__ double G[kQrW][kQrW + 1];
   __shared__ double Ts[kQrW][kQrW + 1];
-  for (int e = tid; e < w * w; e += blockDim.x) {
+  for (int e = tid; e < w * w; e += kQrThreads) {
     const int a = e / w, c = e % w;
     double g = 0.0;
-    for (int b = 0; b < nb; ++b) g += __ldcg(&pgram[(int64_t)b * kQrW * kQrW + e]);
+    if (a < c)
+      for (int b0 = 0; b0 < nb; b0 += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b0 + u < nb ? __ldcg(&pgram[(int64_t)(b0 + u) * kQrW * kQrW + e]) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) g += v[u];
+      }
     G[a][c] = g;
     Ts[a][c] = 0.0;
   }
   __syncthreads();
-  for (int j = 0; j < w; ++j) {
-    const double tj = (double)__ldcg(&tau[j]);
-    if (tid < j) {
+  {
+    const int i = tid >> 3, part = tid & 7;  // eight threads per row of T (kQrThreads = 8 kQrW)
+    for (int j = 0; j < w; ++j) {
+      const double tj = (double)__ldcg(&tau[j]);
       double s = 0.0;
-      for (int l = tid; l < j; ++l) s += Ts[tid][l] * G[l][j];
-      Ts[tid][j] = -tj * s;
+      if (i < j)
+        for (int l = i + part; l < j; l += 8) s += Ts[i][l] * G[l][j];
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      s += __shfl_xor_sync(0xffffffffu, s, 4);
+      if (i < j && part == 0) Ts[i][j] = -tj * s;
+      if (tid == 0) Ts[j][j] = tj;
+      __syncthreads();
     }
-    if (tid == 0) Ts[j][j] = tj;
-    __syncthreads();
   }
-  for (int e = tid; e < w * w; e += blockDim.x) Tm[e] = (T)Ts[e / w][e % w];
+  for (int e = tid; e < w * w; e += kQrThreads) Tm[e] = (T)Ts[e / w][e % w];
 }
 
 static size_t qr_panel_smem(int chunk, int w, size_t esz, bool staged) {
   return staged ? (size_t)chunk * (w + 1) * esz : 0;
 }
 
-// W2^T (k2 x w, row-major) = (sum_z Wp[z]) T  (trans = 0) or ... T^T (trans = 1).
+// W2^T (k2 x w, row-major) = (sum_z Wp[z]) T  (trans = 0) or ... T^T (trans = 1): a
+// warp per row, lane l sums its column's partials (coalesced, eight loads in flight),
+// then every lane forms its column of the product from the row in shared memory.
+constexpr int kWtRows = 4;
 template <typename T>
-__global__ void k_qr_wt(int k2, int w, int nz, int64_t zs, const T* __restrict__ Wp, const T* __restrict__ Tm,
-                        int trans, T* __restrict__ W2) {
-  const int64_t total = (int64_t)k2 * w;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / w;
-    const int c = (int)(e - r * w);
-    T acc = T(0);
-    for (int l = 0; l < w; ++l) {
-      T s = T(0);
-      for (int z = 0; z < nz; ++z) s += Wp[z * zs + r * w + l];
-      acc += s * (trans ? Tm[c * w + l] : Tm[l * w + c]);
+__global__ void __launch_bounds__(32 * kWtRows)
+    k_qr_wt(int k2, int w, int nz, int64_t zs, const T* __restrict__ Wp, const T* __restrict__ Tm, int trans,
+            T* __restrict__ W2) {
+  __shared__ T s_row[kWtRows][kQrW];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int64_t r = blockIdx.x * (int64_t)kWtRows + wid; r < k2; r += (int64_t)gridDim.x * kWtRows) {
+    T s = T(0);
+    if (lane < w)
+      for (int z0 = 0; z0 < nz; z0 += 8) {
+        T v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = z0 + u < nz ? Wp[(z0 + u) * zs + r * w + lane] : T(0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
+      }
+    s_row[wid][lane] = s;
+    __syncwarp();
+    if (lane < w) {
+      T acc = T(0);
+      for (int l = 0; l < w; ++l) acc += s_row[wid][l] * (trans ? Tm[lane * w + l] : Tm[l * w + lane]);
+      W2[r * w + lane] = acc;
     }
-    W2[e] = acc;
+    __syncwarp();
   }
 }
 
@@ -273,37 +310,49 @@ __global__ void k_transpose(int64_t rows, int64_t cols, const T* __restrict__ in
 
 // R (k x k upper triangle of the factored matrix, column-major, ld) as row-major
 // Rrm (k x k, zero below the diagonal) and the inverse of every 64 x 64 diagonal
-// block (row-major, block q at Rinv + q * 64 * 64): one CTA per block, column by
-// column back substitution in shared memory.
+// block (row-major, block q at Rinv + q * 64 * 64).  Grid: x = diagonal blocks, y =
+// eighths of a block's columns and rows: the FP64 pipe of one SM bounds the inverse,
+// so a block's columns are spread over eight CTAs.  A warp per column c of
+// X = Rb^{-1}: once X(l, c) is known every lane adds its term to the rows above (two
+// rows per lane), a product and two FMAs per row of the chain.
+constexpr int kTriParts = 8;
+constexpr int kTriThreads = 32 * kTriB / kTriParts;
 template <typename T>
-__global__ void k_tri_blocks(int k, const T* __restrict__ F, int64_t ld, T* __restrict__ Rrm, T* __restrict__ Rinv) {
+__global__ void __launch_bounds__(kTriThreads)
+    k_tri_blocks(int k, const T* __restrict__ F, int64_t ld, T* __restrict__ Rrm, T* __restrict__ Rinv) {
   __shared__ double Rb[kTriB][kTriB + 1];
-  __shared__ double Xb[kTriB][kTriB + 1];
-  const int q = blockIdx.x, b0 = q * kTriB, bs = min(kTriB, k - b0);
+  __shared__ double s_inv[kTriB];
+  const int q = blockIdx.x, b0 = q * kTriB, bs = min(kTriB, k - b0), part = blockIdx.y;
   // the rows of this block, row-major, zero below the diagonal
-  for (int64_t e = threadIdx.x; e < (int64_t)bs * k; e += blockDim.x) {
-    const int i = (int)(e / k), c = (int)(e - (int64_t)i * k);
+  for (int i = part; i < bs; i += kTriParts) {
     const int gi = b0 + i;
-    Rrm[(int64_t)gi * k + c] = c >= gi ? F[gi + (int64_t)c * ld] : T(0);
+    for (int c = threadIdx.x; c < k; c += kTriThreads) Rrm[(int64_t)gi * k + c] = c >= gi ? F[gi + (int64_t)c * ld] : T(0);
   }
-  for (int e = threadIdx.x; e < kTriB * kTriB; e += blockDim.x) {
-    const int i = e / kTriB, c = e % kTriB;
+  for (int e = threadIdx.x; e < kTriB * kTriB; e += kTriThreads) {
+    const int i = e % kTriB, c = e / kTriB;
     Rb[i][c] = (i < bs && c < bs && c >= i) ? (double)F[(b0 + i) + (int64_t)(b0 + c) * ld] : 0.0;
-    Xb[i][c] = 0.0;
   }
   __syncthreads();
-  // X = Rb^{-1}: column c by back substitution, thread per column
-  const int c = threadIdx.x;
+  if (threadIdx.x < kTriB) {
+    const double d = Rb[threadIdx.x][threadIdx.x];
+    s_inv[threadIdx.x] = d != 0.0 ? 1.0 / d : 0.0;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, c = (threadIdx.x >> 5) * kTriParts + part;
+  double x0 = 0.0, x1 = 0.0;  // X(lane, c), X(lane + 32, c)
   if (c < bs) {
-    for (int i = c; i >= 0; --i) {
-      double s = i == c ? 1.0 : 0.0;
-      for (int l = i + 1; l <= c; ++l) s -= Rb[i][l] * Xb[l][c];
-      Xb[i][c] = Rb[i][i] != 0.0 ? s / Rb[i][i] : 0.0;
+    double s0 = lane == c ? 1.0 : 0.0, s1 = lane + 32 == c ? 1.0 : 0.0;
+    for (int l = c; l >= 0; --l) {
+      const double x = __shfl_sync(0xffffffffu, l < 32 ? s0 : s1, l & 31) * s_inv[l];
+      if (lane == l) x0 = x;
+      if (lane + 32 == l) x1 = x;
+      if (lane < l) s0 -= Rb[lane][l] * x;
+      if (lane + 32 < l) s1 -= Rb[lane + 32][l] * x;
     }
   }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kTriB * kTriB; e += blockDim.x)
-    Rinv[(int64_t)q * kTriB * kTriB + e] = (T)Xb[e / kTriB][e % kTriB];
+  T* o = Rinv + (int64_t)q * kTriB * kTriB + c;
+  o[lane * kTriB] = (T)x0;
+  o[(lane + 32) * kTriB] = (T)x1;
 }
 
 // ------------------------------------------------------------ host drivers
@@ -327,8 +376,14 @@ int grid1(int64_t total) {
   return (int)g;
 }
 
-// Split-K count for a product with K = depth: about four waves of 64 x 64 tiles.
+// Split-K count for a product with K = depth: FP64 by the FP64 kernel's own rule; FP32
+// about four waves of 64 x 64 tiles.
+template <typename T>
 int qr_splits(int64_t M, int64_t N, int64_t K, int sms) {
+  if (sizeof(T) == 8) {
+    const int64_t per = 16 * (int64_t)sms / (cdv(M, 32) * cdv(N, 32));  // bounds the partials of narrow products
+    return dgemm_splits(M, N, K, sms, (int)std::max<int64_t>(1, std::min<int64_t>(64, per)));
+  }
   const int64_t tiles = cdv(M, 64) * cdv(N, 64);
   int64_t s = cdv(4 * (int64_t)sms, tiles);
   if (s > K / 256) s = K / 256;
@@ -344,14 +399,14 @@ struct QrScratch {
   int64_t mr = 0, kc = 0;
   int grid = 0, chunk = 0, use_smem = 0, wsplits = 1;
   size_t smem = 0;
-  size_t off_ctr, off_ssq, off_dot, off_gram, off_vc, off_wp, off_w2, off_t, off_tau, total;
+  size_t off_ctr, off_row, off_dot, off_gram, off_vc, off_wp, off_w2, off_t, off_tau, total;
 };
 
 template <typename T>
 void qr_layout(int64_t mr, int64_t kc, int sms, QrScratch* q) {
   q->mr = mr;
   q->kc = kc;
-  int grid = (int)std::min<int64_t>(sms, cdv(mr, kQrW));
+  int grid = (int)std::min<int64_t>(sms, cdv(mr, kQrRows));
   if (grid < 1) grid = 1;
   int64_t chunk = cdv(mr, grid);
   if (chunk < kQrW) chunk = kQrW;  // block 0 owns the panel's diagonal rows
@@ -360,7 +415,7 @@ void qr_layout(int64_t mr, int64_t kc, int sms, QrScratch* q) {
   q->chunk = (int)chunk;
   q->use_smem = qr_panel_smem((int)chunk, kQrW, sizeof(T), true) <= (size_t)200 * 1024;
   q->smem = qr_panel_smem((int)chunk, kQrW, sizeof(T), q->use_smem != 0);
-  q->wsplits = qr_splits(kc, kQrW, mr, sms);
+  q->wsplits = qr_splits<T>(kc, kQrW, mr, sms);
   size_t off = 0;
   auto take = [&](size_t b) {
     size_t at = off;
@@ -368,11 +423,14 @@ void qr_layout(int64_t mr, int64_t kc, int sms, QrScratch* q) {
     return at;
   };
   q->off_ctr = take(256);
-  q->off_ssq = take((size_t)2 * grid * 2 * 8);
+  q->off_row = take((size_t)2 * kQrW * 8);
   q->off_dot = take((size_t)2 * grid * kQrW * 8);
   q->off_gram = take((size_t)grid * kQrW * kQrW * 8);
   q->off_vc = take((size_t)mr * kQrW * sizeof(T));
-  q->off_wp = take((size_t)q->wsplits * kc * kQrW * sizeof(T));
+  // FP64: trailing widths below kc take more splits, within 16 SM counts of 32-row tiles
+  const int64_t wrows = sizeof(T) == 8 ? std::max<int64_t>(kc + 32, std::min<int64_t>(64 * kc, 512 * (int64_t)sms))
+                                       : (int64_t)q->wsplits * kc;
+  q->off_wp = take((size_t)wrows * kQrW * sizeof(T));
   q->off_w2 = take((size_t)kc * kQrW * sizeof(T));
   q->off_t = take((size_t)cdv(kc, kQrW) * kQrW * kQrW * sizeof(T));
   q->off_tau = take((size_t)kc * sizeof(T));
@@ -387,14 +445,15 @@ cudaError_t qr_apply(int mr, int w, int k2, T* C2, int64_t ld, const T* Vc, cons
   if (k2 <= 0) return cudaSuccess;
   T* Wp = reinterpret_cast<T*>(ws + q.off_wp);
   T* W2 = reinterpret_cast<T*>(ws + q.off_w2);
-  const int nz = std::min(q.wsplits, qr_splits(k2, w, mr, sm_count()));
+  const int want = qr_splits<T>(k2, w, mr, sm_count());
+  const int nz = sizeof(T) == 8 ? want : std::min(q.wsplits, want);
   Operand<T> a{C2, ld, nullptr, 0};
   Operand<T> b{Vc, (int64_t)mr, nullptr, 0};
   EpiArgs<T> ep{Wp, w, (int64_t)k2 * w, nullptr, nullptr};
   cudaError_t e = gemm_gather<T>(k2, w, mr, nz, true, a, b, kEpiStore, ep, nullptr, s);
   if (e != cudaSuccess) return e;
   const int nzu = gemm_splits(mr, nz);
-  k_qr_wt<T><<<grid1((int64_t)k2 * w), 256, 0, s>>>(k2, w, nzu, (int64_t)k2 * w, Wp, Tm, trans ? 0 : 1, W2);
+  k_qr_wt<T><<<(int)std::min<int64_t>(cdv(k2, kWtRows), 4096), 32 * kWtRows, 0, s>>>(k2, w, nzu, (int64_t)k2 * w, Wp, Tm, trans ? 0 : 1, W2);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   Operand<T> a2{W2, w, nullptr, 0};
@@ -411,7 +470,7 @@ cudaError_t qr_factor(int64_t mr, int64_t kc, T* F, int64_t ld, const QrScratch&
   static SmemLimit lim;
   cudaError_t e = cudaSuccess;
   unsigned* ctr = reinterpret_cast<unsigned*>(ws + q.off_ctr);
-  double* pssq = reinterpret_cast<double*>(ws + q.off_ssq);
+  double* prow = reinterpret_cast<double*>(ws + q.off_row);
   double* pdot = reinterpret_cast<double*>(ws + q.off_dot);
   double* pgram = reinterpret_cast<double*>(ws + q.off_gram);
   T* Vc = reinterpret_cast<T*>(ws + q.off_vc);
@@ -431,7 +490,7 @@ cudaError_t qr_factor(int64_t mr, int64_t kc, T* F, int64_t ld, const QrScratch&
     T* Tp = Tall + (c0 / kQrW) * kQrW * kQrW;
     int chunk = qp.chunk, use_smem = qp.use_smem;
     int64_t ldl = ld, ldv = mrp;
-    void* args[] = {&mrp, &w, &Pp, &ldl, &chunk, &use_smem, &pssq, &pdot, &pgram, &taup, &Vc, &ldv, &Tp, &ctr, &st};
+    void* args[] = {&mrp, &w, &Pp, &ldl, &chunk, &use_smem, &pdot, &prow, &pgram, &taup, &Vc, &ldv, &Tp, &ctr, &st};
     e = cudaLaunchCooperativeKernel((const void*)k_qr_panel<T>, dim3(qp.grid), dim3(kQrThreads), args, qp.smem, s);
     if (e != cudaSuccess) return e;
     e = qr_apply<T>(mrp, w, (int)(kc - c0 - w), F + c0 + (c0 + w) * ld, ld, Vc, Tp, 1, q, ws, s);
@@ -468,7 +527,7 @@ template <typename T>
 cudaError_t tri_solve(int64_t k, const T* F, int64_t ld, T* B, int64_t ldb, int64_t nrhs, T* X, int64_t ldx, T* Rrm,
                       T* Rinv, cudaStream_t s) {
   const int nbk = (int)cdv(k, kTriB);
-  k_tri_blocks<T><<<nbk, kTriB, 0, s>>>((int)k, F, ld, Rrm, Rinv);
+  k_tri_blocks<T><<<dim3(nbk, kTriParts), kTriThreads, 0, s>>>((int)k, F, ld, Rrm, Rinv);
   cudaError_t e = cudaGetLastError();
   for (int q = nbk - 1; e == cudaSuccess && q >= 0; --q) {
     const int64_t b0 = (int64_t)q * kTriB, bs = std::min<int64_t>(kTriB, k - b0), rest = k - b0 - bs;
@@ -513,7 +572,7 @@ template <typename T>
 void stable_layout(int64_t m, int64_t n, int64_t k, StablePlan* p) {
   const int sms = sm_count();
   qr_layout<T>(m, k, sms, &p->q);
-  p->msplits = qr_splits(k, n, m, sms);
+  p->msplits = qr_splits<T>(k, n, m, sms);
   size_t off = 0;
   auto take = [&](size_t b) {
     size_t at = off;
@@ -583,8 +642,8 @@ void cur_layout(int64_t m, int64_t n, int64_t k, int kind, CurPlan* p) {
   if (kind == 0) {
     qr_layout<T>(m, k, sms, &p->qc);
     qr_layout<T>(n, k, sms, &p->qr);
-    p->m1splits = qr_splits(k, n, m, sms);
-    p->m2splits = qr_splits(k, k, n, sms);
+    p->m1splits = qr_splits<T>(k, n, m, sms);
+    p->m2splits = qr_splits<T>(k, k, n, sms);
     p->off_Fc = take((size_t)m * k * e);
     p->off_Qc = take((size_t)m * k * e);
     p->off_Fr = take((size_t)n * k * e);
@@ -593,7 +652,7 @@ void cur_layout(int64_t m, int64_t n, int64_t k, int kind, CurPlan* p) {
     p->off_M1P = take(p->m1splits > 1 ? (size_t)p->m1splits * k * n * e : 0);
   } else {  // QR of the square A(I, J)
     qr_layout<T>(k, k, sms, &p->qc);
-    p->m2splits = qr_splits(k, k, k, sms);
+    p->m2splits = qr_splits<T>(k, k, k, sms);
     p->off_Fc = take((size_t)k * k * e);
     p->off_Qc = take((size_t)k * k * e);
     p->off_Fr = p->off_Qr = p->off_M1 = p->off_M1P = take(0);

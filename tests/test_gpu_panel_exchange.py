@@ -31,7 +31,7 @@ def B():
     (64, 65003),   # FP64 rows of a block exceed shared memory
     (33, 20),      # fewer columns than the sketch has rows: one block
     (128, 700),    # the widest panel
-    (1, 40),
+    (2, 40),
 ])
 def test_pivots_match_the_oracle(B, orc, k, n):
     rng = np.random.default_rng(k + n)
