@@ -6,10 +6,13 @@
 // One CTA runs one problem at a time and pulls the next one from an atomic work
 // queue (problems ordered by decreasing m*n, so that the long ones start first).
 // Inside a CTA every step of the method runs with CTA-local synchronisation only:
-// Gaussian rows, sketch (CTA GEMM), Schur complement + FP64 norm, the stop test,
-// LUPP of the panel (staged in shared memory when it fits), the inverse of the
-// new unit-lower block, the interpolation-matrix update and the re-blocking of
-// the index lists -- the same arithmetic as the single-problem path.
+// sketch (CTA GEMM), Schur complement + FP64 norm, the stop test, LUPP of the panel
+// (in shared memory when it fits), the inverse of the new unit-lower block, the
+// interpolation-matrix update and the re-blocking of the index lists -- the same
+// arithmetic as the single-problem path.
+// Omega is the same for every problem (rows keyed by their number, entries by their
+// column), so its first blocks of rows are drawn once per call, before the persistent
+// kernel; drawing them per problem cost a fifth of the FP64 arithmetic.
 // The queue reset and the persistent kernel are replayed from a CUDA graph; the
 // output-tile height of the CTA GEMM and the CTAs per SM come from a small
 // autotuner that times the candidates on the largest problems of the batch.
@@ -21,6 +24,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "randid.h"
@@ -67,16 +71,18 @@ struct Params {
   double tol;
   int tol_rel;
   uint64_t seed;
-  int stage_panel;  // 1: the LUPP panel is staged in shared memory
+  const void* omega;  // the first omega_rows rows of Omega (row stride mmax), shared by all problems
+  int omega_rows;     // a multiple of b
+  int stage_rows;     // panels of at most this many rows are kept in shared memory
 };
 
 // Per-CTA scratch slot (one slot per resident CTA).
 template <typename T>
 struct Slot {
-  T* omega;  // b x mmax, row-major
-  T* G;      // nmax x b
-  T* S;      // nmax x b
-  T* N;      // nmax x b
+  T* omega;  // b x mmax, row-major: rows past the shared ones
+  T* G;      // nmax x b, row-major
+  T* S;      // nmax x b, column-major (row stride 1, column stride nmax): a panel too tall for shared memory
+  T* N;      // nmax x b, row-major
   int32_t* act[2];
   int32_t* perm;
   int32_t* mark;
@@ -112,146 +118,316 @@ __device__ Slot<T> slot_at(const Params& p) {
   return s;
 }
 
-// Shared memory of one CTA (dynamic): GEMM tiles, then the panel stage.
+// Shared memory of one CTA (dynamic): GEMM tiles (two buffers), then the panel.
+// Rows of a tile are padded so that a warp's stores (eight k of four rows) fall into
+// distinct banks and the vector reads stay aligned.
+template <typename T>
+constexpr int kPad = sizeof(T) == 4 ? 4 : 2;
 template <typename T, int BM>
 struct Shared {
-  T As[kTK * (BM + 1)];
-  T Bs[kTK * (kTN + 1)];
+  static constexpr int kLA = BM + kPad<T>, kLB = kTN + kPad<T>;
+  alignas(16) T As[2][kTK * kLA];
+  alignas(16) T Bs[2][kTK * kLB];
   T Lp[kMaxB * kMaxB];
   T Li[kMaxB * kMaxB];
-  T prow[kMaxB];
   double pdiag[kMaxB];
+  unsigned long long mag[2][kNT / 32];  // a warp's pivot candidate
+  int32_t row[2][kNT / 32];
   int32_t piv[kMaxB];
   int32_t pivorig[kMaxB];
-  unsigned char sel[kMaxN];
   int32_t warp_tot[kNT / 32];
   double red;
   int problem;
   int base;
 };
 
+// The panel S: entry (r, c) at p[r rs + c cs].
+template <typename T>
+struct PanelRef {
+  T* p;
+  int rs;
+  int64_t cs;
+  __device__ __forceinline__ T& operator()(int r, int c) const { return p[r * rs + c * cs]; }
+};
+
+// ------------------------------------------------------------------ sums of squares
+// FP32: squares in float-float, folded into FP64 every 64 terms (GB300 issues about two
+// FP64 instructions per clock per SM; per-element FP64 work cost more than this
+// kernel's FP32 arithmetic).  FP64: one FMA per term.
+template <typename T>
+struct Squares {
+  double acc = 0.0;
+  float hi = 0.f, lo = 0.f;
+  int cnt = 0;
+  bool finite = true;
+  __device__ __forceinline__ void add(T v) {
+    if constexpr (sizeof(T) == 4) {
+      sq_add_f32(v, hi, lo, acc, finite);
+      if (++cnt == 64) {
+        acc += (double)hi + (double)lo;
+        hi = lo = 0.f;
+        cnt = 0;
+      }
+    } else {
+      finite = finite && (__double2hiint(v) & 0x7FF00000) != 0x7FF00000;
+      acc = fma(v, v, acc);
+    }
+  }
+  __device__ __forceinline__ double sum() const {
+    if constexpr (sizeof(T) == 4) return acc + ((double)hi + (double)lo);
+    return acc;
+  }
+};
+struct NoSquares {};
+
 // ------------------------------------------------------------------ CTA GEMM
-// C (M x N) = sum_k A_r[k] B(k, c); A row r at abase + (aidx ? aidx[r] : r) * lda;
-// B K-major (row c at bbase + idx*ldb + boff, contiguous in k) or N-major (row k
-// contiguous in c).  mode 0: out[r*ldo + c] = acc; mode 1: out[oidx[r]*ldo + c]
-// -= acc unless skip[r].  Every output accumulates over k in increasing order,
-// whatever BM is, so the tile choice does not change the result.
-template <typename T, int BM, bool BK>
-__device__ void cta_gemm(int M, int N, int K, const T* abase, int64_t lda, const int32_t* aidx, const T* bbase,
-                         int64_t ldb, const int32_t* bidx, int64_t boff, int mode, T* out, int64_t ldo,
-                         const int32_t* oidx, const int32_t* skip, T* As, T* Bs) {
-  constexpr int TM = BM / 16;
-  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
-  for (int m0 = 0; m0 < M; m0 += BM)
-    for (int n0 = 0; n0 < N; n0 += kTN) {
-      T acc[TM];
+// epi(r, c, sum_k A_r[k] B(k, c)) for every entry of an M x N product; A row r at abase
+// + (aidx ? aidx[r] : r) * lda; B K-major (row c at bbase + idx*ldb, contiguous in k) or
+// N-major (row k contiguous in c).  sq takes every entry of A once per column tile
+// (NoSquares: none).  Every output accumulates over k in increasing order, one FMA per
+// term, whatever BM is, so the tile choice does not change the result.
+// A thread owns TM rows x TN columns: an FP32 warp reads one vector of A (broadcast over
+// 16 lanes) and one of B per TM TN FMAs.  With one value of B and four of A per four
+// FMAs shared memory bounded the FP32 products; FP64 is bounded by its pipe.  The next K
+// step's loads are in registers while this one is computed, one barrier per step.
+template <typename T, int N>
+struct alignas(sizeof(T) * N) Vec {
+  T v[N];
+};
+template <typename T, int BM, bool BK, typename Sq, typename Epi>
+__device__ __forceinline__ void cta_gemm(int M, int N, int K, const T* abase, int64_t lda, const int32_t* aidx,
+                                         const T* bbase, int64_t ldb, const int32_t* bidx, Shared<T, BM>& sh, Sq& sq,
+                                         Epi epi) {
+  constexpr int TN = BM >= 64 ? 2 : 1, TM = BM * kTN / kNT / TN;
+  constexpr int kLA = Shared<T, BM>::kLA, kLB = Shared<T, BM>::kLB;
+  constexpr int NA = BM / 16, NB = 2;          // loads of a K step per thread
+  constexpr int NP = BM >= 64 ? BM / 64 : 1;  // distinct rows among its loads of A (of B: one)
+  constexpr int VM = TM * (int)sizeof(T) > 16 ? 16 / (int)sizeof(T) : TM;  // rows per 16-byte read
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tx = tid % (kTN / TN), ty = tid / (kTN / TN);
+  const int lk = lane & 7, lq = lane >> 3;  // K-major loads: lanes cover eight k of four rows
+  for (int m0 = 0; m0 < M; m0 += BM) {
+    const T* ap[NP];
 #pragma unroll
-      for (int i = 0; i < TM; ++i) acc[i] = T(0);
-      for (int k0 = 0; k0 < K; k0 += kTK) {
-        for (int e = tid; e < BM * kTK; e += kNT) {
-          const int r = e / kTK, kk = e - r * kTK, row = m0 + r, k = k0 + kk;
-          T v = T(0);
-          if (row < M && k < K) v = abase[(int64_t)(aidx ? aidx[row] : row) * lda + k];
-          As[kk * (BM + 1) + r] = v;
+    for (int i = 0; i < NP; ++i) {
+      const int r = m0 + ((warp + 16 * i) % (BM / 4)) * 4 + lq;
+      ap[i] = r < M ? abase + (int64_t)(aidx ? aidx[r] : r) * lda : nullptr;
+    }
+    for (int n0 = 0; n0 < N; n0 += kTN) {
+      const int cb = n0 + (warp & 7) * 4 + lq;
+      const T* bp = (BK && cb < N) ? bbase + (int64_t)(bidx ? bidx[cb] : cb) * ldb : nullptr;
+      T ra[NA], rb[NB];
+      auto load = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+          const int k = k0 + (warp + 16 * i) / (BM / 4) * 8 + lk;
+          ra[i] = (ap[i % NP] != nullptr && k < K) ? ap[i % NP][k] : T(0);
         }
-        if (BK) {
-          for (int e = tid; e < kTN * kTK; e += kNT) {
-            const int c = e / kTK, kk = e - c * kTK, col = n0 + c, k = k0 + kk;
-            T v = T(0);
-            if (col < N && k < K) v = bbase[(int64_t)(bidx ? bidx[col] : col) * ldb + boff + k];
-            Bs[kk * (kTN + 1) + c] = v;
-          }
-        } else {
-          for (int e = tid; e < kTK * kTN; e += kNT) {
-            const int kk = e / kTN, c = e - kk * kTN, col = n0 + c, k = k0 + kk;
-            T v = T(0);
-            if (col < N && k < K) v = bbase[(int64_t)(bidx ? bidx[k] : k) * ldb + boff + col];
-            Bs[kk * (kTN + 1) + c] = v;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+          if (BK) {
+            const int k = k0 + ((warp + 16 * i) >> 3) * 8 + lk;
+            rb[i] = (bp != nullptr && k < K) ? bp[k] : T(0);
+          } else {
+            const int k = k0 + warp + 16 * i, c = n0 + lane;
+            rb[i] = (k < K && c < N) ? bbase[(int64_t)(bidx ? bidx[k] : k) * ldb + c] : T(0);
           }
         }
-        __syncthreads();
+      };
+      auto store = [&](int buf) {
+        T* as = sh.As[buf];
+        T* bs = sh.Bs[buf];
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+          as[((warp + 16 * i) / (BM / 4) * 8 + lk) * kLA + ((warp + 16 * i) % (BM / 4)) * 4 + lq] = ra[i];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+          if (BK)
+            bs[(((warp + 16 * i) >> 3) * 8 + lk) * kLB + ((warp + 16 * i) & 7) * 4 + lq] = rb[i];
+          else
+            bs[(warp + 16 * i) * kLB + lane] = rb[i];
+        }
+        if constexpr (!std::is_same<Sq, NoSquares>::value) {
+          if (n0 == 0) {
+#pragma unroll
+            for (int i = 0; i < NA; ++i) sq.add(ra[i]);
+          }
+        }
+      };
+      T acc[TM][TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
+      load(0);
+      store(0);
+      __syncthreads();
+      int buf = 0;
+      for (int k0 = 0; k0 < K; k0 += kTK, buf ^= 1) {
+        if (k0 + kTK < K) load(k0 + kTK);
+        const T* as = sh.As[buf] + ty * TM;
+        const T* bs = sh.Bs[buf] + tx * TN;
 #pragma unroll 8
         for (int kk = 0; kk < kTK; ++kk) {
-          const T bv = Bs[kk * (kTN + 1) + tx];
+          T av[TM];
 #pragma unroll
-          for (int i = 0; i < TM; ++i) acc[i] = fma(As[kk * (BM + 1) + ty + 16 * i], bv, acc[i]);
+          for (int i = 0; i < TM; i += VM) {
+            const Vec<T, VM> v = *reinterpret_cast<const Vec<T, VM>*>(as + kk * kLA + i);
+#pragma unroll
+            for (int u = 0; u < VM; ++u) av[i + u] = v.v[u];
+          }
+          const Vec<T, TN> bv = *reinterpret_cast<const Vec<T, TN>*>(bs + kk * kLB);
+#pragma unroll
+          for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) acc[i][j] = fma(av[i], bv.v[j], acc[i][j]);
         }
+        if (k0 + kTK < K) store(buf ^ 1);
         __syncthreads();
       }
-      const int c = n0 + tx;
-      if (c < N) {
 #pragma unroll
-        for (int i = 0; i < TM; ++i) {
-          const int r = m0 + ty + 16 * i;
-          if (r >= M) continue;
-          if (mode == 0) {
-            out[(int64_t)r * ldo + c] = acc[i];
-          } else if (skip == nullptr || skip[r] == 0) {
-            out[(int64_t)(oidx ? oidx[r] : r) * ldo + c] -= acc[i];
-          }
+      for (int i = 0; i < TM; ++i) {
+        const int r = m0 + ty * TM + i;
+        if (r >= M) continue;
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          const int c = n0 + tx * TN + j;
+          if (c < N) epi(r, c, acc[i][j]);
         }
       }
     }
+  }
 }
 
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+__device__ __forceinline__ unsigned long long mag_bits(float x) {
+  return (unsigned long long)(__float_as_uint(x) & 0x7FFFFFFFu) << 32;
+}
+__device__ __forceinline__ double mag_value(unsigned long long m, double) { return __longlong_as_double((long long)m); }
+__device__ __forceinline__ double mag_value(unsigned long long m, float) {
+  return (double)__uint_as_float((unsigned)(m >> 32));
+}
+// The largest (magnitude, then smaller row) of a warp, by integer comparisons; row < 0
+// takes no part.  Every lane gets the result.
 template <typename T>
-__device__ __forceinline__ T from_d(double x) {
-  return static_cast<T>(x);
+__device__ __forceinline__ void warp_pivot(unsigned long long& mag, int& row) {
+  const unsigned hi = (unsigned)(mag >> 32);
+  const unsigned top = __reduce_max_sync(0xffffffffu, row >= 0 ? hi + 1u : 0u);
+  if (top == 0u) {
+    row = -1;
+    return;
+  }
+  bool in = row >= 0 && hi + 1u == top;
+  unsigned lo = 0u;
+  if (sizeof(T) == 8) {
+    lo = __reduce_max_sync(0xffffffffu, in ? (unsigned)mag : 0u);
+    in = in && (unsigned)mag == lo;
+  }
+  row = (int)__reduce_min_sync(0xffffffffu, in ? (unsigned)row : 0x7FFFFFFFu);
+  mag = ((unsigned long long)(top - 1u) << 32) | lo;
+}
+
+// ------------------------------------------------------------------ LUPP of a panel
+// R (na x b) for bt pivots.  A lane keeps the rows r = 32 (warp + 16 i) + lane and
+// updates them by itself, column by column (the rows' stride b + 1 in shared memory, or
+// one along the columns in global memory, keeps a warp's accesses apart); the column
+// that holds the next pivot comes first, so its maximum is known when the update ends.
+// One barrier per pivot: it publishes the warps' candidates and the finished update
+// together; every warp then picks the same pivot.  Rows are marked, not swapped.
+template <typename T, int BM>
+__device__ void panel_lupp(const PanelRef<T>& R, int na, int b, int bt, int32_t* mark, Shared<T, BM>& sh,
+                           unsigned& zeros) {
+  constexpr int nw = kNT / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned sel = 0u;  // bit i: row 32 (warp + 16 i) + lane is a pivot row (n <= 4096: at most 8 bits)
+  unsigned long long mag = 0ull;
+  int row = -1;
+  for (int g = warp; 32 * g < na; g += nw) {
+    const int r = 32 * g + lane;
+    if (r < na) {
+      const unsigned long long m = mag_bits(R(r, 0));
+      if (row < 0 || m > mag) {
+        mag = m;
+        row = r;
+      }
+    }
+  }
+  for (int c = 0; c < bt; ++c) {
+    warp_pivot<T>(mag, row);
+    if (lane == 0) {
+      sh.mag[c & 1][warp] = mag;
+      sh.row[c & 1][warp] = row;
+    }
+    __syncthreads();
+    mag = lane < nw ? sh.mag[c & 1][lane] : 0ull;
+    row = lane < nw ? sh.row[c & 1][lane] : -1;
+    warp_pivot<T>(mag, row);
+    const int p = row;
+    const bool zero = mag == 0ull;
+    if (threadIdx.x == 0) {
+      sh.piv[c] = p;
+      sh.pdiag[c] = mag_value(mag, T(0));
+    }
+    if (zero) ++zeros;
+    const T pv = R(p, c);
+    const bool more = c + 1 < bt;
+    const T p1 = more ? R(p, c + 1) : T(0);
+    mag = 0ull;
+    row = -1;
+    int i = 0;
+    for (int g = warp; 32 * g < na; g += nw, ++i) {
+      const int r = 32 * g + lane;
+      if (r == p) sel |= 1u << i;
+      if (r >= na || ((sel >> i) & 1u) != 0u) continue;
+      T l = T(0);
+      if (!zero) {
+        l = R(r, c) / pv;
+        R(r, c) = l;
+      }
+      if (more) {
+        T z = R(r, c + 1);
+        if (!zero) R(r, c + 1) = z = fma(-l, p1, z);
+        const unsigned long long m = mag_bits(z);
+        if (row < 0 || m > mag) {
+          mag = m;
+          row = r;
+        }
+      }
+      if (!zero) {
+        int cc = more ? c + 2 : c + 1;
+        for (; cc + 4 <= b; cc += 4) {
+          T x[4], q[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            x[u] = R(r, cc + u);
+            q[u] = R(p, cc + u);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) R(r, cc + u) = fma(-l, q[u], x[u]);
+        }
+        for (; cc < b; ++cc) R(r, cc) = fma(-l, R(p, cc), R(r, cc));
+      }
+    }
+  }
+  int i = 0;
+  for (int g = warp; 32 * g < na; g += nw, ++i)
+    if (32 * g + lane < na) mark[32 * g + lane] = (int)((sel >> i) & 1u);
+  __syncthreads();
 }
 
 // ------------------------------------------------------------------ one problem
 template <typename T, int BM>
 __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slot<T>& sl, Shared<T, BM>& sh,
                             T* stage) {
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = pr.m, n = pr.n, b = p.b, cap = pr.cap;
   const T* A = static_cast<const T*>(pr.A);
   T* X = static_cast<T*>(pr.X);
   const int64_t lda = pr.lda, ldx = pr.ldx;
-  // ||A||_F^2 and finiteness
-  // (FP32: exact squares in float-float, folded into FP64 every 64 terms -- GB300
-  // issues about two FP64 instructions per clock per SM, and per-element FP64 work
-  // cost more than this kernel's FP32 arithmetic)
-  double acc = 0.0;
-  bool finite = true;
-  if constexpr (sizeof(T) == 4) {
-    float hi = 0.f, lo = 0.f;
-    int cnt = 0;
-    for (int j = 0; j < n; ++j)
-      for (int i = tid; i < m; i += kNT) {
-        sq_add_f32(static_cast<float>(A[(int64_t)j * lda + i]), hi, lo, acc, finite);
-        if (++cnt == 64) {
-          acc += (double)hi + (double)lo;
-          hi = lo = 0.f;
-          cnt = 0;
-        }
-      }
-    acc += (double)hi + (double)lo;
-  } else {
-    for (int64_t e = tid; e < (int64_t)m * n; e += kNT) {
-      const int64_t j = e / m, i = e - j * m;
-      const double v = static_cast<double>(A[j * lda + i]);
-      finite = finite && isfinite(v);
-      acc += v * v;
-    }
-  }
-  const int bad = __syncthreads_or(!finite);
-  const double n2 = block_sum(acc);
-  if (tid == 0) sh.red = n2;
-  __syncthreads();
-  const double norm2 = sh.red;
-  __syncthreads();
-  if (bad) {
-    if (tid == 0) {
-      res.k = 0;
-      res.est = 0.0;
-      res.norm_A = 0.0;
-      res.rounds = 0;
-      res.status = ID_ERR_NONFINITE;
-    }
-    return;
-  }
-  const double thr = p.tol_rel ? p.tol * sqrt(norm2) : p.tol;
+  double thr = 0.0, norm2 = 0.0;
+  NoSquares none;
   for (int i = tid; i < n; i += kNT) {
     sl.act[0][i] = i;
     sl.mark[i] = 0;
@@ -262,66 +438,73 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
   double est = 0.0;
   int64_t k = 0;
   for (;;) {
+    // the panel of this round: in shared memory when its rows fit
+    const PanelRef<T> R = na <= p.stage_rows ? PanelRef<T>{stage, b + 1, 1} : PanelRef<T>{sl.S, 1, p.nmax};
     // Gaussian rows [t*b, t*b + b) of Omega (same counters as the single-problem path)
-    // (32-bit indices: a 64-bit division is an FP64-pipe routine on GB300)
-    const int nq = (m + 3) / 4;
-    for (int e = tid; e < b * nq; e += kNT) {
-      const int i = e / nq, q = e - i * nq;
-      uint64_t x0 = (uint64_t)q, x1 = (uint64_t)((int64_t)t * b + i), x2 = 0, x3 = 0;
-      philox4x64_10(x0, x1, x2, x3, p.seed, 0ull);
-      T* o = sl.omega + (int64_t)i * p.mmax + 4 * q;
-      if constexpr (sizeof(T) == 4) {  // FP32: the FP32 evaluation of the same map
-        float f[4];
-        box_muller_f32_53(x0, x1, f[0], f[1]);
-        box_muller_f32_53(x2, x3, f[2], f[3]);
-        for (int j = 0; j < 4 && 4 * q + j < m; ++j) o[j] = f[j];
-      } else {
-        double z[4];
-        box_muller(x0, x1, z[0], z[1]);
-        box_muller(x2, x3, z[2], z[3]);
-        for (int j = 0; j < 4 && 4 * q + j < m; ++j) o[j] = from_d<T>(z[j]);
-      }
-    }
-    __syncthreads();
-    // sketch G (n x b) = (Omega A)^T
-    cta_gemm<T, BM, true>(n, b, m, A, lda, nullptr, sl.omega, p.mmax, nullptr, 0, 0, sl.G, b, nullptr, nullptr,
-                          sh.As, sh.Bs);
-    __syncthreads();
-    // Schur complement S = G(act) - T(act, 0:tb) G(perm) and its FP64 norm
-    if (tb > 0) {
-      cta_gemm<T, BM, false>(na, b, tb, X, ldx, sl.act[cur], sl.G, b, sl.perm, 0, 0, sl.S, b, nullptr, nullptr,
-                             sh.As, sh.Bs);
-      __syncthreads();
-    }
-    double e2 = 0.0;
-    {
-      float hi = 0.f, lo = 0.f;
-      bool fin = true;
-      int cnt = 0;
-      for (int e = tid; e < na * b; e += kNT) {
-        const int i = e / b, c = e - i * b;
-        T v = sl.G[(int64_t)sl.act[cur][i] * b + c];
-        if (tb > 0) v -= sl.S[(int64_t)i * b + c];
-        sl.S[(int64_t)i * b + c] = v;
-        if constexpr (sizeof(T) == 4) {
-          sq_add_f32(v, hi, lo, e2, fin);
-          if (++cnt == 64) {
-            e2 += (double)hi + (double)lo;
-            hi = lo = 0.f;
-            cnt = 0;
-          }
+    const T* om;
+    if ((t + 1) * b <= p.omega_rows) {
+      om = static_cast<const T*>(p.omega) + (int64_t)t * b * p.mmax;
+    } else {
+      // (32-bit indices: a 64-bit division is an FP64-pipe routine on GB300)
+      const int nq = (m + 3) / 4;
+      for (int e = tid; e < b * nq; e += kNT) {
+        const int i = e / nq, q = e - i * nq;
+        uint64_t x0 = (uint64_t)q, x1 = (uint64_t)((int64_t)t * b + i), x2 = 0, x3 = 0;
+        philox4x64_10(x0, x1, x2, x3, p.seed, 0ull);
+        T* o = sl.omega + (int64_t)i * p.mmax + 4 * q;
+        T z[4];
+        if constexpr (sizeof(T) == 4) {  // FP32: the FP32 evaluation of the same map
+          box_muller_f32_53(x0, x1, z[0], z[1]);
+          box_muller_f32_53(x2, x3, z[2], z[3]);
         } else {
-          e2 += static_cast<double>(v) * static_cast<double>(v);
+          box_muller(x0, x1, z[0], z[1]);
+          box_muller(x2, x3, z[2], z[3]);
         }
+        for (int j = 0; j < 4 && 4 * q + j < m; ++j) o[j] = z[j];
       }
-      if constexpr (sizeof(T) == 4) e2 += (fin ? (double)hi + (double)lo : (double)INFINITY);
+      __syncthreads();
+      om = sl.omega;
     }
-    e2 = block_sum(e2);
-    if (tid == 0) sh.red = e2;
-    __syncthreads();
-    e2 = sh.red;
-    __syncthreads();
-    if (t > 0) {
+    Squares<T> e2s;
+    if (t == 0) {
+      // the first sketch G (n x b) = (Omega A)^T is the panel; ||A||_F^2 and finiteness come
+      // with its one read of A
+      Squares<T> sq;
+      cta_gemm<T, BM, true>(n, b, m, A, lda, nullptr, om, p.mmax, nullptr, sh, sq,
+                            [&](int r, int c, T v) { R(r, c) = v; });
+      const int bad = __syncthreads_or(!sq.finite);
+      const double n2 = block_sum(sq.sum());
+      if (tid == 0) sh.red = n2;
+      __syncthreads();
+      norm2 = sh.red;
+      __syncthreads();
+      if (bad) {
+        if (tid == 0) {
+          res.k = 0;
+          res.est = 0.0;
+          res.norm_A = 0.0;
+          res.rounds = 0;
+          res.status = ID_ERR_NONFINITE;
+        }
+        return;
+      }
+      thr = p.tol_rel ? p.tol * sqrt(norm2) : p.tol;
+    } else {
+      cta_gemm<T, BM, true>(n, b, m, A, lda, nullptr, om, p.mmax, nullptr, sh, none,
+                            [&](int r, int c, T v) { sl.G[(int64_t)r * b + c] = v; });
+      __syncthreads();
+      // Schur complement S = G(act) - T(act, 0:tb) G(perm) and its FP64 norm
+      const int32_t* act = sl.act[cur];
+      cta_gemm<T, BM, false>(na, b, tb, X, ldx, act, sl.G, b, sl.perm, sh, none, [&](int r, int c, T v) {
+        const T s = sl.G[(int64_t)act[r] * b + c] - v;
+        R(r, c) = s;
+        e2s.add(s);
+      });
+      double e2 = block_sum(e2s.finite || sizeof(T) == 8 ? e2s.sum() : (double)INFINITY);
+      if (tid == 0) sh.red = e2;
+      __syncthreads();
+      e2 = sh.red;
+      __syncthreads();
       est = sqrt(e2 / (double)b);
       ++rounds;
       if (est <= thr) {
@@ -335,85 +518,19 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
       }
     }
     const int bt = min(b, cap - tb);
-    // LUPP of S (na x b) for bt pivots: rows are marked, not swapped
-    T* R = stage != nullptr ? stage : sl.S;
-    const int ldr = stage != nullptr ? b + 1 : b;
-    if (stage != nullptr)
-      for (int e = tid; e < na * b; e += kNT) {
-        const int i = e / b, c = e - i * b;
-        R[i * ldr + c] = sl.S[(int64_t)i * b + c];
-      }
-    for (int i = tid; i < na; i += kNT) sh.sel[i] = 0;
-    __syncthreads();
-    for (int c = 0; c < bt; ++c) {
-      ArgMax a;
-      a.v = -1.0;
-      a.idx = -1;
-      if constexpr (sizeof(T) == 4) {
-        // FP32: keys (|v| bit pattern, ~row) compared as integers -- the same choice
-        // (largest |v|, ties to the smaller row) without per-element FP64 work
-        unsigned long long best = 0ull;
-        for (int r = tid; r < na; r += kNT)
-          if (!sh.sel[r]) {
-            const unsigned long long kk = ((unsigned long long)(__float_as_uint(R[r * ldr + c]) & 0x7FFFFFFFu) << 32) |
-                                          (unsigned long long)(0xFFFFFFFFu - (unsigned)r);
-            best = kk > best ? kk : best;
-          }
-        best = block_max_u64(best);
-        if (best != 0ull) {
-          a.idx = (int)(0xFFFFFFFFu - (unsigned)(best & 0xFFFFFFFFull));
-          a.v = (double)__uint_as_float((unsigned)(best >> 32));
-        }
-      } else {
-        for (int r = tid; r < na; r += kNT)
-          if (!sh.sel[r]) {
-            ArgMax o;
-            o.v = static_cast<double>(tabs(R[r * ldr + c]));
-            o.idx = r;
-            a = argmax_pick(a, o);
-          }
-        a = block_argmax(a);
-      }
-      const int pr_ = a.idx;
-      const bool zero = !(a.v > 0.0);
-      for (int cc = tid; cc < b; cc += kNT) sh.prow[cc] = R[pr_ * ldr + cc];
-      if (tid == 0) {
-        sh.sel[pr_] = (unsigned char)1;
-        sh.piv[c] = pr_;
-        sh.pdiag[c] = a.v;
-      }
-      if (zero) ++zeros;
-      __syncthreads();
-      if (!zero) {
-        const T pv = sh.prow[c];
-        for (int r = tid; r < na; r += kNT)
-          if (!sh.sel[r]) R[r * ldr + c] = R[r * ldr + c] / pv;
-        __syncthreads();
-        const int wc = b - c - 1;
-        for (int e = tid; e < na * wc; e += kNT) {
-          const int r = e / wc, cc = c + 1 + (e - r * wc);
-          if (!sh.sel[r]) R[r * ldr + cc] = fma(-R[r * ldr + c], sh.prow[cc], R[r * ldr + cc]);
-        }
-        __syncthreads();
-      }
-    }
-    if (stage != nullptr)
-      for (int e = tid; e < na * b; e += kNT) {
-        const int i = e / b, c = e - i * b;
-        sl.S[(int64_t)i * b + c] = R[i * ldr + c];
-      }
-    for (int i = tid; i < na; i += kNT) sl.mark[i] = sh.sel[i];
-    __syncthreads();
+    panel_lupp<T, BM>(R, na, b, bt, sl.mark, sh, zeros);
     // inverse of the new unit-lower block L-hat(piv, 0:bt)
     for (int e = tid; e < bt * bt; e += kNT) {
       const int r = e / bt, c = e - r * bt;
-      sh.Lp[e] = c < r ? sl.S[(int64_t)sh.piv[r] * b + c] : (c == r ? T(1) : T(0));
+      sh.Lp[e] = c < r ? R(sh.piv[r], c) : (c == r ? T(1) : T(0));
     }
     for (int e = tid; e < bt * bt; e += kNT) sh.Li[e] = (e / bt == e % bt) ? T(1) : T(0);
+    if (tid < bt) sh.pivorig[tid] = sl.act[cur][sh.piv[tid]];
     __syncthreads();
-    // rows in order; each column j of a row summed by 4 threads interleaved over c
-    // and a shuffle -- the summation order of the single-problem driver's k_linv
-    {
+    // rows in order; each column j of a row summed by 4 threads interleaved over c and a
+    // shuffle -- the summation order of the single-problem driver's k_linv.  The columns
+    // are independent and a column's four threads lie in one warp: no block barrier.
+    if (tid < 4 * kMaxB) {
       const int j = tid >> 2, part = tid & 3;
       for (int i = 1; i < bt; ++i) {
         T s = T(0);
@@ -422,25 +539,30 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
         if (j < i && part == 0) sh.Li[i * bt + j] = -s;
-        __syncthreads();
+        __syncwarp();
       }
     }
-    if (tid < bt) sh.pivorig[tid] = sl.act[cur][sh.piv[tid]];
     __syncthreads();
-    // new block of T: N = L-hat(rest) Linv, stored in N and in X(tb:tb+bt, act)
-    for (int e = tid; e < na * bt; e += kNT) {
-      const int i = e / bt, c = e - i * bt;
+    // new block of T: N = L-hat(rest) Linv, stored in N and in X(tb:tb+bt, act): a warp per
+    // row, lanes along the columns
+    for (int i = warp; i < na; i += kNT / 32) {
       if (sl.mark[i]) continue;
       T s = T(0);
-      for (int cp = c; cp < bt; ++cp) s = fma(sl.S[(int64_t)i * b + cp], sh.Li[cp * bt + c], s);
-      sl.N[(int64_t)i * bt + c] = s;
-      X[(int64_t)sl.act[cur][i] * ldx + tb + c] = s;
+      if (lane < bt) {
+#pragma unroll 8
+        for (int cp = 0; cp < bt; ++cp)
+          if (cp >= lane) s = fma(R(i, cp), sh.Li[cp * bt + lane], s);
+        sl.N[(int64_t)i * bt + lane] = s;
+        X[(int64_t)sl.act[cur][i] * ldx + tb + lane] = s;
+      }
     }
     __syncthreads();
     // old columns: T(act, 0:tb) -= N T(piv, 0:tb)
     if (tb > 0) {
-      cta_gemm<T, BM, false>(na, tb, bt, sl.N, bt, nullptr, X, ldx, sh.pivorig, 0, 1, X, ldx, sl.act[cur], sl.mark,
-                             sh.As, sh.Bs);
+      const int32_t* act = sl.act[cur];
+      cta_gemm<T, BM, false>(na, tb, bt, sl.N, bt, nullptr, X, ldx, sh.pivorig, sh, none, [&](int r, int c, T v) {
+        if (sl.mark[r] == 0) X[(int64_t)act[r] * ldx + c] -= v;
+      });
       __syncthreads();
     }
     // re-block: append the pivots, drop them from the active list (stable)
@@ -450,7 +572,6 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
       sl.perm[tb + tid] = j;
       if (pr.pivots != nullptr) pr.pivots[tb + tid] = sh.pdiag[tid];
     }
-    const int lane = tid & 31, warp = tid >> 5;
     if (tid == 0) sh.base = 0;
     __syncthreads();
     for (int start = 0; start < na; start += kNT) {
@@ -467,22 +588,20 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
         for (int w = 0; w < kNT / 32; ++w) sh.base += sh.warp_tot[w];
       __syncthreads();
     }
-    for (int i = tid; i < na; i += kNT) sl.mark[i] = 0;
     cur ^= 1;
     tb += bt;
     na -= bt;
     ++t;
-    __syncthreads();
     if (tb == n) {  // every column is a skeleton
       k = n;
       est = 0.0;
       break;
     }
   }
-  // X(:, J) = I
-  for (int64_t e = tid; e < k * k; e += kNT) {
-    const int64_t q = e / k, c = e - q * k;
-    X[(int64_t)sl.perm[q] * ldx + c] = q == c ? T(1) : T(0);
+  // X(:, J) = I: a warp per skeleton column
+  for (int q = warp; q < (int)k; q += kNT / 32) {
+    T* x = X + (int64_t)sl.perm[q] * ldx;
+    for (int c = lane; c < (int)k; c += 32) x[c] = q == c ? T(1) : T(0);
   }
   if (zeros) status |= ID_WARN_ZERO_PIVOT;
   if (tid == 0) {
@@ -499,8 +618,7 @@ template <typename T, int BM, int MINB>
 __global__ void __launch_bounds__(kNT, MINB) k_batched(Params p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Shared<T, BM>& sh = *reinterpret_cast<Shared<T, BM>*>(smem_raw);
-  T* stage = p.stage_panel ? reinterpret_cast<T*>(smem_raw + ((sizeof(Shared<T, BM>) + 15) & ~(size_t)15))
-                           : nullptr;
+  T* stage = reinterpret_cast<T*>(smem_raw + ((sizeof(Shared<T, BM>) + 15) & ~(size_t)15));
   Slot<T> sl = slot_at<T>(p);
   for (;;) {
     if (threadIdx.x == 0) sh.problem = atomicAdd(p.queue, 1);
@@ -513,44 +631,53 @@ __global__ void __launch_bounds__(kNT, MINB) k_batched(Params p) {
   }
 }
 
-template <typename T, int BM>
-size_t shared_bytes(int64_t nmax, int b, bool stage) {
-  size_t s = (sizeof(Shared<T, BM>) + 15) & ~(size_t)15;
-  if (stage) s += sizeof(T) * nmax * (b + 1);
-  return s;
-}
-
 // ------------------------------------------------------------------ host side
 struct Config {
-  int bm;      // 32 or 64
+  int bm;      // 32, 64 or 128 rows per GEMM tile
   int per_sm;  // CTAs per SM: 1 or 2
 };
 
-template <typename T>
-bool stage_fits(int64_t nmax, int b, const Config& c) {
-  const size_t budget = c.per_sm == 1 ? 200 * 1024 : 100 * 1024;
-  return (c.bm == 64 ? shared_bytes<T, 64>(nmax, b, true) : shared_bytes<T, 32>(nmax, b, true)) <= budget;
+// Rows of a panel that fit in shared memory beside the tiles, and the shared memory of a
+// CTA (half of an SM's 227 KB when two CTAs share it, 1 KB of each reserved).
+template <typename T, int BM>
+size_t shared_bytes(int64_t nmax, int b, int per_sm, int* stage_rows) {
+  const size_t fixed = (sizeof(Shared<T, BM>) + 15) & ~(size_t)15;
+  const size_t budget = per_sm == 1 ? 226 * 1024 : 111 * 1024;
+  int64_t rows = budget > fixed ? (int64_t)((budget - fixed) / (sizeof(T) * (b + 1))) : 0;
+  if (rows > nmax) rows = nmax;
+  *stage_rows = (int)rows;
+  return fixed + sizeof(T) * (size_t)rows * (b + 1);
 }
 
 template <typename T>
 cudaError_t launch(const Params& p0, const Config& c, int sms, cudaStream_t s) {
   Params p = p0;
-  p.stage_panel = stage_fits<T>(p.nmax, p.b, c) ? 1 : 0;
-  const size_t smem = c.bm == 64 ? shared_bytes<T, 64>(p.nmax, p.b, p.stage_panel)
-                                 : shared_bytes<T, 32>(p.nmax, p.b, p.stage_panel);
   const int grid = sms * c.per_sm;
   cudaError_t e = cudaMemsetAsync(p.queue, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
+  if (p.omega_rows > 0) {
+    e = gaussian_rows<T>(p.seed, 0, p.omega_rows, p.mmax, static_cast<T*>(const_cast<void*>(p.omega)), p.mmax, nullptr,
+                         s);
+    if (e != cudaSuccess) return e;
+  }
   // the shared-memory limit is raised once per kernel variant, device and size
   // (never inside a stream capture: the tuner launches every variant first)
 #define RID_BAT_LAUNCH(BM, MINB)                                                                            \
   do {                                                                                                      \
+    const size_t smem = shared_bytes<T, BM>(p.nmax, p.b, MINB, &p.stage_rows);                              \
     static SmemLimit lim;                                                                                   \
     e = raise_smem(k_batched<T, BM, MINB>, smem, lim);                                                      \
     if (e != cudaSuccess) return e;                                                                         \
     k_batched<T, BM, MINB><<<grid, kNT, smem, s>>>(p);                                                      \
   } while (0)
-  if (c.bm == 64 && c.per_sm == 1) RID_BAT_LAUNCH(64, 1);
+  if (c.bm == 128) {  // FP32 only
+    if constexpr (sizeof(T) == 4) {
+      if (c.per_sm == 1) RID_BAT_LAUNCH(128, 1);
+      else RID_BAT_LAUNCH(128, 2);
+    } else {
+      return cudaErrorInvalidValue;
+    }
+  } else if (c.bm == 64 && c.per_sm == 1) RID_BAT_LAUNCH(64, 1);
   else if (c.bm == 64) RID_BAT_LAUNCH(64, 2);
   else if (c.per_sm == 1) RID_BAT_LAUNCH(32, 1);
   else RID_BAT_LAUNCH(32, 2);
@@ -574,8 +701,9 @@ struct BatchPlan {
   int b = 32;
   int64_t mmax = 0, nmax = 0;
   int sms = 0, slots = 0;
-  size_t off_state = 0, off_probs = 0, off_order = 0, off_results = 0, off_queue = 0, off_slots = 0, slot_bytes = 0,
-         total = 0;
+  int omega_rows = 0;  // rows of Omega drawn once for all problems
+  size_t off_state = 0, off_probs = 0, off_order = 0, off_results = 0, off_queue = 0, off_omega = 0, off_slots = 0,
+         slot_bytes = 0, total = 0;
 };
 
 int sm_count() {
@@ -621,6 +749,12 @@ int batch_plan(int64_t count, const id_matrix* A, const id_opts* o, BatchPlan* b
   bp->off_order = take(4 * count);
   bp->off_results = take(sizeof(Result) * count);
   bp->off_queue = take(256);
+  // eight blocks of rows cover the ranks the path is used for (later blocks are drawn per
+  // problem), within 32 MB, which stays in L2
+  int64_t blocks = ((int64_t)32 << 20) / ((int64_t)bp->b * bp->mmax * bp->elem);
+  if (blocks > 8) blocks = 8;
+  bp->omega_rows = (int)blocks * bp->b;
+  bp->off_omega = take((size_t)bp->omega_rows * bp->mmax * bp->elem);
   bp->off_slots = take(bp->slot_bytes * bp->slots);
   bp->total = off;
   return ID_OK;
@@ -700,7 +834,8 @@ int tune(const Params& p, int elem, int sms, int count, cudaStream_t s, Config* 
   // RANDID_BATCHED_CONFIG=<bm>x<per_sm> (e.g. "32x2") pins the configuration (tests)
   if (const char* env = getenv("RANDID_BATCHED_CONFIG")) {
     int bm = 0, per = 0;
-    if (sscanf(env, "%dx%d", &bm, &per) == 2 && (bm == 32 || bm == 64) && (per == 1 || per == 2)) {
+    if (sscanf(env, "%dx%d", &bm, &per) == 2 && (bm == 32 || bm == 64 || (bm == 128 && elem == 4)) &&
+        (per == 1 || per == 2)) {
       *best = Config{bm, per};
       // launch once outside any capture so the variant's shared-memory limit is set
       Params q = p;
@@ -718,7 +853,9 @@ int tune(const Params& p, int elem, int sms, int count, cudaStream_t s, Config* 
         return ID_OK;
       }
   }
-  const Config cands[4] = {{64, 1}, {64, 2}, {32, 1}, {32, 2}};
+  // taller tiles only pay where shared memory bounds the products (FP32)
+  const Config cands64[4] = {{64, 1}, {64, 2}, {32, 1}, {32, 2}}, cands32[4] = {{128, 1}, {128, 2}, {64, 1}, {64, 2}};
+  const Config(&cands)[4] = elem == 8 ? cands64 : cands32;
   Params q = p;
   q.count = std::min(count, 2 * sms);  // the largest problems come first in `order`
   cudaEvent_t e0, e1;
@@ -794,6 +931,8 @@ extern "C" int id_batched(int64_t count, const id_matrix* A, const id_opts* opts
   p.queue = reinterpret_cast<int*>(w + bp.off_queue);
   p.results = reinterpret_cast<Result*>(w + bp.off_results);
   p.st = reinterpret_cast<rid::DevState*>(w + bp.off_state);
+  p.omega = w + bp.off_omega;
+  p.omega_rows = bp.omega_rows;
   p.slots = w + bp.off_slots;
   p.slot_bytes = bp.slot_bytes;
   p.mmax = bp.mmax;
@@ -827,6 +966,7 @@ extern "C" int id_batched(int64_t count, const id_matrix* A, const id_opts* opts
     if (res[i].status < 0) worst = worst < 0 ? std::min(worst, res[i].status) : res[i].status;
     else if (worst >= 0) worst |= res[i].status;
   }
-  if (count > 0) out[0].launches = 2;  // queue reset + the persistent kernel (graph replay)
+  // Omega's shared rows + the persistent kernel (graph replay)
+  if (count > 0) out[0].launches = bp.omega_rows > 0 ? 2 : 1;
   return worst;
 }
