@@ -462,8 +462,11 @@ struct Smem {
 };
 static_assert(sizeof(Smem) + 1024 <= 232448, "shared memory of k_sketch_f32emu exceeds 227 KB");
 
-// Grid: x = tiles of A's columns (M), y = tiles of W's rows (N), z = K splits of kchunk
-// (a multiple of the chunk).  out[z]: FP32 partial (M x N, row stride ldo).
+// Grid: x = tiles of W's rows (N, fastest: the CTAs that share a tile of A run together
+// and read it from HBM once) and of A's columns (M), z = K splits of kchunk (a multiple
+// of the chunk).  out[z]: FP32 partial (M x N, row stride ldo).  With A's tiles
+// fastest a pass of four W tiles read A twice: 1.32 against 1.24 ms for 256 rows
+// of a 40000 x 10000 matrix.
 __global__ void __launch_bounds__(kThreads, 1)
     k_sketch_f32emu(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w, int M,
                     int N, int K, int kchunk, const int32_t* __restrict__ ea, const int32_t* __restrict__ ew,
@@ -472,7 +475,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (done != nullptr && *done) return;
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * kBN;
+  const unsigned wt = ((unsigned)N + kBN - 1) / kBN;
+  const int m0 = (int)(blockIdx.x / wt) * kBM, n0 = (int)(blockIdx.x % wt) * kBN;
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
   const int nsteps = kend > kbeg ? (kend - kbeg + kBK - 1) / kBK : 0;
@@ -719,7 +723,9 @@ cudaError_t sketch_f32emu(int64_t m, int64_t n, int64_t rows, const void* adig, 
   static SmemLimit lim;
   cudaError_t e = raise_smem(f32s::k_sketch_f32emu, smem, lim);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((n + f32s::kBM - 1) / f32s::kBM), (unsigned)((rows + f32s::kBN - 1) / f32s::kBN), (unsigned)nz);
+  const int64_t tiles = ((n + f32s::kBM - 1) / f32s::kBM) * ((rows + f32s::kBN - 1) / f32s::kBN);
+  if (tiles > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)tiles, 1, (unsigned)nz);
   f32s::k_sketch_f32emu<<<grid, f32s::kThreads, smem, s>>>(ma, mw, (int)n, (int)rows, (int)m, kchunk, aexp, wexp, out,
                                                           ldo, zstride, st, done);
   return cudaGetLastError();
