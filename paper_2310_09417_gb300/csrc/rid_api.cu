@@ -818,9 +818,10 @@ class Engine {
                                xchg_, st_, s_)));
     RID_TRY(tend(1));
     RID_TRY(tbegin(ID_PHASE_UPDATE));
-    int nl = 3;
+    int nl = 2;
     T* Linv_t = Linv_ + (tb / p_.b) * p_.b * p_.b;  // kept per block for the condition of L1
-    RID_TRY(cuda(linv<T>((int)bt, S_, lds, piv_, Linv_t, done_, s_)));
+    RID_TRY(cuda(linv_compact<T>((int)bt, S_, lds, piv_, Linv_t, (int)na, act_[cur_], act_[cur_ ^ 1], out_->J, perm32_,
+                                 tb, out_->pivots, pivdiag_, done_, s_)));
     if (L_ != nullptr) {
       RID_TRY(cuda(store_l<T>((int)na, (int)bt, S_, lds, piv_, pivmark_, act_[cur_], L_, p_.ldl, tb, done_, s_)));
       ++nl;
@@ -847,8 +848,6 @@ class Engine {
         ++nl;
       }
     }
-    RID_TRY(cuda(compact((int)na, (int)bt, act_[cur_], act_[cur_ ^ 1], pivmark_, piv_, out_->J, perm32_, tb,
-                         out_->pivots, pivdiag_, done_, s_)));
     RID_TRY(tend(nl));
     cur_ ^= 1;
     return 0;

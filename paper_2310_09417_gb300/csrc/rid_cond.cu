@@ -217,7 +217,8 @@ cudaError_t resolve_x_f64(int64_t k, int b, int64_t na, const int32_t* perm, con
       ++nl;
     }
     // times the inverse of the unit-lower diagonal block L1(block q, block q)
-    e = linv<double>(bq, L1 + c0, k, iota + c0, Linv64, nullptr, s);
+    e = linv_compact<double>(bq, L1 + c0, k, iota + c0, Linv64, 0, nullptr, nullptr, nullptr, nullptr, 0, nullptr,
+                             nullptr, nullptr, s);
     if (e != cudaSuccess) return e;
     const size_t smem = (size_t)bq * bq * sizeof(double);
     if (smem > 48 * 1024) {

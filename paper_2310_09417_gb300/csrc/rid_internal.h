@@ -132,21 +132,19 @@ template <typename T>
 cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, unsigned seq, T* S, int64_t lds,
                        int32_t* piv, int32_t* pivmark, double* pivdiag, void* xchg, DevState* st, cudaStream_t s);
 
-// Inverse of the unit-lower block L-hat(piv, 0:bt) (bt x bt, row-major).
+// Inverse of the unit-lower block L-hat(piv, 0:bt) (bt x bt, row-major), and the
+// re-blocking beside it: the new pivots are appended to J / perm32 and dropped from
+// the active list of na rows (stable).  na = 0: the inverse alone.
 template <typename T>
-cudaError_t linv(int bt, const T* S, int64_t lds, const int32_t* piv, T* Linv, const int32_t* done,
-                 cudaStream_t s);
+cudaError_t linv_compact(int bt, const T* S, int64_t lds, const int32_t* piv, T* Linv, int na, const int32_t* act_in,
+                         int32_t* act_out, int64_t* J, int32_t* perm32, int64_t tb, double* pivots_out,
+                         const double* pivdiag, const int32_t* done, cudaStream_t s);
 
 // N = L-hat(rest) * Linv; X(tb:tb+bt, act[i]) = N(i,:) for non-pivot rows; pivorig = act[piv].
 template <typename T>
 cudaError_t make_n(int na, int bt, const T* S, int64_t lds, const T* Linv, const int32_t* pivmark,
                    const int32_t* act, T* Nbuf, T* X, int64_t ldx, int64_t tb, const int32_t* piv,
                    int32_t* pivorig, const int32_t* done, cudaStream_t s);
-
-// Drop the new pivots from the active list (stable), append them to J / perm32.
-cudaError_t compact(int na, int bt, const int32_t* act_in, int32_t* act_out, int32_t* pivmark,
-                    const int32_t* piv, int64_t* J, int32_t* perm32, int64_t tb, double* pivots_out,
-                    const double* pivdiag, const int32_t* done, cudaStream_t s);
 
 // X(:, perm32[q]) = e_q for q < k.
 template <typename T>
