@@ -323,6 +323,26 @@ int make_plan(const id_matrix* A, const id_opts* o, int64_t k, int64_t l, Plan* 
     if (rid_rc_ != 0) return rid_rc_; \
   } while (0)
 
+// Two page-locked DevStates of the calling thread, freed with it: a call uses them from
+// its first posted state to its last read one, and calls of one thread follow each other.
+DevState* pinned_states() {
+  struct Holder {
+    DevState* p = nullptr;
+    ~Holder() {
+      if (p != nullptr) cudaFreeHost(p);
+    }
+  };
+  static thread_local Holder h;
+  if (h.p == nullptr) {
+    void* q = nullptr;
+    if (cudaHostAlloc(&q, 2 * sizeof(DevState), cudaHostAllocPortable) == cudaSuccess)
+      h.p = static_cast<DevState*>(q);
+    else
+      cudaGetLastError();  // no page-locked memory: the caller waits for every round
+  }
+  return h.p;
+}
+
 // One call's state and the steps of the method.
 template <typename T>
 class Engine {
@@ -387,12 +407,21 @@ class Engine {
   }
   ~Engine() {
     for (cudaEvent_t e : events_) cudaEventDestroy(e);
+    for (cudaEvent_t e : posted_)
+      if (e != nullptr) cudaEventDestroy(e);
   }
 
+  // Algorithm 1's loop, launched one round ahead of its stop test: while the host waits
+  // for the decision of round t-1 the GPU has round t queued, so it never idles for a
+  // host round trip (about 45 us of a 0.4 - 2 ms round otherwise).  Once the decision
+  // "stop" is on the device every later kernel of the call returns at once, so the round
+  // queued past it leaves no trace: k, the skeleton, the pass count and the active list
+  // are those of the stopping round.
   int run_adaptive() {
     RID_TRY(start());
     int64_t tb = 0, na = p_.n, t = 0, sketched = 0, gstart = 0;
     const int64_t b = p_.b;
+    const bool ahead = !o_.profile && can_post();
     bool full = false;
     for (;;) {
       if (t >= sketched) {
@@ -407,10 +436,15 @@ class Engine {
       }
       RID_TRY(schur((t - gstart) * b, b, tb, na));
       if (t > 0) {
-        RID_TRY(decide(b, tb, tb == p_.cap, (int)(t - 1)));
-        RID_TRY(sync_state());
-        if (h_.err) break;
-        if (h_.done) break;
+        const bool last = tb == p_.cap;
+        RID_TRY(decide(b, tb, last, (int)(t - 1)));
+        if (ahead) {
+          RID_TRY(post_state(t));
+          if (t > 1 || last) RID_TRY(read_state(last ? t : t - 1));
+        } else {
+          RID_TRY(sync_state());
+        }
+        if (h_.err || h_.done) break;
       }
       const int64_t bt = imin(b, p_.cap - tb);
       RID_TRY(factor(b, bt, tb, na));
@@ -422,6 +456,7 @@ class Engine {
                                       o_.tol_relative, st_, s_)));
         RID_TRY(tend(1));
         RID_TRY(sync_state());
+        if (h_.err) break;
         pred_blocks_ = imin(cdiv(imax(h_.k_pred, 1), b), cdiv(p_.cap, b));
         predicted_ = h_.k_pred;
       }
@@ -429,7 +464,8 @@ class Engine {
       na -= bt;
       ++t;
       if (tb == p_.n) {  // every column is a skeleton: X is a permutation, the residual is 0
-        full = true;
+        if (ahead && t > 1) RID_TRY(read_state(t - 1));  // unless the round before it stopped
+        full = !(h_.err || h_.done);
         break;
       }
     }
@@ -554,8 +590,8 @@ class Engine {
       RID_TRY(cuda(norm2_partial<T>(p_.m, p_.n, A_, lda_, normp_, p_.nparts, st_, s_)));
     RID_TRY(cuda(norm2_final(normp_, p_.nparts, st_, s_)));
     RID_TRY(tend(3));
-    RID_TRY(sync_state());
-    if (h_.err & kErrNonFinite) return ID_ERR_NONFINITE;
+    // NaN or Inf in A sets the stop flag as well: every kernel from here on returns at
+    // once and the first read of the state ends the call
     if (p_.path == 33 && !p_.sparse) {  // digits of A's columns, once per call
       RID_TRY(tbegin(ID_PHASE_SKETCH));
       RID_TRY(cuda(sketch_f32emu_slice((int)p_.n, (int)p_.m, reinterpret_cast<const float*>(Araw_), lda_, f32a_, p_.n,
@@ -580,6 +616,32 @@ class Engine {
     RID_TRY(cuda(cudaMemcpyAsync(&h_, st_, sizeof(DevState), cudaMemcpyDeviceToHost, s_)));
     RID_TRY(cuda(cudaStreamSynchronize(s_)));
     collect_times();
+    return 0;
+  }
+
+  // The state as of decision t, copied to page-locked memory in stream order; read_state
+  // waits for that copy only, not for what was queued after it.
+  bool can_post() {
+    pinned_ = pinned_states();
+    for (cudaEvent_t& e : posted_)
+      if (pinned_ != nullptr && e == nullptr && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
+        pinned_ = nullptr;
+    return pinned_ != nullptr;
+  }
+  int post_state(int64_t t) {
+    RID_TRY(cuda(cudaMemcpyAsync(&pinned_[t & 1], st_, sizeof(DevState), cudaMemcpyDeviceToHost, s_)));
+    RID_TRY(cuda(cudaEventRecord(posted_[t & 1], s_)));
+    posted_passes_[t & 1] = passes_;
+    posted_cur_[t & 1] = cur_;
+    return 0;
+  }
+  int read_state(int64_t t) {
+    RID_TRY(cuda(cudaEventSynchronize(posted_[t & 1])));
+    h_ = pinned_[t & 1];
+    if (h_.done) {  // what was queued past the stop did nothing
+      passes_ = posted_passes_[t & 1];
+      cur_ = posted_cur_[t & 1];
+    }
     return 0;
   }
 
@@ -881,9 +943,14 @@ class Engine {
   }
 
   int finish(int64_t k) {
-    if (o_.x_solve_f64 != 0 && k > 0) RID_TRY(condition_and_solve(k));
+    if (o_.x_solve_f64 != 0 && k > 0) {
+      RID_TRY(sync_state());  // it reads the pivot list on the host's word that there is one
+      if (h_.err & kErrTimeout) return ID_ERR_TIMEOUT;
+      if (h_.err & kErrNonFinite) return ID_ERR_NONFINITE;
+      RID_TRY(condition_and_solve(k));
+    }
     RID_TRY(tbegin(ID_PHASE_OTHER));
-    RID_TRY(cuda(finalize_x<T>(k, perm32_, X_, ldx_, s_)));
+    RID_TRY(cuda(finalize_x<T>(k, perm32_, X_, ldx_, st_, s_)));
     RID_TRY(tend(1));
     RID_TRY(sync_state());
     int status = ID_OK;
@@ -957,6 +1024,10 @@ class Engine {
   int64_t phase_launches_[kNumPhases];
   std::vector<cudaEvent_t> events_;
   std::vector<int> pending_;
+  DevState* pinned_ = nullptr;  // two posted states (can_post)
+  cudaEvent_t posted_[2] = {nullptr, nullptr};
+  int32_t posted_passes_[2] = {0, 0};
+  int posted_cur_[2] = {0, 0};
 };
 
 int check_ws(const Plan& p, void* ws, size_t ws_bytes) {

@@ -148,7 +148,7 @@ cudaError_t make_n(int na, int bt, const T* S, int64_t lds, const T* Linv, const
 
 // X(:, perm32[q]) = e_q for q < k.
 template <typename T>
-cudaError_t finalize_x(int64_t k, const int32_t* perm32, T* X, int64_t ldx, cudaStream_t s);
+cudaError_t finalize_x(int64_t k, const int32_t* perm32, T* X, int64_t ldx, const DevState* st, cudaStream_t s);
 
 // Clears the state, lists every column as active and zeroes `clear` (16-byte words).
 cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, void* clear, size_t clear_bytes,

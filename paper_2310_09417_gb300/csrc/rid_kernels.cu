@@ -817,6 +817,7 @@ __global__ void __launch_bounds__(kPanelThreads)
           bad = 1;
         } else if (now - t0 > kWaitLimitNs) {
           atomicOr(&st->err, kErrTimeout);
+          st->done = 1;  // the kernels queued after this launch return at once
           bad = 1;
         }
       }
@@ -1265,7 +1266,9 @@ cudaError_t make_n(int na, int bt, const T* S, int64_t lds, const T* Linv, const
 }
 
 template <typename T>
-__global__ void k_finalize_x(int64_t k, const int32_t* __restrict__ perm32, T* __restrict__ X, int64_t ldx) {
+__global__ void k_finalize_x(int64_t k, const int32_t* __restrict__ perm32, T* __restrict__ X, int64_t ldx,
+                             const DevState* st) {
+  if (st->err != 0u) return;  // the pivot list is not complete
   const int64_t total = k * k;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -1275,11 +1278,11 @@ __global__ void k_finalize_x(int64_t k, const int32_t* __restrict__ perm32, T* _
 }
 
 template <typename T>
-cudaError_t finalize_x(int64_t k, const int32_t* perm32, T* X, int64_t ldx, cudaStream_t s) {
+cudaError_t finalize_x(int64_t k, const int32_t* perm32, T* X, int64_t ldx, const DevState* st, cudaStream_t s) {
   if (k <= 0) return cudaSuccess;
   int64_t blocks = (k * k + 255) / 256;
   if (blocks > 4096) blocks = 4096;
-  k_finalize_x<T><<<(int)blocks, 256, 0, s>>>(k, perm32, X, ldx);
+  k_finalize_x<T><<<(int)blocks, 256, 0, s>>>(k, perm32, X, ldx, st);
   return cudaGetLastError();
 }
 
@@ -1386,7 +1389,7 @@ cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, 
   template cudaError_t make_n<T>(int, int, const T*, int64_t, const T*, const int32_t*, const int32_t*, T*, \
                                  T*, int64_t, int64_t, const int32_t*, int32_t*, const int32_t*,            \
                                  cudaStream_t);                                                             \
-  template cudaError_t finalize_x<T>(int64_t, const int32_t*, T*, int64_t, cudaStream_t);                  \
+  template cudaError_t finalize_x<T>(int64_t, const int32_t*, T*, int64_t, const DevState*, cudaStream_t);  \
   template cudaError_t gather_panel<T>(const T*, int64_t, int64_t, int64_t, const int64_t*, int64_t, T*,     \
                                        DevState*, cudaStream_t);                                            \
   template cudaError_t transpose_w<T>(const T*, int64_t, int64_t, int64_t, T*, int64_t, cudaStream_t);

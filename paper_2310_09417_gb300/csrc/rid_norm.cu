@@ -279,7 +279,10 @@ __global__ void k_norm2_final(const double* part, int nparts, DevState* st) {
   double acc = 0.0;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[i];
   const double tot = block_sum(acc);
-  if (threadIdx.x == 0) st->norm2_A = tot;
+  if (threadIdx.x == 0) {
+    st->norm2_A = tot;
+    if (st->err & kErrNonFinite) st->done = 1;  // nothing of the call runs after this
+  }
 }
 
 // E4M3 with one FP32 scale per 128 rows of a column: sum of scale^2 times the exact
