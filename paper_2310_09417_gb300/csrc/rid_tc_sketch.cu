@@ -4,15 +4,14 @@
 // row-major, BF16), FP32 accumulation in tensor memory (Sec. 2.4; the sampling step of Algorithm 1).
 // Both operands are K-major (K = m): a column of A and a row of Omega are contiguous.
 //
-// One CTA computes a 128 (columns of A) x NT BN (rows of Omega) tile over a K range:
-//   warp 0   one lane issues TMA loads (128B-swizzled boxes of 64 K x 128 / 64 x up to
-//            256 rows of Omega)
-//   warp 1   allocates tensor memory; one lane issues tcgen05.mma (M=128, K=16; N=BN
-//            for one sub-tile, N=256 over four back-to-back sub-tiles), all reading the
-//            same stage of A: a pass of many blocks reads each tile of A once per CTA
-//            instead of once per BN rows, and every entry's sums are the same whatever
-//            NT is (the same bits for any pass size, checked against one-block passes)
-//   warps 2-5 drain the accumulator with tcgen05.ld and write FP32 rows of G
+// One block of 64 rows of Omega: a CTA computes a 128 (columns of A) x 64 tile over a K
+// range.  Several blocks: a CTA pair computes 256 x 256 (described at the kernel).
+// Every entry's sums are the same whichever kernel takes the pass (the same bits for
+// any pass size, checked against one-block passes).
+//
+//   warp 0    one lane issues the TMA loads
+//   warp 1    allocates tensor memory; one lane issues tcgen05.mma
+//   warps 2-5 epilogue: tensor memory -> FP32 rows of G
 // A STAGES-deep ring of shared-memory stages is guarded by "full" (TMA bytes landed)
 // and "empty" (the MMAs that read the stage completed) mbarriers.  Every wait is
 // bounded by %globaltimer; on a timeout the CTA records kErrTimeout, waits (bounded)
@@ -32,18 +31,15 @@ namespace tc {
 
 constexpr int kBM = 128;        // columns of A per tile (MMA M)
 constexpr int kBK = 64;         // K per stage: 64 BF16 = one 128-byte swizzle row
-// stages per CTA: 4 of (16 + 8 NT) KB, NT = 1 (two CTAs per SM) or 4 sub-tiles of Omega
-__host__ __device__ constexpr int stages_for(int) { return 4; }
-constexpr int kWBox = 256;     // rows of Omega per TMA box (the box limit)
+constexpr int kBN1 = 64;        // rows of Omega per CTA (one block)
+constexpr int kStages = 4;      // of 24 KB: two CTAs per SM
 constexpr int kThreads = 192;   // 6 warps
 
 using namespace tcx;
 
-template <int BN, int NT>
 struct Smem {
-  static constexpr int kStages = stages_for(NT);
-  alignas(1024) __nv_bfloat16 a[kStages][kBM * kBK];      // 16 KB per stage
-  alignas(1024) __nv_bfloat16 w[kStages][NT * BN * kBK];  // NT BN * 128 bytes per stage
+  alignas(1024) __nv_bfloat16 a[kStages][kBM * kBK];   // 16 KB per stage
+  alignas(1024) __nv_bfloat16 w[kStages][kBN1 * kBK];  // 8 KB per stage
   uint64_t full[kStages];
   uint64_t empty[kStages];
   uint64_t accum;
@@ -52,9 +48,11 @@ struct Smem {
   int abort;
 };
 
-// Grid: x = groups of NT BN rows of Omega (fastest, so the CTAs that share a tile of
-// A run together and reuse it from L2), y = tiles of A's columns, z = K splits.
-template <int BN, int NT>
+static_assert(2 * (sizeof(Smem) + 1024 + 1024) <= 228 * 1024, "two CTAs of k_sketch_tc_bf16 per SM");
+
+// One block of Omega rows.  Grid: x = groups of kBN1 rows of Omega (fastest, so the CTAs
+// that share a tile of A run together and reuse it from L2), y = tiles of A's columns,
+// z = K splits.
 __global__ void __launch_bounds__(kThreads, 1)
     k_sketch_tc_bf16(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w, int n,
                      int rows, int K, int kchunk, float* __restrict__ out, int64_t out_ld, int64_t zstride,
@@ -62,16 +60,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   if (done != nullptr && *done) return;
   // dynamic shared memory is only guaranteed 16-byte aligned: align the carve-out to 1024
-  Smem<BN, NT>& sm =
-      *reinterpret_cast<Smem<BN, NT>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  constexpr int kStages = Smem<BN, NT>::kStages;
+  Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * kBM;       // first column of A
-  const int n0 = blockIdx.x * NT * BN;   // first row of Omega
+  const int n0 = blockIdx.x * kBN1;   // first row of Omega
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
   const int nkb = (kend - kbeg + kBK - 1) / kBK;
-  constexpr uint32_t kTmemCols = NT * BN < 32 ? 32 : NT * BN;
+  constexpr uint32_t kTmemCols = kBN1;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -100,12 +96,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int kb = 0; kb < nkb; ++kb) {
       const int s = kb % kStages;
       if (kb >= kStages && !mbar_wait(&sm.empty[s], ((kb / kStages) + 1) & 1, st)) break;
-      mbar_expect_tx(&sm.full[s], (kBM + NT * BN) * kBK * 2);
+      mbar_expect_tx(&sm.full[s], (kBM + kBN1) * kBK * 2);
       const int k0 = kbeg + kb * kBK;
       tma_load_2d(sm.a[s], &map_a, &sm.full[s], k0, m0);
-#pragma unroll
-      for (int h = 0; h < (NT * BN + kWBox - 1) / kWBox; ++h)  // boxes of at most 256 rows
-        tma_load_2d(sm.w[s] + h * kWBox * kBK, &map_w, &sm.full[s], k0, n0 + h * kWBox);
+      tma_load_2d(sm.w[s], &map_w, &sm.full[s], k0, n0);
       issued = kb + 1;
     }
     // copies still in flight must land before the CTA can leave
@@ -113,9 +107,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_wait_drain(&sm.full[kb % kStages], (kb / kStages) & 1);
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer
-    constexpr uint32_t idesc = idesc_bf16(kBM, BN);
-    constexpr int kNW = NT * BN < 256 ? NT * BN : 256;       // N of one MMA over back-to-back sub-tiles
-    constexpr uint32_t idesc_wide = idesc_bf16(kBM, kNW);
+    constexpr uint32_t idesc = idesc_bf16(kBM, kBN1);
     int consumed = 0;
     for (int kb = 0; kb < nkb; ++kb) {
       const int s = kb % kStages;
@@ -124,21 +116,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t da = desc_sw128(sm.a[s]);
       const uint64_t dw = desc_sw128(sm.w[s]);
 #pragma unroll
-      for (int kk = 0; kk < kBK / 16; ++kk) {  // advance 16 BF16 = 32 bytes inside the swizzle row
-        if constexpr (NT > 1) {
-          // the sub-tiles lie back to back (BN rows of 128 bytes each): MMAs of N = 256
-          // (the same per-entry sums as one MMA per sub-tile, checked bit for bit)
-#pragma unroll
-          for (int h = 0; h < NT * BN / kNW; ++h)
-            mma_bf16(tmem + h * kNW, da + 2 * kk, dw + (uint64_t)((h * kNW * kBK * 2) >> 4) + 2 * kk, idesc_wide,
-                     (kb | kk) != 0);
-        } else {
-#pragma unroll
-          for (int t = 0; t < NT; ++t)  // sub-tile t: BN rows of 128 bytes, 1024-byte aligned
-            mma_bf16(tmem + t * BN, da + 2 * kk, dw + (uint64_t)((t * BN * kBK * 2) >> 4) + 2 * kk, idesc,
-                     (kb | kk) != 0);
-        }
-      }
+      for (int kk = 0; kk < kBK / 16; ++kk)  // advance 16 BF16 = 32 bytes inside the swizzle row
+        mma_bf16(tmem, da + 2 * kk, dw + 2 * kk, idesc, (kb | kk) != 0);
       mma_commit(&sm.empty[s]);
       consumed = kb + 1;
     }
@@ -159,7 +138,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int row = m0 + quarter * 32 + lane;
       float* o = out + blockIdx.z * zstride + static_cast<int64_t>(row) * out_ld;
 #pragma unroll 1
-      for (int c0 = 0; c0 < NT * BN; c0 += 16) {
+      for (int c0 = 0; c0 < kBN1; c0 += 16) {
         float v[16];
         tmem_ld16(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0, v);
         if (row < n) {
@@ -175,6 +154,130 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) {
     fence_after_sync();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ CTA pairs
+// Passes of several 64-row blocks: a CTA pair multiplies 256 columns of A (128 per CTA)
+// by 256 rows of Omega (128 per CTA, the halves of the MMA's N = 256).  A single CTA has
+// to load 48 KB per 512 clocks of MMA for the same tile (A and all of Omega's rows),
+// more than an SM takes from L2 (about 64 bytes per clock); a CTA of a pair loads 32 KB.
+// The same products in the same K order: the sums are those of the single-CTA kernel.
+// 512 rows of a 100000 x 20000 matrix: 1.68 -> 1.53 ms (1.34 PFLOP/s).
+constexpr int kPairN = 256;     // rows of Omega per pair
+constexpr int kPairDual = 2;    // K steps per stage (one barrier per 64 KB)
+constexpr int kPairStages = 3;
+
+struct PairSmem {
+  alignas(1024) __nv_bfloat16 a[kPairStages][kPairDual][kBM * kBK];         // 16 KB per K step
+  alignas(1024) __nv_bfloat16 w[kPairStages][kPairDual][kPairN / 2 * kBK];  // 16 KB per K step
+  uint64_t full[kPairStages];   // (even CTA) both CTAs' boxes have arrived
+  uint64_t empty[kPairStages];  // the MMAs have read them
+  uint64_t accum;               // the accumulators are final
+  uint32_t tmem_base;
+};
+static_assert(sizeof(PairSmem) + 1024 <= 232448, "shared memory of k_sketch_tc_bf16_pair exceeds 227 KB");
+
+// Grid: x = 2 x groups of 256 rows of Omega (fastest; the cluster is two along x), y =
+// pairs of tiles of A's columns, z = K splits.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+    k_sketch_tc_bf16_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w, int n,
+                          int rows, int K, int kchunk, float* __restrict__ out, int64_t out_ld, int64_t zstride,
+                          DevState* st, const int32_t* done) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  if (done != nullptr && *done) return;  // set before the launch: the same in both CTAs
+  PairSmem& sm = *reinterpret_cast<PairSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cta_rank_in_cluster();
+  const int m0 = (2 * (int)blockIdx.y + (int)rank) * kBM;  // first column of A; may lie past A in the odd CTA
+  const int n0 = (int)(blockIdx.x >> 1) * kPairN;          // first row of Omega
+  const int kbeg = blockIdx.z * kchunk;
+  const int kend = min(K, kbeg + kchunk);
+  const int nkb = (kend - kbeg + kBK - 1) / kBK;  // K steps
+  const int nst = (nkb + kPairDual - 1) / kPairDual;
+  constexpr uint32_t kTmemCols = kPairN;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kPairStages; ++s) {
+      mbar_init(&sm.full[s], 1);
+      mbar_init(&sm.empty[s], 1);
+    }
+    mbar_init(&sm.accum, 1);
+    mbar_init_fence();
+  }
+  if (warp == 1) tmem_alloc_pair(&sm.tmem_base, kTmemCols);
+  fence_before_sync();
+  __syncthreads();
+  cluster_barrier();
+  fence_after_sync();
+  const uint32_t tmem = sm.tmem_base;
+
+  if (warp == 0 && lane == 0) {
+    // ---------------- TMA producer (each CTA its own operands; the even CTA's barriers
+    // count the bytes of both).  A K step past the split's end is loaded and not used.
+    int issued = 0;
+    for (int t = 0; t < nst; ++t) {
+      const int s = t % kPairStages;
+      if (t >= kPairStages && !mbar_wait_cluster(&sm.empty[s], ((t / kPairStages) + 1) & 1, st)) break;
+      if (rank == 0) mbar_expect_tx(&sm.full[s], 2 * kPairDual * (kBM + kPairN / 2) * kBK * 2);
+      const uint32_t bar = smem_in_cta(&sm.full[s], 0);
+#pragma unroll
+      for (int h = 0; h < kPairDual; ++h) {
+        const int k0 = kbeg + (t * kPairDual + h) * kBK;
+        tma_load_2d_pair(sm.a[s][h], &map_a, bar, k0, m0);
+        tma_load_2d_pair(sm.w[s][h], &map_w, bar, k0, n0 + (int)rank * (kPairN / 2));
+      }
+      issued = t + 1;
+    }
+    if (rank == 0)  // the copies of both CTAs have landed before either may leave
+      for (int t = issued - kPairStages < 0 ? 0 : issued - kPairStages; t < issued; ++t)
+        mbar_wait_drain(&sm.full[t % kPairStages], (t / kPairStages) & 1);
+  } else if (warp == 1 && lane == 0) {
+    // ---------------- MMA issuer (even CTA)
+    if (rank == 0) {
+      constexpr uint32_t idesc = idesc_bf16(2 * kBM, kPairN);
+      for (int t = 0; t < nst; ++t) {
+        const int s = t % kPairStages;
+        if (!mbar_wait_cluster(&sm.full[s], (t / kPairStages) & 1, st)) break;
+        fence_after_sync();
+        for (int h = 0; h < kPairDual && t * kPairDual + h < nkb; ++h) {
+          const uint64_t da = desc_sw128(sm.a[s][h]), dw = desc_sw128(sm.w[s][h]);
+#pragma unroll
+          for (int kk = 0; kk < kBK / 16; ++kk)  // advance 16 BF16 = 32 bytes inside the swizzle row
+            mma_bf16_pair(tmem, da + 2 * kk, dw + 2 * kk, idesc, (t | h | kk) != 0);
+        }
+        mma_commit_pair(&sm.empty[s]);
+      }
+      mma_commit_pair(&sm.accum);  // also after a timeout: what was issued has completed
+      mbar_wait_drain(&sm.accum, 0);
+    }
+  } else if (warp >= 2) {
+    // ---------------- epilogue: tensor memory -> G
+    bool ok = mbar_wait_cluster(&sm.accum, 0, st);
+    fence_after_sync();
+    ok = ok && (ld_acquire_u32(&st->err) & kErrTimeout) == 0u;  // an aborted sum is not stored
+    if (ok) {
+      const int quarter = warp & 3;  // warps 2..5 own lane quarters 2,3,0,1
+      const int row = m0 + quarter * 32 + lane;
+      float* o = out + blockIdx.z * zstride + static_cast<int64_t>(row) * out_ld;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kPairN; c0 += 16) {
+        float v[16];
+        tmem_ld16(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0, v);
+        if (row < n) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (n0 + c0 + i < rows) o[n0 + c0 + i] = v[i];
+        }
+      }
+    }
+  }
+  fence_before_sync();
+  __syncthreads();
+  cluster_barrier();  // neither CTA leaves while the other's MMAs, copies or arrivals may still touch it
+  if (warp == 1) {
+    fence_after_sync();
+    tmem_dealloc_pair(tmem, kTmemCols);
   }
 }
 
@@ -213,12 +316,6 @@ bool make_map_bf16(CUtensorMap* map, const void* base, int64_t inner, int64_t ou
   return r == CUDA_SUCCESS;
 }
 
-template <int BN, int NT>
-size_t smem_bytes() {
-  static_assert(sizeof(Smem<BN, NT>) + 1024 <= 232448, "shared memory of k_sketch_tc_bf16 exceeds 227 KB");
-  return sizeof(Smem<BN, NT>) + 1024;  // + alignment slack
-}
-
 }  // namespace tc
 
 bool tc_sketch_supported(const void* A, int64_t lda, const void* W, int64_t ldw) {
@@ -238,35 +335,33 @@ int tc_sketch_splits(int64_t m, int64_t n, int64_t rows, int sms) {
 cudaError_t tc_sketch_bf16(const void* A, int64_t lda, int64_t m, int64_t n, const void* W, int64_t ldw,
                            int64_t rows, float* out, int64_t out_ld, int64_t zstride, int splits, DevState* st,
                            const int32_t* done, cudaStream_t s) {
-  constexpr int BN = 64;
-  // passes of several blocks: four BN-row sub-tiles of Omega per CTA, and as many
-  // CTAs per tile of A as groups of four blocks (they run together, x fastest, and
-  // share the tile through L2).  Eight sub-tiles per CTA (two N = 256 MMAs per step,
-  // two stages of 80 KB) measured slower: 11.4 against 9.4 ms of sketch per ID at
-  // eight blocks per pass, 16.3 against 14.2 ms for one pass of 37 blocks.
-  const int nt = rows > BN ? 4 : 1;
+  // more than one block of 64 rows: CTA pairs; one block: a CTA per tile, two CTAs per SM
+  const bool pair = rows > tc::kBN1;
   CUtensorMap ma, mw;
   if (!tc::make_map_bf16(&ma, A, m, n, lda, tc::kBM)) return cudaErrorInvalidValue;
-  if (!tc::make_map_bf16(&mw, W, m, rows, ldw, nt * BN < tc::kWBox ? nt * BN : tc::kWBox)) return cudaErrorInvalidValue;
+  if (!tc::make_map_bf16(&mw, W, m, rows, ldw, pair ? tc::kPairN / 2 : tc::kBN1)) return cudaErrorInvalidValue;
   int kchunk = (int)((m + splits - 1) / splits);
   kchunk = ((kchunk + tc::kBK - 1) / tc::kBK) * tc::kBK;
   const int nz = (int)((m + kchunk - 1) / kchunk);
   const int64_t ytiles = (n + tc::kBM - 1) / tc::kBM;
   if (ytiles > 65535 || nz > 65535) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)((rows + nt * BN - 1) / (nt * BN)), (unsigned)ytiles, (unsigned)nz);
   cudaError_t e;
-  if (nt == 4) {
-    static SmemLimit lim4;
-    e = raise_smem(tc::k_sketch_tc_bf16<BN, 4>, tc::smem_bytes<BN, 4>(), lim4);
+  if (pair) {
+    constexpr size_t smem = sizeof(tc::PairSmem) + 1024;  // + alignment slack
+    static SmemLimit lim;
+    e = raise_smem(tc::k_sketch_tc_bf16_pair, smem, lim);
     if (e != cudaSuccess) return e;
-    tc::k_sketch_tc_bf16<BN, 4><<<grid, tc::kThreads, tc::smem_bytes<BN, 4>(), s>>>(
-        ma, mw, (int)n, (int)rows, (int)m, kchunk, out, out_ld, zstride, st, done);
+    dim3 grid(2 * (unsigned)((rows + tc::kPairN - 1) / tc::kPairN), (unsigned)((ytiles + 1) / 2), (unsigned)nz);
+    tc::k_sketch_tc_bf16_pair<<<grid, tc::kThreads, smem, s>>>(ma, mw, (int)n, (int)rows, (int)m, kchunk, out, out_ld,
+                                                               zstride, st, done);
   } else {
-    static SmemLimit lim1;
-    e = raise_smem(tc::k_sketch_tc_bf16<BN, 1>, tc::smem_bytes<BN, 1>(), lim1);
+    constexpr size_t smem = sizeof(tc::Smem) + 1024;
+    static SmemLimit lim;
+    e = raise_smem(tc::k_sketch_tc_bf16, smem, lim);
     if (e != cudaSuccess) return e;
-    tc::k_sketch_tc_bf16<BN, 1><<<grid, tc::kThreads, tc::smem_bytes<BN, 1>(), s>>>(
-        ma, mw, (int)n, (int)rows, (int)m, kchunk, out, out_ld, zstride, st, done);
+    dim3 grid((unsigned)((rows + tc::kBN1 - 1) / tc::kBN1), (unsigned)ytiles, (unsigned)nz);
+    tc::k_sketch_tc_bf16<<<grid, tc::kThreads, smem, s>>>(ma, mw, (int)n, (int)rows, (int)m, kchunk, out, out_ld,
+                                                          zstride, st, done);
   }
   return cudaGetLastError();
 }
