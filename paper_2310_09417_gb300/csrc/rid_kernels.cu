@@ -653,8 +653,9 @@ cudaError_t decide(const double* e2part, int nparts, int w, double tol, int tol_
 //  - warp 0 alone polls every block's magnitude words (a lane reads up to five
 //    blocks at once), picks the winner by integer maxima, and reads its row: one
 //    trip for the candidates, one for the row, which was stored at the same time
-//    and is normally there.  The larger magnitude wins; block b's rows come before
-//    block b+1's, so ties go to the smaller block.
+//    and is normally there.  In FP64 the polling trips already bring the row of the best
+//    candidate so far.  The larger magnitude wins; block b's rows come before block
+//    b+1's, so ties go to the smaller block.
 //  - the other warps run the rank-1 update of the previous pivot meanwhile.  Column
 //    c+1 and the candidate's row are updated before (look-ahead), so the bulk of the
 //    update is never waited for unless it is longer than the exchange.
@@ -666,6 +667,7 @@ cudaError_t decide(const double* e2part, int nparts, int w, double tol, int tol_
 constexpr int kPanelThreads = 256;
 constexpr int kPanelMaxW = 128;
 constexpr int kPanelPoll = 5;  // candidates a lane of the polling warp reads at once
+constexpr int kPanelMaxBlocks = 32 * kPanelPoll;
 
 __device__ __forceinline__ unsigned long long mag_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
@@ -693,14 +695,15 @@ __device__ __forceinline__ int warp_mag_argmax(bool have, unsigned long long mag
   return __ffs(__ballot_sync(0xffffffffu, in)) - 1;
 }
 
-// 64-bit words of one block's publication: the magnitude (kMagWords), then the row
-// index, then the row's entries (kValWords each).  A block without a candidate
-// stores kNoCand.
+// 64-bit words of one block's publication: the magnitude (kMag), then the row index,
+// (FP64) the reciprocal of its pivot entry, and the row's entries (kVal each).  A block
+// without a candidate stores kNoCand.
 template <typename T>
 struct PanelWords {
-  static constexpr int kMag = 2;                  // magnitude words (16-byte stride; FP32 uses the first)
-  static constexpr int kVal = (int)sizeof(T) / 4;  // words per entry
-  __host__ __device__ static constexpr int row_words(int w) { return 2 + kVal * ((w + 1) & ~1); }
+  static constexpr int kMag = 2;                         // magnitude words (16-byte stride; FP32 uses the first)
+  static constexpr int kVal = (int)sizeof(T) / 4;         // words per entry
+  static constexpr int kHead = sizeof(T) == 8 ? 4 : 2;    // words before the entries
+  __host__ __device__ static constexpr int row_words(int w) { return kHead + kVal * ((w + 1) & ~1); }
   __host__ __device__ static constexpr int slot_words(int w) { return kMag + row_words(w); }
 };
 constexpr unsigned kNoCand = 0xFFFFFFFFu;
@@ -715,6 +718,29 @@ __device__ __forceinline__ unsigned long long tagged(unsigned data, unsigned tag
   return ((unsigned long long)tag << 32) | data;
 }
 
+// a / b rounded to nearest given r = 1 / b rounded to nearest: q = a r is within one ulp
+// of the quotient, a - b q is exact in an FMA, and the corrected q is the rounded
+// quotient unless b's significand is all ones (P. W. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990).  `ok`: b is such
+// and far from the ends of the exponent range; an a that is not, and zeros, take the
+// division itself.  On GB300 an FP64 division is a chain of a dozen instructions at
+// sixty-four clocks each, this one of three; the reciprocal is computed by the block that
+// publishes the row, while the others wait for it.
+__device__ __forceinline__ bool recip_usable(double b) {
+  const unsigned hi = (unsigned)__double2hiint(b), e = (hi >> 20) & 0x7FFu;
+  return e - 523u <= 1000u && !((hi & 0xFFFFFu) == 0xFFFFFu && __double2loint(b) == -1);
+}
+__device__ __forceinline__ double divide_by(double a, double b, double r, bool ok) {
+  const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7FFu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7FFu;
+  if (ok && ea - 523u <= 1000u && ea + 500u >= eb) {
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+  }
+  return a / b;
+}
+__device__ __forceinline__ bool recip_usable(float) { return false; }
+__device__ __forceinline__ float divide_by(float a, float b, float, bool) { return a / b; }
+
 template <typename T>
 __global__ void __launch_bounds__(kPanelThreads)
     k_panel_lupp(int na, int w, int steps, T* __restrict__ S, int64_t lds, int chunk, int use_smem, unsigned tag0,
@@ -722,6 +748,7 @@ __global__ void __launch_bounds__(kPanelThreads)
   using PW = PanelWords<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T prow[2][kPanelMaxW];
+  __shared__ T s_rcp[2];  // FP64: the pivot's reciprocal
   __shared__ int s_piv[2];
   __shared__ unsigned long long s_mag[kPanelThreads / 32];
   __shared__ int s_row[kPanelThreads / 32];
@@ -790,10 +817,22 @@ __global__ void __launch_bounds__(kPanelThreads)
       }
       if constexpr (sizeof(T) == 8) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-        st_relaxed_v2(rw + 2 + 2 * cc, tagged((unsigned)(b >> 32), tag), tagged((unsigned)b, tag));
+        st_relaxed_v2(rw + PW::kHead + 2 * cc, tagged((unsigned)(b >> 32), tag), tagged((unsigned)b, tag));
       } else {
-        st_relaxed(rw + 2 + cc, tagged(__float_as_uint(v), tag));
+        st_relaxed(rw + PW::kHead + cc, tagged(__float_as_uint(v), tag));
       }
+    }
+  };
+  // Warp 1 (FP64), meanwhile: the reciprocal of the candidate's entry in column c.
+  auto publish_rcp = [&](int c, int cand) {
+    if constexpr (sizeof(T) == 8) {
+      if (cand < 0) return;
+      const unsigned tag = tag0 + (unsigned)c;
+      const unsigned long long b =
+          (unsigned long long)__double_as_longlong(1.0 / Ss[(int64_t)cand * ldl + c]);
+      if (lane == 0)
+        st_relaxed_v2(rows + ((size_t)(c & 1) * nb + bid) * rwords + 2, tagged((unsigned)(b >> 32), tag),
+                      tagged((unsigned)b, tag));
     }
   };
   // Warp 0: wait until every block's magnitude for pivot c is there, pick the winner
@@ -802,9 +841,6 @@ __global__ void __launch_bounds__(kPanelThreads)
   auto collect = [&](int c) {
     const unsigned tag = tag0 + (unsigned)c;
     const unsigned long long* mw = xchg + (size_t)(c & 1) * nb * PW::kMag;
-    bool have = false;
-    unsigned long long bmag = 0ull;
-    int bq = 0;
     unsigned spins = 0;
     uint64_t t0 = 0;
     auto gave_up = [&]() {  // uniform over the warp
@@ -823,71 +859,110 @@ __global__ void __launch_bounds__(kPanelThreads)
       }
       return __shfl_sync(0xffffffffu, bad, 0) != 0;
     };
-    for (int q0 = 0; q0 < nb; q0 += 32 * kPanelPoll) {
-      unsigned long long v[kPanelPoll], u[kPanelPoll];
-      for (;;) {
-        bool all = true;
+    // The row of block q: its words, and whether all of them are this step's.
+    unsigned long long g = 0ull, ih = 0ull, il = 0ull, rh[kPanelMaxW / 32], rl[kPanelMaxW / 32];
+    auto load_row = [&](int q) {
+      const unsigned long long* rw = rows + ((size_t)(c & 1) * nb + q) * rwords;
+      g = ld_relaxed(rw);
+      if (sizeof(T) == 8) ld_relaxed_v2(rw + 2, ih, il);
 #pragma unroll
-        for (int i = 0; i < kPanelPoll; ++i) {
-          const int q = q0 + lane + 32 * i;
-          v[i] = u[i] = tagged(kNoCand, tag);
-          if (q < nb) {
-            if (sizeof(T) == 8)
-              ld_relaxed_v2(mw + (size_t)q * PW::kMag, v[i], u[i]);
-            else
-              v[i] = ld_relaxed(mw + (size_t)q * PW::kMag);
-          }
+      for (int j = 0; j < kPanelMaxW / 32; ++j) {
+        const int cc = c + lane + 32 * j;
+        rh[j] = rl[j] = tagged(0u, tag);
+        if (cc < w) {
+          if (sizeof(T) == 8)
+            ld_relaxed_v2(rw + PW::kHead + 2 * cc, rh[j], rl[j]);
+          else
+            rh[j] = ld_relaxed(rw + PW::kHead + cc);
         }
+      }
+    };
+    auto row_ready = [&]() {
+      bool all = (unsigned)(g >> 32) == tag;
+      if (sizeof(T) == 8) all = all && (unsigned)(ih >> 32) == tag && (unsigned)(il >> 32) == tag;
 #pragma unroll
-        for (int i = 0; i < kPanelPoll; ++i)
-          all = all && (unsigned)(v[i] >> 32) == tag && (sizeof(T) == 4 || (unsigned)(u[i] >> 32) == tag);
-        if (__all_sync(0xffffffffu, all)) break;
+      for (int j = 0; j < kPanelMaxW / 32; ++j)
+        all = all && (unsigned)(rh[j] >> 32) == tag && (unsigned)(rl[j] >> 32) == tag;
+      return __all_sync(0xffffffffu, all) != 0;
+    };
+    // FP64: a trip also brings the row of the best candidate known so far (the last blocks
+    // to publish seldom hold the maximum); FP32 steps are too short to pay for the maximum
+    // of every unfinished trip
+    constexpr bool kGuess = sizeof(T) == 8;
+    int guess = -1;  // the block whose row the last trip brought along
+    for (;;) {
+      unsigned long long v[kPanelPoll], u[kPanelPoll];
+#pragma unroll
+      for (int i = 0; i < kPanelPoll; ++i) {
+        const int q = lane + 32 * i;
+        v[i] = u[i] = tagged(kNoCand, tag);
+        if (q < nb) {
+          if (sizeof(T) == 8)
+            ld_relaxed_v2(mw + (size_t)q * PW::kMag, v[i], u[i]);
+          else
+            v[i] = ld_relaxed(mw + (size_t)q * PW::kMag);
+        }
+      }
+      if (kGuess && guess >= 0) load_row(guess);
+      bool all = true, have = false;
+      unsigned long long bmag = 0ull;
+      int bq = 0;
+#pragma unroll
+      for (int i = 0; i < kPanelPoll; ++i) {
+        const bool in = (unsigned)(v[i] >> 32) == tag && (sizeof(T) == 4 || (unsigned)(u[i] >> 32) == tag);
+        all = all && in;
+        const unsigned hi = (unsigned)v[i];
+        const unsigned long long mag = ((unsigned long long)hi << 32) | (sizeof(T) == 8 ? (unsigned)u[i] : 0u);
+        if (in && hi != kNoCand && (!have || mag > bmag)) {  // ascending blocks: ties keep the smaller
+          have = true;
+          bmag = mag;
+          bq = lane + 32 * i;
+        }
+      }
+      const bool complete = __all_sync(0xffffffffu, all) != 0;
+      if (!kGuess && !complete) {
         if (gave_up()) {
           if (lane == 0) s_piv[c & 1] = -2;
           return;
         }
+        continue;
       }
-#pragma unroll
-      for (int i = 0; i < kPanelPoll; ++i) {
-        const unsigned hi = (unsigned)v[i];
-        const unsigned long long mag = ((unsigned long long)hi << 32) | (sizeof(T) == 8 ? (unsigned)u[i] : 0u);
-        if (hi != kNoCand && (!have || mag > bmag)) {  // ascending blocks: ties keep the smaller
-          have = true;
-          bmag = mag;
-          bq = q0 + lane + 32 * i;
-        }
-      }
-    }
-    unsigned long long best = 0ull;
-    if (warp_mag_argmax<T>(have, bmag, best) < 0) {
-      if (lane == 0) s_piv[c & 1] = -1;
-      return;
-    }
-    const int q = (int)__reduce_min_sync(0xffffffffu, have && bmag == best ? (unsigned)bq : 0x7FFFFFFFu);
-    const unsigned long long* rw = rows + ((size_t)(c & 1) * nb + q) * rwords;
-    for (;;) {
-      const unsigned long long g = ld_relaxed(rw);
-      bool all = (unsigned)(g >> 32) == tag;
-#pragma unroll
-      for (int j = 0; j < kPanelMaxW / 32; ++j) {
-        const int cc = c + lane + 32 * j;
-        if (cc < w) {
-          if constexpr (sizeof(T) == 8) {
-            unsigned long long h, l;
-            ld_relaxed_v2(rw + 2 + 2 * cc, h, l);
-            all = all && (unsigned)(h >> 32) == tag && (unsigned)(l >> 32) == tag;
-            prow[c & 1][cc] = __longlong_as_double((long long)((h << 32) | (l & 0xFFFFFFFFull)));
-          } else {
-            const unsigned long long h = ld_relaxed(rw + 2 + cc);
-            all = all && (unsigned)(h >> 32) == tag;
-            prow[c & 1][cc] = __uint_as_float((unsigned)h);
-          }
-        }
-      }
-      if (__all_sync(0xffffffffu, all)) {
-        if (lane == 0) s_piv[c & 1] = (int)(unsigned)g;
+      unsigned long long best = 0ull;
+      int q = -1;
+      if (warp_mag_argmax<T>(have, bmag, best) >= 0)
+        q = (int)__reduce_min_sync(0xffffffffu, have && bmag == best ? (unsigned)bq : 0x7FFFFFFFu);
+      if (complete && q < 0) {
+        if (lane == 0) s_piv[c & 1] = -1;
         return;
       }
+      bool there = complete && kGuess && q == guess && row_ready();
+      while (complete && !kGuess && !there) {
+        load_row(q);
+        there = row_ready();
+        if (!there && gave_up()) {
+          if (lane == 0) s_piv[c & 1] = -2;
+          return;
+        }
+      }
+      if (there) {
+#pragma unroll
+        for (int j = 0; j < kPanelMaxW / 32; ++j) {
+          const int cc = c + lane + 32 * j;
+          if (cc < w) {
+            if constexpr (sizeof(T) == 8)
+              prow[c & 1][cc] = __longlong_as_double((long long)((rh[j] << 32) | (rl[j] & 0xFFFFFFFFull)));
+            else
+              prow[c & 1][cc] = __uint_as_float((unsigned)rh[j]);
+          }
+        }
+        if (lane == 0) {
+          s_piv[c & 1] = (int)(unsigned)g;
+          if constexpr (sizeof(T) == 8)
+            s_rcp[c & 1] = __longlong_as_double((long long)((ih << 32) | (il & 0xFFFFFFFFull)));
+        }
+        return;
+      }
+      guess = q;
       if (gave_up()) {
         if (lane == 0) s_piv[c & 1] = -2;
         return;
@@ -910,9 +985,12 @@ __global__ void __launch_bounds__(kPanelThreads)
     }
     if (steps > 0) warp_cand(have, mag, row);
     __syncthreads();
-    if (steps > 0 && wid == 0) {
+    if (steps > 0 && wid <= 1) {
       const int cand = block_cand(mag);
-      publish(0, cand, mag, nullptr, T(0), false);
+      if (wid == 0)
+        publish(0, cand, mag, nullptr, T(0), false);
+      else
+        publish_rcp(0, cand);
     }
   }
 
@@ -929,7 +1007,8 @@ __global__ void __launch_bounds__(kPanelThreads)
     const bool more = c + 1 < steps;
     // 2. multipliers l(i) = S(i,c) / pivot, column c+1 of the update and its maximum
     {
-      const T p1 = more ? pr[c + 1] : T(0);
+      const T p1 = more ? pr[c + 1] : T(0), rcp = sizeof(T) == 8 ? s_rcp[c & 1] : T(0);
+      const bool usable = recip_usable(pv);
       bool have = false;
       unsigned long long mag = 0ull;
       int brow = 0;
@@ -940,7 +1019,7 @@ __global__ void __launch_bounds__(kPanelThreads)
           T* row = Ss + (int64_t)r * ldl;
           T v = more ? row[c + 1] : T(0);
           if (elim) {
-            const T l = row[c] / pv;
+            const T l = divide_by(row[c], pv, rcp, usable);
             row[c] = l;
             if (more) row[c + 1] = v = fma(-l, p1, v);
           }
@@ -968,6 +1047,8 @@ __global__ void __launch_bounds__(kPanelThreads)
       if (wid == 0) {
         const T l = cand >= 0 ? Ss[(int64_t)cand * ldl + c] : T(0);
         publish(c + 1, cand, mag, pr, l, elim);
+      } else if (wid == 1) {
+        publish_rcp(c + 1, cand);
       }
     }
     // 4. the rest of the rank-1 update: a warp per row, lanes along the row, four rows
@@ -1044,6 +1125,7 @@ PanelCfg panel_config(int na, int w, int num_sms) {
   const int need = (na + fit - 1) / fit;
   int most = (na + 31) / 32;
   if (most > num_sms) most = num_sms;
+  if (most > kPanelMaxBlocks) most = kPanelMaxBlocks;
   if (most < 1) most = 1;
   int grid = panel_blocks_env();
   if (grid == 0) grid = most;
@@ -1079,7 +1161,7 @@ cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, unsigned s
   static SmemLimit lim;
   if (w > kPanelMaxW || steps > w) return cudaErrorInvalidValue;
   // the kernel addresses chunk rows at stride w + 1 and the selection bytes after them
-  if (cfg.chunk < 1 || (int64_t)cfg.chunk * cfg.grid < na ||
+  if (cfg.chunk < 1 || cfg.grid > kPanelMaxBlocks || (int64_t)cfg.chunk * cfg.grid < na ||
       cfg.smem < panel_smem_bytes(cfg.chunk, w, sizeof(T), cfg.use_smem != 0))
     return cudaErrorInvalidValue;
   cudaError_t e = raise_smem(k_panel_lupp<T>, cfg.smem, lim);
