@@ -1292,58 +1292,172 @@ cudaError_t linv_compact(int bt, const T* S, int64_t lds, const int32_t* piv, T*
   return cudaGetLastError();
 }
 
-// N(i, c) = sum_{c' >= c} L-hat(i, c') Linv(c', c) for non-pivot rows; the new
-// columns tb..tb+bt of X(:, act[i]) are N(i, :) (the new block of L2 L1^{-1}).
-// Each sum runs in ascending c' (one FMA per term from 0).  A thread takes the
-// columns q and bt-1-q of a row (bt + 1 terms together), so the lanes of a warp
-// do equal work: one thread per column spent a third of the FP64 pipe on the
-// short sums' idle lanes.
-template <typename T>
-__global__ void k_make_n(int na, int bt, const T* __restrict__ S, int64_t lds, const T* __restrict__ Linv,
-                         const int32_t* __restrict__ pivmark, const int32_t* __restrict__ act, T* __restrict__ Nbuf,
-                         T* __restrict__ X, int64_t ldx, int64_t tb, const int32_t* __restrict__ piv,
-                         int32_t* __restrict__ pivorig, const int32_t* done) {
+// N(i, c) = sum_{c' >= c} L-hat(i, c') Linv(c', c) for non-pivot rows; the new columns
+// tb..tb+bt of X(:, act[i]) are N(i, :) (the new block of L2 L1^{-1}).  Each sum runs in
+// ascending c' (one FMA per term from 0).
+//
+// FP64: bound by its pipe, sixteen clocks per warp instruction whatever the active
+// lanes (sixty-four on one scheduler).  Lanes are rows, so every lane works in every term
+// of the triangle; a warp takes 32 rows and CW columns and their mirror images, bt + CW
+// terms of CW columns whichever they are.  CW is four, and less where that would leave
+// schedulers without a warp.  With lanes along the columns a third of the pipe went to
+// idle lanes: n = 10000, bt = 64: 60 -> 40 us, n = 400,
+// bt = 48: 10.9 -> 7.2.
+// FP32: a warp takes four rows at a time, lanes along the columns; a term costs one
+// broadcast vector of the rows' multipliers and one value of Linv per 32 columns, both
+// from shared memory, where a read of S per FMA bounded it: n = 12003, bt = 64: 18.6 -> 8.3 us.
+constexpr int kNRows64 = 128;  // rows of a CTA (four warps)
+template <int CW>
+__global__ void __launch_bounds__(kNRows64)
+    k_make_n64(int na, int bt, const double* __restrict__ S, int64_t lds, const double* __restrict__ Linv,
+               const int32_t* __restrict__ pivmark, const int32_t* __restrict__ act, double* __restrict__ Nbuf,
+               double* __restrict__ X, int64_t ldx, int64_t tb, const int32_t* __restrict__ piv,
+               int32_t* __restrict__ pivorig, const int32_t* done) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (done != nullptr && *done) return;
-  T* Li = reinterpret_cast<T*>(smem_raw);
-  for (int e = threadIdx.x; e < bt * bt; e += blockDim.x) Li[e] = Linv[e];
-  if (blockIdx.x == 0)
-    for (int c = threadIdx.x; c < bt; c += blockDim.x) pivorig[c] = act[piv[c]];
+  double* Lq = reinterpret_cast<double*>(smem_raw);  // two groups of Linv's columns: bt x 2 CW
+  if (blockIdx.x == 0 && blockIdx.y == 0)
+    for (int c = threadIdx.x; c < bt; c += kNRows64) pivorig[c] = act[piv[c]];
+  const int nq = (bt + CW - 1) / CW, qa = blockIdx.y, qb = nq - 1 - qa;
+  for (int e = threadIdx.x; e < bt * 2 * CW; e += kNRows64) {
+    const int cp = e / (2 * CW), u = e % (2 * CW), c = CW * (u >= CW ? qb : qa) + u % CW;
+    Lq[e] = c < bt ? Linv[cp * bt + c] : 0.0;
+  }
   __syncthreads();
-  const int hb = (bt + 1) / 2;
-  const int64_t total = (int64_t)na * hb;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / hb;
-    const int q = (int)(e - i * hb);
-    if (pivmark[i]) continue;
-    const T* l = S + i * lds;
-    T* xr = X + (int64_t)act[i] * ldx + tb;
+  const int i = blockIdx.x * kNRows64 + threadIdx.x;
+  if (i >= na || pivmark[i]) return;
+  const double* l = S + (int64_t)i * lds;
+  double* nr = Nbuf + (int64_t)i * bt;
+  double* xr = X + (int64_t)act[i] * ldx + tb;
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const int c = h == 0 ? q : bt - 1 - q;
-      if (h == 1 && c == q) break;  // the middle column of an odd bt
-      T acc = T(0);
+  for (int h = 0; h < 2; ++h) {
+    const int q = h == 0 ? qa : qb;
+    if (h == 1 && qb == qa) break;  // the middle group of an odd count
+    const int c0 = CW * q;
+    double acc[CW];
+#pragma unroll
+    for (int j = 0; j < CW; ++j) acc[j] = 0.0;
+    const double* lq = Lq + CW * h;
+#pragma unroll
+    for (int u = 0; u < CW; ++u)  // the diagonal: column c0 + j starts at term c0 + j
+      if (c0 + u < bt) {
+        const double x = l[c0 + u];
+#pragma unroll
+        for (int j = 0; j <= u; ++j) acc[j] = fma(x, lq[(c0 + u) * 2 * CW + j], acc[j]);
+      }
 #pragma unroll 8
-      for (int cp = c; cp < bt; ++cp) acc = fma(l[cp], Li[cp * bt + c], acc);
-      Nbuf[i * bt + c] = acc;
-      xr[c] = acc;
+    for (int cp = c0 + CW; cp < bt; ++cp) {
+      const double x = l[cp];
+#pragma unroll
+      for (int j = 0; j < CW; ++j) acc[j] = fma(x, lq[cp * 2 * CW + j], acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < CW; ++j)
+      if (c0 + j < bt) {
+        nr[c0 + j] = acc[j];
+        xr[c0 + j] = acc[j];
+      }
+  }
+}
+
+constexpr int kNRows32 = 32;             // rows of a CTA (eight warps of four)
+constexpr int kNLd = kNRows32 + 4;       // keeps a warp's four rows 16-byte aligned
+__global__ void __launch_bounds__(256)
+    k_make_n32(int na, int bt, const float* __restrict__ S, int64_t lds, const float* __restrict__ Linv,
+               const int32_t* __restrict__ pivmark, const int32_t* __restrict__ act, float* __restrict__ Nbuf,
+               float* __restrict__ X, int64_t ldx, int64_t tb, const int32_t* __restrict__ piv,
+               int32_t* __restrict__ pivorig, const int32_t* done) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (done != nullptr && *done) return;
+  float* Ls = reinterpret_cast<float*>(smem_raw);  // bt x kNLd: the rows' multipliers, transposed
+  float* Li = Ls + bt * kNLd;                      // bt x bt
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * kNRows32;
+  if (blockIdx.x == 0)
+    for (int c = threadIdx.x; c < bt; c += 256) pivorig[c] = act[piv[c]];
+  for (int e = threadIdx.x; e < bt * bt; e += 256) Li[e] = Linv[e];
+  for (int e = threadIdx.x; e < kNRows32 * bt; e += 256) {
+    const int r = e / bt, c = e - r * bt;
+    Ls[c * kNLd + r] = i0 + r < na ? S[(int64_t)(i0 + r) * lds + c] : 0.f;
+  }
+  __syncthreads();
+  const float* lw = Ls + 4 * warp;
+  for (int g = 0; g < bt; g += 64) {  // two columns per lane
+    const int ca = g + lane, cb = ca + 32;
+    float a[4] = {0.f, 0.f, 0.f, 0.f}, b[4] = {0.f, 0.f, 0.f, 0.f};
+    const int mid = min(g + 32, bt);
+#pragma unroll 4
+    for (int cp = g; cp < mid; ++cp) {
+      const float4 l = *reinterpret_cast<const float4*>(lw + cp * kNLd);
+      if (cp >= ca) {
+        const float y = Li[cp * bt + ca];
+        a[0] = fmaf(l.x, y, a[0]);
+        a[1] = fmaf(l.y, y, a[1]);
+        a[2] = fmaf(l.z, y, a[2]);
+        a[3] = fmaf(l.w, y, a[3]);
+      }
+    }
+#pragma unroll 4
+    for (int cp = mid; cp < bt; ++cp) {
+      const float4 l = *reinterpret_cast<const float4*>(lw + cp * kNLd);
+      const float y = Li[cp * bt + ca];  // ca < mid <= cp
+      a[0] = fmaf(l.x, y, a[0]);
+      a[1] = fmaf(l.y, y, a[1]);
+      a[2] = fmaf(l.z, y, a[2]);
+      a[3] = fmaf(l.w, y, a[3]);
+      if (cp >= cb) {
+        const float z = Li[cp * bt + cb];
+        b[0] = fmaf(l.x, z, b[0]);
+        b[1] = fmaf(l.y, z, b[1]);
+        b[2] = fmaf(l.z, z, b[2]);
+        b[3] = fmaf(l.w, z, b[3]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = i0 + 4 * warp + r;
+      if (i >= na || pivmark[i]) continue;
+      float* nr = Nbuf + (int64_t)i * bt;
+      float* xr = X + (int64_t)act[i] * ldx + tb;
+      if (ca < bt) nr[ca] = xr[ca] = a[r];
+      if (cb < bt) nr[cb] = xr[cb] = b[r];
     }
   }
 }
 
-template <typename T>
-cudaError_t make_n(int na, int bt, const T* S, int64_t lds, const T* Linv, const int32_t* pivmark,
-                   const int32_t* act, T* Nbuf, T* X, int64_t ldx, int64_t tb, const int32_t* piv,
-                   int32_t* pivorig, const int32_t* done, cudaStream_t s) {
-  static SmemLimit lim;
-  cudaError_t e = raise_smem(k_make_n<T>, (size_t)bt * bt * sizeof(T), lim);
+template <>
+cudaError_t make_n<double>(int na, int bt, const double* S, int64_t lds, const double* Linv, const int32_t* pivmark,
+                           const int32_t* act, double* Nbuf, double* X, int64_t ldx, int64_t tb, const int32_t* piv,
+                           int32_t* pivorig, const int32_t* done, cudaStream_t s) {
+  if (na <= 0 || bt <= 0) return cudaSuccess;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  int64_t blocks = ((int64_t)na * ((bt + 1) / 2) + 255) / 256;
-  if (blocks > 1216) blocks = 1216;
-  if (blocks < 1) blocks = 1;
-  k_make_n<T><<<(int)blocks, 256, (size_t)bt * bt * sizeof(T), s>>>(na, bt, S, lds, Linv, pivmark, act, Nbuf, X,
-                                                                      ldx, tb, piv, pivorig, done);
+  const int64_t warps1 = ((int64_t)na + 31) / 32 * ((bt + 1) / 2);  // of one column and its image each
+  auto run = [&](auto cw) {
+    constexpr int CW = decltype(cw)::value;
+    const dim3 grid((na + kNRows64 - 1) / kNRows64, ((bt + CW - 1) / CW + 1) / 2);
+    k_make_n64<CW><<<grid, kNRows64, (size_t)bt * 2 * CW * sizeof(double), s>>>(
+        na, bt, S, lds, Linv, pivmark, act, Nbuf, X, ldx, tb, piv, pivorig, done);
+    return cudaGetLastError();
+  };
+  if (warps1 >= 16 * (int64_t)sms) return run(std::integral_constant<int, 4>());  // four warps per scheduler's SM at least
+  if (warps1 >= 8 * (int64_t)sms) return run(std::integral_constant<int, 2>());
+  return run(std::integral_constant<int, 1>());
+}
+
+template <>
+cudaError_t make_n<float>(int na, int bt, const float* S, int64_t lds, const float* Linv, const int32_t* pivmark,
+                          const int32_t* act, float* Nbuf, float* X, int64_t ldx, int64_t tb, const int32_t* piv,
+                          int32_t* pivorig, const int32_t* done, cudaStream_t s) {
+  if (na <= 0 || bt <= 0) return cudaSuccess;
+  static SmemLimit lim;
+  const size_t smem = ((size_t)bt * kNLd + (size_t)bt * bt) * sizeof(float);
+  cudaError_t e = raise_smem(k_make_n32, smem, lim);
+  if (e != cudaSuccess) return e;
+  k_make_n32<<<(na + kNRows32 - 1) / kNRows32, 256, smem, s>>>(na, bt, S, lds, Linv, pivmark, act, Nbuf, X, ldx, tb,
+                                                               piv, pivorig, done);
   return cudaGetLastError();
 }
 
@@ -1468,9 +1582,6 @@ cudaError_t init_state(DevState* st, int32_t* act, int32_t* pivmark, int64_t n, 
   template cudaError_t linv_compact<T>(int, const T*, int64_t, const int32_t*, T*, int, const int32_t*,      \
                                        int32_t*, int64_t*, int32_t*, int64_t, double*, const double*,       \
                                        const int32_t*, cudaStream_t);                                       \
-  template cudaError_t make_n<T>(int, int, const T*, int64_t, const T*, const int32_t*, const int32_t*, T*, \
-                                 T*, int64_t, int64_t, const int32_t*, int32_t*, const int32_t*,            \
-                                 cudaStream_t);                                                             \
   template cudaError_t finalize_x<T>(int64_t, const int32_t*, T*, int64_t, const DevState*, cudaStream_t);  \
   template cudaError_t gather_panel<T>(const T*, int64_t, int64_t, int64_t, const int64_t*, int64_t, T*,     \
                                        DevState*, cudaStream_t);                                            \
