@@ -67,24 +67,38 @@ struct Smem {
 static_assert(sizeof(Smem) + 1024 <= 232448, "shared memory of k_sketch_f64emu exceeds 227 KB");
 static_assert(kChunkSteps % kDual == 0, "a stage never straddles an exact chunk");
 
-// Grid: x = tiles of Omega rows (fastest, so CTAs that share an A tile run
-// together and reuse it from L2), y = tiles of A's columns, z = K splits of
-// kchunk (a multiple of the exact chunk).  out: FP64 partial (n x rows, row
-// stride out_ld) of split blockIdx.z.
+// Work items: (tile of Omega rows x, tile of A's columns y, K split z), x fastest, then y;
+// split z covers kchunk (a multiple of the exact chunk) of K and writes the FP64 partial
+// out[z] (n x rows, row stride out_ld).  The kernel is persistent, one CTA per SM: CTA b
+// takes the items b, b + gridDim.x, ..., so the CTAs that share an A tile still run
+// together and reuse it from L2.  The split count is high (it fixes the order of the FP64
+// sums, hence their bits), so an item is only a few chunks long: as a CTA of its own it
+// paid for its start, its first loads and the conversion and store of its 8192 sums with
+// the tensor cores idle.  Here the loads and MMAs of the next item run meanwhile.
+// 128 rows of a 40000 x 10000 matrix (40 splits): 1.90 -> 1.56 ms.
 __global__ void __launch_bounds__(kThreads, 1)
     k_sketch_f64emu(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
-                    const int32_t* __restrict__ colexp, int n, int rows, int K, int kchunk,
-                    double* __restrict__ out, int64_t out_ld, int64_t zstride, DevState* st, const int32_t* done) {
+                    const int32_t* __restrict__ colexp, int n, int rows, int K, int kchunk, int xtiles, int ytiles,
+                    int64_t items, double* __restrict__ out, int64_t out_ld, int64_t zstride, DevState* st,
+                    const int32_t* done) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   if (done != nullptr && *done) return;
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * kBN;
-  const int m0 = blockIdx.y * kBM;
-  const int kbeg = blockIdx.z * kchunk;
-  const int kend = min(K, kbeg + kchunk);
-  const int nsteps = (kend - kbeg + kBK - 1) / kBK;  // K stages of this split
-  const int nchunks = (nsteps + kChunkSteps - 1) / kChunkSteps;
+  struct Item {
+    int x, y, z, kbeg, nsteps, nchunks;  // nsteps: K stages of the split
+  };
+  auto item_at = [&](int64_t id) {
+    Item t;
+    const int64_t yz = id / xtiles;
+    t.x = (int)(id - yz * xtiles);
+    t.z = (int)(yz / ytiles);
+    t.y = (int)(yz - (int64_t)t.z * ytiles);
+    t.kbeg = t.z * kchunk;
+    t.nsteps = (min(K, t.kbeg + kchunk) - t.kbeg + kBK - 1) / kBK;
+    t.nchunks = (t.nsteps + kChunkSteps - 1) / kChunkSteps;
+    return t;
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -110,67 +124,83 @@ __global__ void __launch_bounds__(kThreads, 1)
     // adjacent tiles) and both Omega digits at those steps.  Splits start and end on
     // chunk boundaries, so a step j+1 past the chunk only occurs at the end of K,
     // where the boxes read the zero fill past the tensors' extents.
-    int it = 0;
+    int b = 0;                      // the stage's buffer
+    uint32_t par = 0, wrapped = 0;  // the parity of its use; whether it was used before
     bool ok = true;
-    for (int c = 0; c < nchunks && ok; ++c) {
-      const int steps_c = min(kChunkSteps, nsteps - c * kChunkSteps);
-      for (int s = 0; s < kSlices && ok; ++s) {
-        for (int j = 0; j < steps_c; j += kDual, ++it) {
-          const int b = it % kStages;
-          if (it >= kStages && !mbar_wait(&sm.empty[b], ((it / kStages) + 1) & 1, st)) { ok = false; break; }
-          mbar_expect_tx(&sm.full[b], kDual * (kBM + 2 * kBN) * kBK * 2);
-          const int k0 = kbeg + (c * kChunkSteps + j) * kBK;
-          tma_load_4d(sm.a[b], &map_a, &sm.full[b], 0, 0, k0 / kBK, s * (int)gridDim.y + (int)blockIdx.y);
+    for (int64_t id = blockIdx.x; id < items && ok; id += gridDim.x) {
+      const Item t = item_at(id);
+      for (int c = 0; c < t.nchunks && ok; ++c) {
+        const int steps_c = min(kChunkSteps, t.nsteps - c * kChunkSteps);
+        for (int s = 0; s < kSlices && ok; ++s) {
+          for (int j = 0; j < steps_c; j += kDual) {
+            if (wrapped && !mbar_wait(&sm.empty[b], par ^ 1, st)) { ok = false; break; }
+            mbar_expect_tx(&sm.full[b], kDual * (kBM + 2 * kBN) * kBK * 2);
+            const int k0 = t.kbeg + (c * kChunkSteps + j) * kBK;
+            tma_load_4d(sm.a[b], &map_a, &sm.full[b], 0, 0, k0 / kBK, s * ytiles + t.y);
 #pragma unroll
-          for (int h = 0; h < kDual; ++h) tma_load_3d(sm.w[b][h], &map_w, &sm.full[b], k0 + h * kBK, n0, 0);
+            for (int h = 0; h < kDual; ++h) tma_load_3d(sm.w[b][h], &map_w, &sm.full[b], k0 + h * kBK, t.x * kBN, 0);
+            if (++b == kStages) {
+              b = 0;
+              par ^= 1;
+              wrapped = 1;
+            }
+          }
         }
       }
     }
     // the copies still in flight land before the CTA may exit
-    for (int t = it - kStages < 0 ? 0 : it - kStages; t < it; ++t) mbar_wait_drain(&sm.full[t % kStages], (t / kStages) & 1);
+    for (int u = 0; u < kStages; ++u)
+      if (u < b || wrapped) mbar_wait_drain(&sm.full[u], u < b ? par : par ^ 1);
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer
     constexpr uint32_t id128 = idesc_bf16(kBM, 2 * kBN), id64 = idesc_bf16(kBM, kBN);
-    int it = 0;
+    int b = 0;                   // the stage's buffer
+    uint32_t spar = 0, gc = 0;  // the parity of its use; chunks of this CTA, over its items
     bool ok = true;
-    for (int c = 0; c < nchunks && ok; ++c) {
-      const int steps_c = min(kChunkSteps, nsteps - c * kChunkSteps);
-      for (int s = 0; s < kSlices && ok; ++s) {
-        if (c > 0) {
-          // groups s and s+1 are overwritten from here on: the epilogue must have
-          // read them for chunk c-1 (group s was already awaited at slice s-1)
-          const uint32_t par = (c - 1) & 1;
-          if (s == 0 && !mbar_wait(&sm.free_[0], par, st)) { ok = false; break; }
-          if (!mbar_wait(&sm.free_[s + 1], par, st)) { ok = false; break; }
-          fence_after_sync();
-        }
-        const uint32_t dst = tmem + s * kBN;
-        for (int j = 0; j < steps_c; j += kDual, ++it) {
-          const int b = it % kStages;
-          if (!mbar_wait(&sm.full[b], (it / kStages) & 1, st)) { ok = false; break; }
-          fence_after_sync();
-          for (int h = 0; h < kDual && j + h < steps_c; ++h) {
-            const uint64_t da = desc_sw128(sm.a[b][h]);
-            const uint64_t dq1 = desc_sw128(sm.w[b][h]);             // high digit of Omega (weight 1)
-            const uint64_t dq0 = desc_sw128(sm.w[b][h] + kBN * kBK);  // low digit (weight 2^-8)
+    for (int64_t id = blockIdx.x; id < items && ok; id += gridDim.x) {
+      const Item t = item_at(id);
+      for (int c = 0; c < t.nchunks && ok; ++c, ++gc) {
+        const int steps_c = min(kChunkSteps, t.nsteps - c * kChunkSteps);
+        for (int s = 0; s < kSlices && ok; ++s) {
+          if (gc > 0) {
+            // groups s and s+1 are overwritten from here on: the epilogue must have
+            // read them for the chunk before (group s was already awaited at slice s-1)
+            const uint32_t par = (gc - 1) & 1;
+            if (s == 0 && !mbar_wait(&sm.free_[0], par, st)) { ok = false; break; }
+            if (!mbar_wait(&sm.free_[s + 1], par, st)) { ok = false; break; }
+            fence_after_sync();
+          }
+          const uint32_t dst = tmem + s * kBN;
+          for (int j = 0; j < steps_c; j += kDual) {
+            if (!mbar_wait(&sm.full[b], spar, st)) { ok = false; break; }
+            fence_after_sync();
+            for (int h = 0; h < kDual && j + h < steps_c; ++h) {
+              const uint64_t da = desc_sw128(sm.a[b][h]);
+              const uint64_t dq1 = desc_sw128(sm.w[b][h]);             // high digit of Omega (weight 1)
+              const uint64_t dq0 = desc_sw128(sm.w[b][h] + kBN * kBK);  // low digit (weight 2^-8)
 #pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              const bool first = (j + h == 0 && kk == 0);
-              if (first && s > 0) {
-                // group s continues, group s+1 starts: two MMAs with their own flags
-                mma_bf16(dst, da, dq1, id64, 1u);
-                mma_bf16(dst + kBN, da, dq0, id64, 0u);
-              } else {
-                // groups s and s+1 at once (N = 128: q1 rows then q0 rows)
-                mma_bf16(dst, da + 2 * kk, dq1 + 2 * kk, id128, (first && s == 0) ? 0u : 1u);
+              for (int kk = 0; kk < kBK / 16; ++kk) {
+                const bool first = (j + h == 0 && kk == 0);
+                if (first && s > 0) {
+                  // group s continues, group s+1 starts: two MMAs with their own flags
+                  mma_bf16(dst, da, dq1, id64, 1u);
+                  mma_bf16(dst + kBN, da, dq0, id64, 0u);
+                } else {
+                  // groups s and s+1 at once (N = 128: q1 rows then q0 rows)
+                  mma_bf16(dst, da + 2 * kk, dq1 + 2 * kk, id128, (first && s == 0) ? 0u : 1u);
+                }
               }
             }
+            mma_commit(&sm.empty[b]);
+            if (++b == kStages) {
+              b = 0;
+              spar ^= 1;
+            }
           }
-          mma_commit(&sm.empty[b]);
-        }
-        if (ok) {
-          mma_commit(&sm.ready[s]);  // group s is final for chunk c
-          if (s == kSlices - 1) mma_commit(&sm.ready[s + 1]);  // and the last group with it
+          if (ok) {
+            mma_commit(&sm.ready[s]);  // group s is final for chunk c
+            if (s == kSlices - 1) mma_commit(&sm.ready[s + 1]);  // and the last group with it
+          }
         }
       }
     }
@@ -182,45 +212,49 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int ew = warp - 2;
     const int quarter = warp & 3;  // TMEM lanes this warp may read
     const int half = ew >> 2;      // columns [32 half, 32 half + 32) of the tile
-    const int row = m0 + quarter * 32 + lane;
     const uint32_t base = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + half * 32;
-    long long hi[32], lo[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) hi[i] = lo[i] = 0;
+    uint32_t gc = 0;
     bool ok = true;
-    for (int c = 0; c < nchunks && ok; ++c) {
+    for (int64_t id = blockIdx.x; id < items && ok; id += gridDim.x) {
+      const Item t = item_at(id);
+      long long hi[32], lo[32];
 #pragma unroll
-      for (int g = 0; g < kGroups; ++g) {
-        if (!mbar_wait(&sm.ready[g], c & 1, st)) { ok = false; break; }
-        fence_after_sync();
+      for (int i = 0; i < 32; ++i) hi[i] = lo[i] = 0;
+      for (int c = 0; c < t.nchunks && ok; ++c, ++gc) {
 #pragma unroll
-        for (int cb = 0; cb < 32; cb += 16) {
-          float v[16];
-          tmem_ld16(base + g * kBN + cb, v);
+        for (int g = 0; g < kGroups; ++g) {
+          if (!mbar_wait(&sm.ready[g], gc & 1, st)) { ok = false; break; }
+          fence_after_sync();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            if (g == 0) add_scaled<24>(hi[cb + i], v[i]);
-            else if (g == 1) add_scaled<16>(hi[cb + i], v[i]);
-            else if (g == 2) add_scaled<8>(hi[cb + i], v[i]);
-            else if (g == 3) add_scaled<0>(hi[cb + i], v[i]);
-            else if (g == 4) add_scaled<24>(lo[cb + i], v[i]);
-            else if (g == 5) add_scaled<16>(lo[cb + i], v[i]);
-            else if (g == 6) add_scaled<8>(lo[cb + i], v[i]);
-            else add_scaled<0>(lo[cb + i], v[i]);
+          for (int cb = 0; cb < 32; cb += 16) {
+            float v[16];
+            tmem_ld16(base + g * kBN + cb, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              if (g == 0) add_scaled<24>(hi[cb + i], v[i]);
+              else if (g == 1) add_scaled<16>(hi[cb + i], v[i]);
+              else if (g == 2) add_scaled<8>(hi[cb + i], v[i]);
+              else if (g == 3) add_scaled<0>(hi[cb + i], v[i]);
+              else if (g == 4) add_scaled<24>(lo[cb + i], v[i]);
+              else if (g == 5) add_scaled<16>(lo[cb + i], v[i]);
+              else if (g == 6) add_scaled<8>(lo[cb + i], v[i]);
+              else add_scaled<0>(lo[cb + i], v[i]);
+            }
           }
+          fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.free_[g]);
         }
-        fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.free_[g]);
       }
-    }
-    if (ok && row < n) {
-      const int e = colexp[row];
-      double* o = out + blockIdx.z * zstride + static_cast<int64_t>(row) * out_ld + n0 + half * 32;
-      const int lim = rows - n0 - half * 32;
+      const int row = t.y * kBM + quarter * 32 + lane;
+      if (ok && row < n) {
+        const int e = colexp[row];
+        double* o = out + t.z * zstride + static_cast<int64_t>(row) * out_ld + t.x * kBN + half * 32;
+        const int lim = rows - t.x * kBN - half * 32;
 #pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (i < lim) o[i] = fixed_to_double(hi[i], lo[i], e - 66);
+        for (int i = 0; i < 32; ++i)
+          if (i < lim) o[i] = fixed_to_double(hi[i], lo[i], e - 66);
+      }
     }
   }
   fence_before_sync();
@@ -563,9 +597,15 @@ cudaError_t f64emu_sketch(const void* digits, const int32_t* colexp, int64_t m, 
   static SmemLimit lim;
   cudaError_t e = raise_smem(tc64::k_sketch_f64emu, smem, lim);
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)((rows + tc64::kBN - 1) / tc64::kBN), (unsigned)ytiles, (unsigned)nz);
-  tc64::k_sketch_f64emu<<<grid, tc64::kThreads, smem, s>>>(ma, mw, colexp, (int)n, (int)rows, (int)mp, kchunk, out,
-                                                           out_ld, zstride, st, done);
+  const int64_t xtiles = (rows + tc64::kBN - 1) / tc64::kBN, items = xtiles * ytiles * nz;
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int grid = (int)(items < sms ? items : sms);
+  tc64::k_sketch_f64emu<<<grid, tc64::kThreads, smem, s>>>(ma, mw, colexp, (int)n, (int)rows, (int)mp, kchunk,
+                                                           (int)xtiles, (int)ytiles, items, out, out_ld, zstride, st,
+                                                           done);
   return cudaGetLastError();
 }
 
