@@ -82,6 +82,9 @@ __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kBM;
   const int n0 = blockIdx.y * C::kCols;
+  // the last group of rows may hold fewer blocks than the tile: only their columns are
+  // multiplied and drained (576 rows on 256-row tiles, 50001 x 12003: 0.73 -> 0.71 ms)
+  const int ncols = min(C::kCols, (rows - n0 + 31) / 32 * 32);
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
   const int nkb = (kend - kbeg + kBK - 1) / kBK;
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
       mbar_wait_drain(&sm.full[kb % kStages], (kb / kStages) & 1);
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer: scale block kb -> accumulator kb % kAcc
-    constexpr uint32_t idesc = idesc_e4m3(kBM, C::kCols);
+    const uint32_t idesc = idesc_e4m3(kBM, ncols);
     for (int kb = 0; kb < nkb; ++kb) {
       const int s = kb % kStages, a = kb % C::kAcc;
       if (kb >= C::kAcc && !mbar_wait(&sm.acc_empty[a], ((kb / C::kAcc) + 1) & 1, st)) break;
@@ -159,6 +162,7 @@ __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
       fence_after_sync();
 #pragma unroll
       for (int cb = 0; cb < C::kWarpCols; cb += 32) {  // 32 columns per wait on tensor memory
+        if (col0 + cb >= ncols) break;
         float v[32];
         tmem_ld32(lane_base + a * C::kCols + cb, v);
 #pragma unroll
