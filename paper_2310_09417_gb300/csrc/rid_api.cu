@@ -586,6 +586,9 @@ class Engine {
     else if (p_.path == 65 && !p_.sparse)  // the column exponents of the digit slices come with the norm
       RID_TRY(cuda(norm2_f64(p_.m, p_.n, reinterpret_cast<const double*>(Araw_), lda_, normp_, p_.nparts, colexp_, st_,
                              s_)));
+    else if (p_.path == 33 && !p_.sparse)
+      RID_TRY(cuda(norm2_f32(p_.m, p_.n, reinterpret_cast<const float*>(Araw_), lda_, normp_, p_.nparts, f32ae_, st_,
+                             s_)));
     else
       RID_TRY(cuda(norm2_partial<T>(p_.m, p_.n, A_, lda_, normp_, p_.nparts, st_, s_)));
     RID_TRY(cuda(norm2_final(normp_, p_.nparts, st_, s_)));
@@ -594,8 +597,8 @@ class Engine {
     // once and the first read of the state ends the call
     if (p_.path == 33 && !p_.sparse) {  // digits of A's columns, once per call
       RID_TRY(tbegin(ID_PHASE_SKETCH));
-      RID_TRY(cuda(sketch_f32emu_slice((int)p_.n, (int)p_.m, reinterpret_cast<const float*>(Araw_), lda_, f32a_, p_.n,
-                                       f32ae_, nullptr, nullptr, s_)));
+      RID_TRY(cuda(sketch_f32emu_split(p_.n, (int)p_.m, reinterpret_cast<const float*>(Araw_), lda_, f32a_, p_.n,
+                                       f32ae_, s_)));
       RID_TRY(tend(1));
     }
     if (p_.sparse && sizeof(T) == 8) {  // FP64 A in 64-bit fixed point, once per call

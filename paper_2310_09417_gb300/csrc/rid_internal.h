@@ -89,7 +89,9 @@ cudaError_t gaussian_rows(uint64_t seed, int64_t row0, int64_t rows, int64_t m, 
 template <typename T>
 cudaError_t norm2_partial(int64_t m, int64_t n, const T* A, int64_t lda, double* part, int nparts,
                           DevState* st, cudaStream_t s);
-// FP64, and with `colexp` also every column's exponent E_j (max_i |A_ij| < 2^E_j).
+// With `colexp` also every column's exponent E_j (max_i |A_ij| < 2^E_j).
+cudaError_t norm2_f32(int64_t m, int64_t n, const float* A, int64_t lda, double* part, int nparts, int32_t* colexp,
+                      DevState* st, cudaStream_t s);
 cudaError_t norm2_f64(int64_t m, int64_t n, const double* A, int64_t lda, double* part, int nparts, int32_t* colexp,
                       DevState* st, cudaStream_t s);
 cudaError_t norm2_final(const double* part, int nparts, DevState* st, cudaStream_t s);
@@ -266,6 +268,8 @@ cudaError_t gemm_f64emu(int M, int N, int K, const double* A, int64_t lda, const
 // and W's digits.
 size_t sketch_f32emu_digit_bytes(int64_t rows, int64_t K);
 int sketch_f32emu_splits(int64_t m, int64_t n, int64_t unit_rows, int sms);
+cudaError_t sketch_f32emu_split(int64_t rows, int K, const float* src, int64_t lds, void* dig, int64_t rows_alloc,
+                                const int32_t* ex, cudaStream_t s);  // exponents known
 cudaError_t sketch_f32emu_slice(int rows, int K, const float* src, int64_t lds, void* dig, int64_t rows_alloc,
                                 int32_t* ex, unsigned long long* rowmax, const int32_t* done, cudaStream_t s);
 cudaError_t sketch_f32emu(int64_t m, int64_t n, int64_t rows, const void* adig, const int32_t* aexp, const void* wdig,

@@ -1,4 +1,5 @@
-// rid_norm.cu -- ||A||_F^2, finiteness, and for FP64 the column exponents, in one read of A.
+// rid_norm.cu -- ||A||_F^2, finiteness, and for the digit-sliced paths the column
+// exponents, in one read of A.
 //
 // One pass at HBM rate is the floor (A is read once, nothing is written).  GB300
 // issues about two FP64 instructions per clock per SM against 128 FP32 lanes, so
@@ -152,16 +153,34 @@ __global__ void __launch_bounds__(kNormThreads)
   put_part(acc + sum.value(), finite, part, st);
 }
 
+// The column's exponent e, max_i |A_ij| < 2^e (0 for a zero column), from the threads'
+// largest magnitudes; one barrier per column, the buffers alternate.
+__device__ __forceinline__ void put_colexp_f32(unsigned mx, unsigned (*s_mx)[kNormThreads / 32], int par, int32_t* out) {
+  const unsigned wm = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) s_mx[par][threadIdx.x >> 5] = wm;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  unsigned cm = 0u;
+#pragma unroll
+  for (int w = 0; w < kNormThreads / 32; ++w) cm = max(cm, s_mx[par][w]);
+  const int E = (int)(cm >> 23);
+  *out = cm == 0u ? 0 : (E == 0 ? -149 + (32 - __clz((int)cm)) : E - 126);
+}
+
 // FP32 columns of any alignment: the entries before a column's first 16-byte
-// boundary and after its last whole vector are added one by one.
+// boundary and after its last whole vector are added one by one.  With `colexp` also the
+// columns' exponents.
 __global__ void __launch_bounds__(kNormThreads)
-    k_norm2_f32(int64_t m, int64_t n, const float* __restrict__ A, int64_t lda, double* part, DevState* st) {
+    k_norm2_f32(int64_t m, int64_t n, const float* __restrict__ A, int64_t lda, double* part,
+                int32_t* __restrict__ colexp, DevState* st) {
   constexpr int U = 4;
+  __shared__ unsigned s_mx[2][kNormThreads / 32];
   double acc = 0.0;
   bool finite = true;
   SqSum sum;
   sum.clear();
-  int cnt = 0;
+  int cnt = 0, flip = 0;
+  unsigned col = 0u;  // largest magnitude of this thread's part of the column
   auto vec = [&](const float4& w) {
     const float x[4] = {w.x, w.y, w.z, w.w};
     uint32_t mx = 0u, mn = 0xFFFFFFFFu;
@@ -171,6 +190,7 @@ __global__ void __launch_bounds__(kNormThreads)
       mx = max(mx, u);
       mn = min(mn, u - 1u);
     }
+    col = max(col, mx);
     if (mx < kHighF32 && mn >= kLowF32) {
       sum.add_square(pack2(x[0], x[1]));
       sum.add_square(pack2(x[2], x[3]));
@@ -183,12 +203,17 @@ __global__ void __launch_bounds__(kNormThreads)
       cnt = 0;
     }
   };
+  auto one = [&](float x) {
+    col = max(col, __float_as_uint(x) & 0x7FFFFFFFu);
+    slow_square(x, acc, finite);
+  };
   for (int64_t j = blockIdx.x; j < n; j += gridDim.x) {
     const float* a = A + j * lda;
     int64_t head = (int64_t)((16u - (unsigned)(reinterpret_cast<uintptr_t>(a) & 15u)) & 15u) / 4;
     if (head > m) head = m;
     const int64_t nv = (m - head) / 4;
     const float4* a4 = reinterpret_cast<const float4*>(a + head);
+    col = 0u;
     int64_t v = threadIdx.x;
     for (; v + (U - 1) * kNormThreads < nv; v += U * kNormThreads) {
       float4 w[U];
@@ -198,9 +223,13 @@ __global__ void __launch_bounds__(kNormThreads)
       for (int u = 0; u < U; ++u) vec(w[u]);
     }
     for (; v < nv; v += kNormThreads) vec(__ldg(a4 + v));
-    if (threadIdx.x < head) slow_square(a[threadIdx.x], acc, finite);
+    if (threadIdx.x < head) one(a[threadIdx.x]);
     const int64_t i = head + 4 * nv + threadIdx.x;
-    if (i < m) slow_square(a[i], acc, finite);
+    if (i < m) one(a[i]);
+    if (colexp != nullptr) {
+      put_colexp_f32(col, s_mx, flip, colexp + j);
+      flip ^= 1;
+    }
   }
   put_part(acc + sum.value(), finite, part, st);
 }
@@ -351,7 +380,11 @@ __global__ void __launch_bounds__(kNormThreads)
 template <>
 cudaError_t norm2_partial<float>(int64_t m, int64_t n, const float* A, int64_t lda, double* part, int nparts,
                                  DevState* st, cudaStream_t s) {
-  k_norm2_f32<<<nparts, kNormThreads, 0, s>>>(m, n, A, lda, part, st);
+  return norm2_f32(m, n, A, lda, part, nparts, nullptr, st, s);
+}
+cudaError_t norm2_f32(int64_t m, int64_t n, const float* A, int64_t lda, double* part, int nparts, int32_t* colexp,
+                      DevState* st, cudaStream_t s) {
+  k_norm2_f32<<<nparts, kNormThreads, 0, s>>>(m, n, A, lda, part, colexp, st);
   return cudaGetLastError();
 }
 template <>
