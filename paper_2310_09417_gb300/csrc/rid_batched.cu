@@ -164,7 +164,7 @@ struct Squares {
     if constexpr (sizeof(T) == 4) {
       sq_add_f32(v, hi, lo, acc, finite);
       if (++cnt == 64) {
-        acc += (double)hi + (double)lo;
+        acc = sq_fold(acc, hi, lo);
         hi = lo = 0.f;
         cnt = 0;
       }

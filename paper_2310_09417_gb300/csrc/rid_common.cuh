@@ -178,22 +178,11 @@ __device__ __forceinline__ void sq_twosum(float t, float& hi, float& lo) {
   lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(t, bb)));
   hi = s;
 }
-// x given by its FP32 bit pattern (a BF16 value widened): squares of |x| in
-// [2^-63, 2^54) go to the float-float sum (below 2^108 each, so a group of 64 stays
-// finite), zeros are skipped, NaN / Inf clear `finite`, the rest (subnormal,
-// tiny or huge values) are added in FP64.
-__device__ __forceinline__ void sq_add_bits(uint32_t bits, float& hi, float& lo, double& acc, bool& finite) {
-  const uint32_t ex = (bits >> 23) & 0xFFu;
-  const float x = __uint_as_float(bits);
-  if (ex - 64u <= 116u) {
-    sq_twosum(__fmul_rn(x, x), hi, lo);
-  } else if ((bits << 1) == 0u) {
-  } else if (ex == 0xFFu) {
-    finite = false;
-  } else {
-    acc += (double)x * (double)x;
-  }
-}
+// The FP64 additions of these sums are functions of their own: as predicated
+// instructions, which the compiler makes of a short branch, they took GB300's FP64 pipe
+// for sixteen clocks per warp and element even when no lane needed them.
+static __device__ __noinline__ double sq_add_f64(double acc, float x) { return acc + (double)x * (double)x; }
+static __device__ __noinline__ double sq_fold(double acc, float hi, float lo) { return acc + ((double)hi + (double)lo); }
 
 // x^2 added to a float-float sum for an FP32 x: the square's rounding error comes
 // exactly from an FMA (TwoProduct) and the sum's from TwoSum; |x| outside
@@ -212,7 +201,7 @@ __device__ __forceinline__ void sq_add_f32(float x, float& hi, float& lo, double
   } else if (ex == 0xFFu) {
     finite = false;
   } else {
-    acc += (double)x * (double)x;
+    acc = sq_add_f64(acc, x);
   }
 }
 

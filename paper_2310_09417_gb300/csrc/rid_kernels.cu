@@ -581,7 +581,7 @@ __global__ void k_schur_finish(int na, int w, const int32_t* __restrict__ act, c
       if constexpr (sizeof(T) == 4) {
         sq_add_f32(v, hi, lo, acc2, finite);
         if (++grp == 64) {
-          acc2 += (double)hi + (double)lo;
+          acc2 = sq_fold(acc2, hi, lo);
           hi = lo = 0.f;
           grp = 0;
         }
