@@ -194,6 +194,15 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Results outside the normal range.  Functions of their own: inlined, their FP64
+// instructions became predicated ones, which hold GB300's FP64 pipe for sixteen clocks
+// per warp and value although no lane needs them.
+static __device__ __noinline__ double fixed_to_double_ends(long long hi, long long lo, int ex) {
+  return ldexp((double)hi + ldexp((double)lo, -32), ex + 32);
+}
+static __device__ __noinline__ double i64_to_double_ends(long long w, int ex) { return ldexp((double)w, ex); }
+static __device__ __noinline__ float i64_to_float_ends(long long w, int ex) { return ldexpf((float)w, ex); }
+
 // (hi 2^32 + lo) 2^ex as a double, rounded to nearest even, assembled with integer
 // operations (GB300 issues about two FP64 instructions per clock per SM).
 // hi, lo: any int64 values; results outside the normal range take the FP64 route.
@@ -221,7 +230,7 @@ __device__ __forceinline__ double fixed_to_double(long long hi, long long lo, in
     mant = (unsigned long long)(U << (-sh));
   }
   const int e = msb + ex + 1023;
-  if (e <= 0 || e >= 2047) return ldexp((double)hi + ldexp((double)lo, -32), ex + 32);
+  if (e <= 0 || e >= 2047) return fixed_to_double_ends(hi, lo, ex);
   return __longlong_as_double((long long)(((unsigned long long)neg << 63) | ((unsigned long long)e << 52) |
                                           (mant & ((1ull << 52) - 1))));
 }
@@ -238,7 +247,7 @@ __device__ __forceinline__ double i64_to_double(long long w, int ex) {
   const unsigned rem = (unsigned)(nrm & 0x7ffull);
   mant += (rem > 0x400u || (rem == 0x400u && (mant & 1ull))) ? 1ull : 0ull;
   const int e = 1023 + 63 - lz + ex;  // biased exponent of the leading one
-  if (e <= 0 || e >= 2046) return ldexp((double)w, ex);
+  if (e <= 0 || e >= 2046) return i64_to_double_ends(w, ex);
   // the leading one (bit 52 of mant) adds 1 to the field; a carry to 2^53 adds one more
   return __longlong_as_double((long long)(sgn | (((unsigned long long)(e - 1) << 52) + mant)));
 }
@@ -256,7 +265,7 @@ __device__ __forceinline__ float i64_to_float(long long w, int ex) {
   const unsigned long long half = 1ull << 39;
   mant += (rem > half || (rem == half && (mant & 1u))) ? 1u : 0u;
   const int e = 127 + 63 - lz + ex;  // biased exponent of the leading one
-  if (e <= 0 || e >= 254) return ldexpf((float)w, ex);
+  if (e <= 0 || e >= 254) return i64_to_float_ends(w, ex);
   return __uint_as_float(sgn | (((unsigned)(e - 1) << 23) + mant));
 }
 
