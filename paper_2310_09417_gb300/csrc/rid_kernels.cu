@@ -662,8 +662,12 @@ cudaError_t decide(const double* e2part, int nparts, int w, double tol, int tol_
 // A step has two block barriers.  Two word buffers alternate between steps: a block
 // stores step c+2's words only after it has seen every block's word of step c+1,
 // and each block stored that after it had read step c's.
-// Measured on GB300 per pivot (w = 64): FP64 3.1 us (n = 10000; 4.2 with a
-// counter barrier and atomic keys), FP32 2.0 us (n = 3000; 2.9) and 2.3 us (n = 20000; 3.6).
+// FP64 that few threads need stays out of predicated code (a predicated-off FP64
+// instruction takes its issue slot all the same): the record of a pivot is a call by a
+// thread of a warp that does not poll, and the update leaves its loop at the last column.
+// Measured on GB300 per pivot (w = 64, a first panel): FP64 2.8 us (n = 10000; 4.2 with a
+// counter barrier and atomic keys), mean over a 4096-column factorization 2.54 us (2.65
+// with the predicated code); FP32 2.0 us (n = 3000; 2.9) and 2.3 us (n = 20000; 3.6).
 constexpr int kPanelThreads = 256;
 constexpr int kPanelMaxW = 128;
 constexpr int kPanelPoll = 5;  // candidates a lane of the polling warp reads at once
@@ -740,6 +744,15 @@ __device__ __forceinline__ double divide_by(double a, double b, double r, bool o
 }
 __device__ __forceinline__ bool recip_usable(float) { return false; }
 __device__ __forceinline__ float divide_by(float a, float b, float, bool) { return a / b; }
+
+// Block 0's record of a pivot (a call: its FP64 conversion is not to be predicated code
+// of every warp).
+template <typename T>
+__device__ __noinline__ void record_pivot(int c, int gi, T pv, int32_t* piv, double* pivdiag, DevState* st) {
+  piv[c] = gi;
+  if (pivdiag != nullptr) pivdiag[c] = (double)tabs(pv);
+  if (pv == T(0)) atomicAdd(&st->zero_pivots, 1u);
+}
 
 template <typename T>
 __global__ void __launch_bounds__(kPanelThreads)
@@ -1033,12 +1046,8 @@ __global__ void __launch_bounds__(kPanelThreads)
       }
       if (more) warp_cand(have, mag, brow);
     }
-    if (bid == 0 && tid == 0) {
-      piv[c] = gi;
-      if (pivdiag != nullptr) pivdiag[c] = (double)tabs(pv);
-      if (pv == T(0)) atomicAdd(&st->zero_pivots, 1u);
-    }
     __syncthreads();
+    if (bid == 0 && tid == kPanelThreads - 1) record_pivot<T>(c, gi, pv, piv, pivdiag, st);
     // 3. warp 0 completes the candidate's row and publishes it
     int cand = -1;
     if (more) {
@@ -1077,6 +1086,7 @@ __global__ void __launch_bounds__(kPanelThreads)
 #pragma unroll
         for (int j = 0; j < kPanelMaxW / 32; ++j) {
           const int cc = cfirst + lane + 32 * j;
+          if (cfirst + 32 * j >= w) break;  // uniform: no FP64 issue for columns that are done
           if (cc < w) {
             T x[4];
 #pragma unroll
@@ -1193,6 +1203,9 @@ cudaError_t panel_lupp(const PanelCfg& cfg, int na, int w, int steps, unsigned s
 // Row i moves up by the number of pivot rows before it, counted against the sorted
 // pivots in shared memory, so the list needs no scan over its length: one CTA's scan took
 // 14 us of a round at n = 10000 and 27 at 20000; beside the inverse it takes none.
+// The inverse is bound by its chain of bt steps: per step one barrier and one FMA, into a
+// partial sum that the unrolled loop names (as a choice at run time it was four predicated
+// FMAs).  bt = 64: FP64 20.9 -> 18.9 us, FP32 8.8 -> 7.1 us.
 constexpr int kLinvLoadThreads = 256;
 constexpr int kCompactRows = 1024;  // rows of the active list per CTA
 
@@ -1257,20 +1270,17 @@ __global__ void __launch_bounds__(1024)
     for (int u = 0; u < 8; ++u)
       if (e0 + u * nt < bt * bt) Lp[e0 + u * nt] = v[u];
   }
-  T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
+  T s[4] = {T(0), T(0), T(0), T(0)};
   __syncthreads();
-  for (int c = j; c < bt; ++c) {
-    if (i == c) xs[c] = c == j ? T(1) : -((s0 + s1) + (s2 + s3));
-    __syncthreads();
-    if (i > c && i < bt) {
-      const T l = Lp[i * bt + c], x = xs[c];
-      const int p = (c - j) & 3;
-      if (p == 0) s0 = fma(l, x, s0);
-      else if (p == 1) s1 = fma(l, x, s1);
-      else if (p == 2) s2 = fma(l, x, s2);
-      else s3 = fma(l, x, s3);
+  for (int c0 = j; c0 < bt; c0 += 4)
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {  // the partial is known here: one FMA, not four predicated ones
+      const int c = c0 + p;
+      if (c >= bt) break;
+      if (i == c) xs[c] = c == j ? T(1) : -((s[0] + s[1]) + (s[2] + s[3]));
+      __syncthreads();
+      if (i > c && i < bt) s[p] = fma(Lp[i * bt + c], xs[c], s[p]);
     }
-  }
   if (i < bt) Linv[i * bt + j] = i < j ? T(0) : xs[i];  // xs[i] was written by this thread
 }
 
