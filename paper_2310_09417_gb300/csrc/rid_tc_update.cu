@@ -31,14 +31,21 @@
 //             accumulator sets let a tile's MMAs run during the last tile's epilogue
 //   warps 2-17 epilogue: four warps per lane quarter, 16 columns each; the
 //             accumulators are read with one row per lane and released before
-//             the stores, T is read (before the accumulators are ready) and
-//             written coalesced, the products passing through shared memory
+//             the stores, T is read (two tiles ahead) and written coalesced, the
+//             products passing through shared memory
+//
+// What bounds it: the epilogue -- its instructions and T's traffic in runs of 128 or 256
+// bytes per row.  n = 20000 FP32, mean over 37 rounds to 2368 columns: 79 us with 64-bit
+// divisions per tile and an int64 fold, 67 us (2.8 TB/s of T) with counters, the fold in
+// 32 bits and T read two tiles ahead; n = 10000 FP64: 83 -> 78 us.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "rid_internal.h"
 #include "rid_tc_common.cuh"
@@ -85,45 +92,55 @@ static_assert(2 * set_cols<7>() <= 512 && 2 * set_cols<3>() <= 512, "two accumul
 
 // The folded accumulators of 8 columns of this lane's row; group g of the set
 // starts at column g * bn.
-template <int KD>
+// KD = 7: int64 sums; the loads come in batches, one wait per batch (groups 0-3, then 4-6).
 __device__ __forceinline__ void fold8(uint32_t taddr, long long* w) {
-  constexpr int kG = bn<KD>();
-  // loads issued in batches, one wait per batch (KD = 7: groups 0-3, then 4-6)
+  constexpr int kG = bn<7>();
   uint32_t r[4][8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) w[i] = 0;
-  if constexpr (KD == 7) {
+  for (int g = 0; g < 4; ++g) tmem_ld8_nowait(taddr + g * kG, r[g]);
+  tmem_wait_ld();
 #pragma unroll
-    for (int g = 0; g < 4; ++g) tmem_ld8_nowait(taddr + g * kG, r[g]);
-    tmem_wait_ld();
+  for (int i = 0; i < 8; ++i) {
+    w[i] = 0;
+    add_scaled<16>(w[i], __uint_as_float(r[0][i]));
+    add_scaled<8>(w[i], __uint_as_float(r[1][i]));
+    add_scaled<0>(w[i], __uint_as_float(r[2][i]));
+    w[i] <<= 24;  // |w| < 2^37 before the shift
+    add_scaled<16>(w[i], __uint_as_float(r[3][i]));
+  }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      add_scaled<16>(w[i], __uint_as_float(r[0][i]));
-      add_scaled<8>(w[i], __uint_as_float(r[1][i]));
-      add_scaled<0>(w[i], __uint_as_float(r[2][i]));
-      w[i] <<= 24;  // |w| < 2^37 before the shift
-      add_scaled<16>(w[i], __uint_as_float(r[3][i]));
-    }
+  for (int g = 0; g < 3; ++g) tmem_ld8_nowait(taddr + (4 + g) * kG, r[g]);
+  tmem_wait_ld();
 #pragma unroll
-    for (int g = 0; g < 3; ++g) tmem_ld8_nowait(taddr + (4 + g) * kG, r[g]);
-    tmem_wait_ld();
+  for (int i = 0; i < 8; ++i) {
+    add_scaled<8>(w[i], __uint_as_float(r[0][i]));
+    add_scaled<0>(w[i], __uint_as_float(r[1][i]));
+    w[i] += __float2int_rn(__uint_as_float(r[2][i]) * 0x1.0p-8f);
+  }
+}
+// KD = 3: W = G_0 2^16 + G_1 2^8 + G_2, rounded once to FP32, in 32-bit integers.  The
+// groups (|G_g| <= (g + 1) 2^20) become integers by one addition each: 1.5 2^23 + G is
+// exact for |G| <= 2^22.  a = 2^8 G_0 + G_1 (|a| < 2^29); W = 2^8 a + G_2 = 2^23 h + l with
+// h = (a + (G_2 >> 8)) >> 15 (|h| < 2^15) and l the low 23 bits of W, which the low 32 bits
+// hold.  h and l become floats the same way; fma(h, 2^23, l) is the exact sum rounded once.
+__device__ __forceinline__ void fold8(uint32_t taddr, float* w) {
+  constexpr int kG = bn<3>();
+  constexpr float kMagic = 12582912.0f;  // 1.5 2^23, pattern 0x4B400000
+  uint32_t r[3][8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      add_scaled<8>(w[i], __uint_as_float(r[0][i]));
-      add_scaled<0>(w[i], __uint_as_float(r[1][i]));
-      w[i] += __float2int_rn(__uint_as_float(r[2][i]) * 0x1.0p-8f);
-    }
-  } else {
-    static_assert(KD == 3, "KD is 7 or 3");
+  for (int g = 0; g < 3; ++g) tmem_ld8_nowait(taddr + g * kG, r[g]);
+  tmem_wait_ld();
 #pragma unroll
-    for (int g = 0; g < 3; ++g) tmem_ld8_nowait(taddr + g * kG, r[g]);
-    tmem_wait_ld();
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      add_scaled<16>(w[i], __uint_as_float(r[0][i]));
-      add_scaled<8>(w[i], __uint_as_float(r[1][i]));
-      add_scaled<0>(w[i], __uint_as_float(r[2][i]));
-    }
+  for (int i = 0; i < 8; ++i) {
+    const int g0 = __float_as_int(__uint_as_float(r[0][i]) + kMagic) - 0x4B400000;
+    const int g1 = __float_as_int(__uint_as_float(r[1][i]) + kMagic) - 0x4B400000;
+    const int g2 = __float_as_int(__uint_as_float(r[2][i]) + kMagic) - 0x4B400000;
+    const int a = g0 * 256 + g1;
+    const int h = (a + (g2 >> 8)) >> 15;
+    const int l = (int)((unsigned)a * 256u + (unsigned)g2) & 0x7FFFFF;
+    const float fh = __int_as_float(0x4B400000 + h) - kMagic;
+    const float fl = __int_as_float(0x4B000000 | l) - 8388608.0f;  // 2^23 + l, 0 <= l < 2^23
+    w[i] = fmaf(fh, 8388608.0f, fl);
   }
 }
 // unit of the fold: 2^(e_i + f_c + fold_exp)
@@ -131,21 +148,15 @@ template <int KD>
 __host__ __device__ constexpr int fold_exp() {
   return KD == 7 ? 2 - 56 : 2 - 32;
 }
-__device__ __forceinline__ double fold_value(long long w, int ex, double) { return i64_to_double(w, ex); }
-// |w| < 2^38, rounded once to FP32 without the 64-bit conversion instruction (it
-// runs on GB300's FP64 pipe, about two per clock per SM): w = 2^23 h + l with
-// 0 <= l < 2^23 and |h| < 2^15, both made exact floats by magic-number additions,
-// then fma(h, 2^23, l) -- the exact sum rounded once, as the conversion would.  The
-// power-of-two scale is exact for normal results.
-__device__ __forceinline__ float fold_value(long long w, int ex, float) {
-  const int h = (int)(w >> 23);
-  const int l = (int)(w - ((long long)h << 23));
-  const float fh = __int_as_float(0x4B400000 + h) - 12582912.0f;  // 1.5 * 2^23 + h, |h| < 2^22
-  const float fl = __int_as_float(0x4B000000 | l) - 8388608.0f;   // 2^23 + l, 0 <= l < 2^23
-  const float f = fmaf(fh, 8388608.0f, fl);
-  if (ex >= -126 && ex <= 127) return f * __int_as_float((ex + 127) << 23);
-  return ldexpf(f, ex);
+__device__ __noinline__ float scale_ends(float f, int ex) { return ldexpf(f, ex); }
+__device__ __forceinline__ double fold_value(long long w, int ex) { return i64_to_double(w, ex); }
+// The power-of-two scale is exact for normal results.
+__device__ __forceinline__ float fold_value(float w, int ex) {
+  if (ex >= -126 && ex <= 127) return w * __int_as_float((ex + 127) << 23);
+  return scale_ends(w, ex);
 }
+template <int KD>
+using fold_t = std::conditional_t<KD == 7, long long, float>;
 
 // Tiles (row tile, column tile) in row-major order are split into one contiguous,
 // balanced range per CTA (one CTA per SM): a range spans few row tiles, whose N
@@ -171,6 +182,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int64_t total = (int64_t)rt * ct;
   const int64_t t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
   const int my = (int)(t1 - t0);
+  // first tile; the roles step through theirs by counting (a 64-bit division per tile and
+  // thread cost the epilogue as much as its arithmetic)
+  int row = (int)(t0 / ct), col = (int)(t0 % ct);
+  auto next_tile = [&] {
+    if (++col == ct) {
+      col = 0;
+      ++row;
+    }
+  };
 
   if (threadIdx.x == 0) {
     mbar_init(&sm.n_full, 1);
@@ -194,8 +214,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     int issued = 0, cur = -1, segs = 0;
     bool ok = true;
     for (int u = 0; u < my && ok; ++u) {
-      const int64_t t = t0 + u;
-      const int row = (int)(t / ct), col = (int)(t % ct);
       const int b = u & 1;
       if (row != cur) {
         // N's tile is free once the MMAs of tile u - 1 (and all before) completed
@@ -212,15 +230,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_expect_tx(&sm.p_full[b], kD * kBN * kK * 2);
       for (int q = 0; q < kD; ++q) tma_load_3d(sm.p[b][q], &map_p, &sm.p_full[b], 0, col * kBN, q);
       issued = u + 1;
+      next_tile();
     }
     for (int u = issued - 2 < 0 ? 0 : issued - 2; u < issued; ++u) mbar_wait_drain(&sm.p_full[u & 1], (u >> 1) & 1);
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer: per K step and slice s of N, one MMA against P's
     // planes 0 .. KD-1-s stacked along N writes groups s .. KD-1 at once
     int cur = -1, segs = 0;
-    for (int u = 0; u < my; ++u) {
-      const int64_t t = t0 + u;
-      const int row = (int)(t / ct);
+    for (int u = 0; u < my; ++u, next_tile()) {
       const int b = u & 1;
       if (row != cur) {
         cur = row;
@@ -265,50 +282,42 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       cur = row;
     };
-    // T's entries and the column exponents of tile u + 1 are loaded while tile u is
-    // processed when both lie in the same row tile
-    TX xn[kHalves][8];
-    int pn = 0;
-    auto fetch = [&](int col) {
+    // T's entries and the column exponents of the tiles ahead, within the row tile: two
+    // register sets, tile u's filled again for tile u + 2 as soon as it is used.
+    TX xa[kHalves][8], xb[kHalves][8];
+    int pa = 0, pb = 0;
+    bool ha = false, hb = false;  // the set holds the tile it is used for next
+    auto fetch = [&](TX(&x)[kHalves][8], int& pe, int col) {
       const int c0 = col * kBN + part * kCols;
-      pn = (lane < kCols && c0 + lane < tb) ? pexp[c0 + lane] : 0;
+      pe = (lane < kCols && c0 + lane < tb) ? pexp[c0 + lane] : 0;
 #pragma unroll
       for (int h = 0; h < kHalves; ++h)
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int c = c0 + 8 * h + jc;
           TX* const rp = rowp[4 * i];
-          xn[h][i] = (rp != nullptr && c < tb) ? rp[c] : TX(0);
+          x[h][i] = (rp != nullptr && c < tb) ? rp[c] : TX(0);
         }
     };
-    bool have = false;  // xn / pn hold tile u
-    for (int u = 0; u < my; ++u) {
-      const int64_t t = t0 + u;
-      const int row = (int)(t / ct), col = (int)(t % ct);
+    // tile u with the set (x, pe, have); the other set is tile u + 1's
+    auto tile = [&](int u, TX(&x)[kHalves][8], int& pe, bool& have, TX(&x1)[kHalves][8], int& pe1, bool& have1) {
       const int b = u & 1;
       if (row != cur) {
         enter_row(row);
-        have = false;
+        have = have1 = false;
       }
-      if (!have) fetch(col);
+      if (!have) fetch(x, pe, col);
+      if (!have1 && u + 1 < my && col + 1 < ct) {
+        fetch(x1, pe1, col + 1);
+        have1 = true;
+      }
       const int c0 = col * kBN + part * kCols;
-      TX xv[kHalves][8];
-#pragma unroll
-      for (int h = 0; h < kHalves; ++h)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) xv[h][i] = xn[h][i];
-      const int pe = pn;  // lane j < kCols: the exponent of column c0 + j
-      have = false;
-      if (u + 1 < my && (t + 1) / ct == row) {
-        fetch((int)((t + 1) % ct));
-        have = true;
-      }
-      if (!mbar_wait(&sm.t_full[b], (u >> 1) & 1, st)) break;
+      if (!mbar_wait(&sm.t_full[b], (u >> 1) & 1, st)) return false;
       fence_after_sync();
 #pragma unroll
       for (int h = 0; h < kHalves; ++h) {
-        long long w[8];
-        fold8<KD>(lane_base + b * kSet + 8 * h, w);
+        fold_t<KD> w[8];
+        fold8(lane_base + b * kSet + 8 * h, w);
         if (h == kHalves - 1) {
           // this accumulator set is free for tile u + 2
           fence_before_sync();
@@ -317,18 +326,26 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-          const int ec = __shfl_sync(0xffffffffu, pe, 8 * h + j);
-          stage[lane][j] = fold_value(w[j], er + ec + fold_exp<KD>(), TX(0));
+          const int ec = __shfl_sync(0xffffffffu, pe, 8 * h + j);  // lane j < kCols: column c0 + j
+          stage[lane][j] = fold_value(w[j], er + ec + fold_exp<KD>());
         }
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int c = c0 + 8 * h + jc;
           TX* const rp = rowp[4 * i];
-          if (rp != nullptr && c < tb) rp[c] = xv[h][i] - stage[4 * i + (lane >> 3)][jc];
+          if (rp != nullptr && c < tb) rp[c] = x[h][i] - stage[4 * i + (lane >> 3)][jc];
         }
         __syncwarp();
       }
+      have = u + 2 < my && col + 2 < ct;
+      if (have) fetch(x, pe, col + 2);
+      next_tile();
+      return true;
+    };
+    for (int u = 0; u < my; u += 2) {
+      if (!tile(u, xa, pa, ha, xb, pb, hb)) break;
+      if (u + 1 < my && !tile(u + 1, xb, pb, hb, xa, pa, ha)) break;
     }
   }
   fence_before_sync();
