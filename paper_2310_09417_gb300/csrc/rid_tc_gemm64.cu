@@ -321,7 +321,7 @@ __global__ void k_slice_rows(int M, int K, int Kq, int64_t Kp, const T* __restri
     for (int k = 4 * lane; k < Kq; k += 128) {  // Kq is a multiple of 64
       T v[4];
       load4(row + k, K - k, vec, v);
-      long long F[4];
+      decltype(fixed_of<KD>(T(0), 0)) F[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) F[q] = fixed_of<KD>(v[q], e);  // zero past K
       write_digits4<KD>(F, D + r * Kp + k, plane);
@@ -331,7 +331,8 @@ __global__ void k_slice_rows(int M, int K, int Kq, int64_t Kp, const T* __restri
 
 // The digits of rows whose exponents are known: every 1024 entries of a row are one
 // CTA's work, in one read.  With the exponents from the norm's pass over A the second
-// read of each row went away (1.57 -> 1.17 ms for 40000 x 10000).
+// read of each row went away (1.57 -> 1.17 ms for 40000 x 10000; 0.67 since the digits are
+// cheap).
 constexpr int kSplitSeg = 1024;
 template <typename T, int KD>
 __global__ void __launch_bounds__(kSplitSeg / 4)
@@ -347,7 +348,7 @@ __global__ void __launch_bounds__(kSplitSeg / 4)
     T v[4];
     load4(row + k, K - k, (reinterpret_cast<uintptr_t>(row) & 15u) == 0u, v);
     const int e = ex[r];
-    long long F[4];
+    decltype(fixed_of<KD>(T(0), 0)) F[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) F[q] = fixed_of<KD>(v[q], e);
     write_digits4<KD>(F, D + r * Kp + k, plane);
@@ -376,7 +377,7 @@ __global__ void k_rows_digits(int M, int K, int Kq, int64_t Kp, const T* __restr
   const int e = exp_above(rowmax[r], T(0));
   if (blockIdx.x == 0 && threadIdx.x == 0) ex[r] = e;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < Kq; k += (int64_t)gridDim.x * blockDim.x)
-    write_digits<KD>(k < K ? fixed_of<KD>(src[(int64_t)r * lds + k], e) : 0ll, D + (int64_t)r * Kp + k, plane);
+    write_digits<KD>(k < K ? fixed_of<KD>(src[(int64_t)r * lds + k], e) : 0, D + (int64_t)r * Kp + k, plane);
 }
 
 // B (K x N): element (k, n) = src[idx[k] * lds + off + n].  First the largest
@@ -423,7 +424,7 @@ __global__ void k_col_digits(int K, int N, int Kp, const T* __restrict__ src, in
     const int k = k0 + kl;
     if (n < N && k < Kp) {
       const int en = exp_above(colmax[n], T(0));
-      write_digits<KD>(k < K ? fixed_of<KD>(tile[kl][n], en) : 0ll, D + (int64_t)n * Kp + k, plane);
+      write_digits<KD>(k < K ? fixed_of<KD>(tile[kl][n], en) : 0, D + (int64_t)n * Kp + k, plane);
       if (blockIdx.x == 0 && kl == 0) ex[n] = en;
     }
   }
