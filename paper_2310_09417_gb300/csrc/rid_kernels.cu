@@ -528,7 +528,10 @@ cudaError_t gemm_gather<float>(int M, int N, int K, int splits, bool b_kmajor, O
 
 // ============================================================ split-K reductions
 // Threads over the rows of a row-block (x), rows of G over y and the grid: no
-// 64-bit division per element; the partials are summed in split order.
+// 64-bit division per element; the partials are summed in split order, eight loads in
+// flight.  FP64 adds bound the FP64 form (40 partials of 10000 x 128: 81 us of adds;
+// 113 -> 97 us), the loads the FP32 form (10000 x 256, 49.6 -> 35 us).
+constexpr int kReduceAhead = 8;
 template <typename T>
 __global__ void k_splitk_reduce(int64_t n, int rows, int64_t ldp, int64_t ldg, int nz, int64_t zs,
                                 const T* __restrict__ P, T* __restrict__ G, const int32_t* done) {
@@ -537,7 +540,15 @@ __global__ void k_splitk_reduce(int64_t n, int rows, int64_t ldp, int64_t ldg, i
     for (int c = threadIdx.x; c < rows; c += blockDim.x) {
       const int64_t off = j * ldp + c;
       T acc = P[off];
-      for (int z = 1; z < nz; ++z) acc += P[z * zs + off];
+      int z = 1;
+      for (; z + kReduceAhead <= nz; z += kReduceAhead) {  // loads in flight together, sums in order
+        T v[kReduceAhead];
+#pragma unroll
+        for (int u = 0; u < kReduceAhead; ++u) v[u] = P[(z + u) * zs + off];
+#pragma unroll
+        for (int u = 0; u < kReduceAhead; ++u) acc += v[u];
+      }
+      for (; z < nz; ++z) acc += P[z * zs + off];
       G[j * ldg + c] = acc;
     }
 }
