@@ -70,7 +70,7 @@ struct Smem {
 // out: FP32 partial (n x rows, row stride out_ld) of split blockIdx.z.  Every entry
 // gets the same sums (block sums in K order, scaled and added in block order)
 // whatever NT is.
-template <int NT>
+template <int NT, bool kRagged>
 __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
     k_sketch_tc_fp8(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                     const float* __restrict__ scale, int64_t nbs, int n, int rows, int K, int kchunk,
@@ -82,9 +82,11 @@ __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kBM;
   const int n0 = blockIdx.y * C::kCols;
-  // the last group of rows may hold fewer blocks than the tile: only their columns are
-  // multiplied and drained (576 rows on 256-row tiles, 50001 x 12003: 0.73 -> 0.71 ms)
-  const int ncols = min(C::kCols, (rows - n0 + 31) / 32 * 32);
+  // kRagged: the last group of rows holds fewer blocks than the tile; only their columns
+  // are multiplied and drained (576 rows on 256-row tiles, 50001 x 12003: 0.73 -> 0.71 ms).
+  // Whole groups keep the fixed width: the test per 32 columns took 5 % of a pass of 512
+  // rows at 100000 x 20000.
+  const int ncols = kRagged ? min(C::kCols, (rows - n0 + 31) / 32 * 32) : C::kCols;
   const int kbeg = blockIdx.z * kchunk;
   const int kend = min(K, kbeg + kchunk);
   const int nkb = (kend - kbeg + kBK - 1) / kBK;
@@ -160,13 +162,21 @@ __global__ void __launch_bounds__(Cfg<NT>::kThreads, Cfg<NT>::kMinBlocks)
         break;
       }
       fence_after_sync();
-#pragma unroll
-      for (int cb = 0; cb < C::kWarpCols; cb += 32) {  // 32 columns per wait on tensor memory
-        if (col0 + cb >= ncols) break;
+      auto drain = [&](int cb) {  // 32 columns per wait on tensor memory
         float v[32];
         tmem_ld32(lane_base + a * C::kCols + cb, v);
 #pragma unroll
         for (int i = 0; i < 32; ++i) acc[cb + i] = fmaf(v[i], s_kb, acc[cb + i]);
+      };
+      if (!kRagged || ncols == C::kCols) {
+#pragma unroll
+        for (int cb = 0; cb < C::kWarpCols; cb += 32) drain(cb);
+      } else {
+#pragma unroll
+        for (int cb = 0; cb < C::kWarpCols; cb += 32) {
+          if (col0 + cb >= ncols) break;
+          drain(cb);
+        }
       }
       fence_before_sync();
       __syncwarp();
@@ -277,21 +287,29 @@ int tc_fp8_effective_splits(int64_t m, int splits) {
   return (int)((m + kchunk - 1) / kchunk);
 }
 
-template <int NT>
-static cudaError_t launch_fp8(const CUtensorMap& ma, const CUtensorMap& mw, const float* scale, int64_t nbs,
+template <int NT, bool kRagged>
+static cudaError_t launch_fp8_groups(const CUtensorMap& ma, const CUtensorMap& mw, const float* scale, int64_t nbs,
                               int64_t m, int64_t n, int64_t rows, int64_t kchunk, int nz, float* out, int64_t out_ld,
                               int64_t zstride, DevState* st, const int32_t* done, cudaStream_t s) {
   static_assert(sizeof(tc8::Smem<NT>) + 1024 <= 232448, "shared memory of k_sketch_tc_fp8 exceeds 227 KB");
   const size_t smem = sizeof(tc8::Smem<NT>) + 1024;
   static SmemLimit lim;
-  cudaError_t e = raise_smem(tc8::k_sketch_tc_fp8<NT>, smem, lim);
+  cudaError_t e = raise_smem(tc8::k_sketch_tc_fp8<NT, kRagged>, smem, lim);
   if (e != cudaSuccess) return e;
   const int64_t ytiles = (rows + tc8::Cfg<NT>::kCols - 1) / tc8::Cfg<NT>::kCols;
   if (ytiles > 65535 || nz > 65535) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((n + tc8::kBM - 1) / tc8::kBM), (unsigned)ytiles, (unsigned)nz);
-  tc8::k_sketch_tc_fp8<NT><<<grid, tc8::Cfg<NT>::kThreads, smem, s>>>(ma, mw, scale, nbs, (int)n, (int)rows, (int)m,
-                                                                     (int)kchunk, out, out_ld, zstride, st, done);
+  tc8::k_sketch_tc_fp8<NT, kRagged><<<grid, tc8::Cfg<NT>::kThreads, smem, s>>>(
+      ma, mw, scale, nbs, (int)n, (int)rows, (int)m, (int)kchunk, out, out_ld, zstride, st, done);
   return cudaGetLastError();
+}
+
+template <int NT>
+static cudaError_t launch_fp8(const CUtensorMap& ma, const CUtensorMap& mw, const float* scale, int64_t nbs,
+                              int64_t m, int64_t n, int64_t rows, int64_t kchunk, int nz, float* out, int64_t out_ld,
+                              int64_t zstride, DevState* st, const int32_t* done, cudaStream_t s) {
+  const auto f = rows % tc8::Cfg<NT>::kCols ? launch_fp8_groups<NT, true> : launch_fp8_groups<NT, false>;
+  return f(ma, mw, scale, nbs, m, n, rows, kchunk, nz, out, out_ld, zstride, st, done, s);
 }
 
 cudaError_t tc_sketch_fp8(const void* A, int64_t lda, int64_t m, int64_t n, const float* scale, const void* W,
