@@ -440,7 +440,10 @@ class Engine {
         RID_TRY(decide(b, tb, last, (int)(t - 1)));
         if (ahead) {
           RID_TRY(post_state(t));
-          if (t > 1 || last) RID_TRY(read_state(last ? t : t - 1));
+          // at the cap also this round's decision, after the one before: read alone it
+          // would hold the earlier stop together with what was queued past it
+          if (t > 1) RID_TRY(read_state(t - 1));
+          if (last && !(h_.err || h_.done)) RID_TRY(read_state(t));
         } else {
           RID_TRY(sync_state());
         }
