@@ -246,14 +246,6 @@ cudaError_t update_f64emu(int na, int bt, int tb, const double* N, const int32_t
 // kmax) bytes, aexp / bexp arows / brows exponents, colmax N words.
 int64_t gemm_f64emu_kpad(int64_t K);
 size_t gemm_f64emu_digit_bytes(int64_t rows, int64_t Kmax);
-// out[z] (M x N, row stride ldo) = split z of A^T B, A (K x M) and B (K x N) column-major,
-// FP64 accurate on the tensor cores; ws: gemm_f64emu_tn_bytes(), 256-byte aligned.  A
-// column with NaN or Inf gives NaN in its row (of B: its column) of the result.
-size_t gemm_f64emu_tn_bytes(int64_t M, int64_t N, int64_t K);
-int gemm_f64emu_tn_splits(int64_t M, int64_t N, int64_t K, int sms);
-cudaError_t gemm_f64emu_tn(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B, int64_t ldb,
-                           void* ws, double* out, int64_t ldo, int64_t zstride, int splits, DevState* st,
-                           cudaStream_t s);
 int gemm_f64emu_splits(int64_t M, int64_t N, int64_t K, int sms);
 cudaError_t gemm_f64emu(int M, int N, int K, const double* A, int64_t lda, const int32_t* aidx, const double* B,
                         int64_t ldb, int64_t boff, const int32_t* bidx, void* adig, int64_t arows, int32_t* aexp,

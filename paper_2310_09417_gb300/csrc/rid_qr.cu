@@ -584,68 +584,28 @@ cudaError_t tri_solve(int64_t k, const T* F, int64_t ld, T* B, int64_t ldb, int6
   return e;
 }
 
-// M (k x n, row-major) = Q^T A for Q (m x k) and A (m x n), both column-major.  FP64 with
-// enough work goes to the tensor cores by exact digit slicing (rid_tc_gemm64.cu): the FP64
-// pipe runs the product at its 1.2 TFLOP/s, 1.36 ms for 4000 x 2000 and k = 96 against
-// 0.23 with the slicing, and the result is as near the 64-bit values (CUR factors and
-// stable X of that matrix: 9.1e-14 with either).  Narrow or short products, where the
-// slicing costs what it saves, and those whose digits (14 bytes per element of A) would
-// not leave room on the card, stay on the FP64 pipe, as FP32 does on its own units.
-struct QtaPlan {
-  bool tc = false;
-  int splits = 1;
-  size_t part = 0, dig = 0, total = 0;  // split-K partials (and the transposed sum), digit slices
-};
+// out (M x N, row-major, ldo) = A^T B for A (K x M) and B (K x N), both column-major
+// (columns contiguous along K): split-K partials in P, then their sum.
+// FP64 stays on the FP64 pipe, which bounds Q^T A (4000 x 2000, k = 96: 1.36 ms).  The
+// tensor cores by digit slicing take 0.23 ms, but a sliced column holds 55 bits below its
+// largest entry, not below each entry: with rows in two units 2^27 apart the block of X in
+// the smaller unit came out 1e-9 off where the FP64 product leaves 1e-15.
 template <typename T>
-QtaPlan qta_plan(int64_t m, int64_t n, int64_t k, int sms) {
-  QtaPlan p;
-  const size_t dig = gemm_f64emu_tn_bytes(n, k, m);
-  p.tc = sizeof(T) == 8 && k >= 16 && (double)m * n * k >= 16e6 && dig <= ((size_t)16 << 30) && n < (1 << 30) &&
-         cdv(n, 128) <= 65535;
-  if (p.tc) {
-    p.splits = gemm_f64emu_tn_splits(n, k, m, sms);
-    p.part = al((size_t)(p.splits + 1) * n * k * sizeof(T));
-    p.dig = dig;
-  } else {
-    p.splits = qr_splits<T>(k, n, m, sms);
-    p.part = al(p.splits > 1 ? (size_t)p.splits * k * n * sizeof(T) : 1);
-  }
-  p.total = p.part + al(p.dig);
-  return p;
-}
-
-template <typename T>
-cudaError_t qta(int64_t m, int64_t n, int64_t k, const T* Q, int64_t ldq, const T* A, int64_t lda, T* M, const QtaPlan& p,
-                unsigned char* ws, DevState* st, cudaStream_t s) {
-  T* P = reinterpret_cast<T*>(ws);
-  cudaError_t e;
-  if constexpr (sizeof(T) == 8) {
-    if (p.tc) {  // A^T Q (n x k) in split-K partials, their sum, its transpose
-      e = gemm_f64emu_tn(n, k, m, A, lda, Q, ldq, ws + p.part, P, k, n * k, p.splits, st, s);
-      T* sum = p.splits > 1 ? P + (int64_t)p.splits * n * k : P;
-      if (e == cudaSuccess && p.splits > 1)
-        e = splitk_reduce_ld<T>(n, (int)k, k, k, p.splits, n * k, P, sum, nullptr, s);
-      if (e == cudaSuccess) {
-        dim3 g((unsigned)std::min<int64_t>(cdv(k, 32), 1024), (unsigned)std::min<int64_t>(cdv(n, 32), 1024));
-        k_transpose<T><<<g, dim3(32, 8), 0, s>>>(k, n, sum, k, M, n);
-        e = cudaGetLastError();
-      }
-      return e;
-    }
-  }
-  Operand<T> a{Q, ldq, nullptr, 0};
-  Operand<T> b{A, lda, nullptr, 0};
-  const int nz = gemm_splits((int)m, p.splits);
-  EpiArgs<T> ep{nz > 1 ? P : M, n, k * n, nullptr, nullptr};
-  e = gemm_gather<T>((int)k, (int)n, (int)m, nz, true, a, b, kEpiStore, ep, nullptr, s);
-  if (e == cudaSuccess && nz > 1) e = splitk_reduce_ld<T>(k, (int)n, n, n, nz, k * n, P, M, nullptr, s);
+cudaError_t gemm_tn(int64_t M, int64_t N, int64_t K, const T* A, int64_t lda, const T* B, int64_t ldb, T* out,
+                    int64_t ldo, T* P, int splits, cudaStream_t s) {
+  Operand<T> a{A, lda, nullptr, 0};
+  Operand<T> b{B, ldb, nullptr, 0};
+  const int nz = gemm_splits((int)K, splits);
+  EpiArgs<T> ep{nz > 1 ? P : out, nz > 1 ? N : ldo, M * N, nullptr, nullptr};
+  cudaError_t e = gemm_gather<T>((int)M, (int)N, (int)K, nz, true, a, b, kEpiStore, ep, nullptr, s);
+  if (e == cudaSuccess && nz > 1) e = splitk_reduce_ld<T>(M, (int)N, N, ldo, nz, M * N, P, out, nullptr, s);
   return e;
 }
 
 // ------------------------------------------------------------ stable X
 struct StablePlan {
   QrScratch q;
-  QtaPlan qta;
+  int msplits = 1;
   size_t off_st, off_F, off_Q, off_M, off_MP, off_X, off_R, off_Ri, off_qr, total;
 };
 
@@ -653,7 +613,7 @@ template <typename T>
 void stable_layout(int64_t m, int64_t n, int64_t k, StablePlan* p) {
   const int sms = sm_count();
   qr_layout<T>(m, k, sms, &p->q);
-  p->qta = qta_plan<T>(m, n, k, sms);
+  p->msplits = qr_splits<T>(k, n, m, sms);
   size_t off = 0;
   auto take = [&](size_t b) {
     size_t at = off;
@@ -665,7 +625,7 @@ void stable_layout(int64_t m, int64_t n, int64_t k, StablePlan* p) {
   p->off_F = take((size_t)m * k * e);
   p->off_Q = take((size_t)m * k * e);
   p->off_M = take((size_t)k * n * e);
-  p->off_MP = take(p->qta.total);
+  p->off_MP = take(p->msplits > 1 ? (size_t)p->msplits * k * n * e : 0);
   p->off_X = take((size_t)k * n * e);
   p->off_R = take((size_t)k * k * e);
   p->off_Ri = take((size_t)cdv(k, kTriB) * kTriB * kTriB * e);
@@ -680,6 +640,7 @@ cudaError_t stable_x_run(const T* A, int64_t lda, int64_t m, int64_t n, const in
   T* F = reinterpret_cast<T*>(ws + p.off_F);
   T* Q = reinterpret_cast<T*>(ws + p.off_Q);
   T* M = reinterpret_cast<T*>(ws + p.off_M);
+  T* MP = reinterpret_cast<T*>(ws + p.off_MP);
   T* X = reinterpret_cast<T*>(ws + p.off_X);
   T* R = reinterpret_cast<T*>(ws + p.off_R);
   T* Ri = reinterpret_cast<T*>(ws + p.off_Ri);
@@ -690,7 +651,7 @@ cudaError_t stable_x_run(const T* A, int64_t lda, int64_t m, int64_t n, const in
   e = cudaGetLastError();
   if (e == cudaSuccess) e = qr_factor<T>(m, k, F, m, p.q, qws, st, s);
   if (e == cudaSuccess) e = qr_form_q<T>(m, k, F, m, Q, m, p.q, qws, s);
-  if (e == cudaSuccess) e = qta<T>(m, n, k, Q, m, A, lda, M, p.qta, ws + p.off_MP, st, s);  // M = Q^T A
+  if (e == cudaSuccess) e = gemm_tn<T>(k, n, m, Q, m, A, lda, M, n, MP, p.msplits, s);  // M = Q^T A
   if (e == cudaSuccess) e = tri_solve<T>(k, F, m, M, n, n, X, n, R, Ri, s);              // X = R^{-1} M
   if (e == cudaSuccess) {  // the caller's X (k x n, column-major) = X (k x n, row-major)
     dim3 g((unsigned)std::min<int64_t>(cdv(k, 32), 1024), (unsigned)std::min<int64_t>(cdv(n, 32), 1024));
@@ -703,8 +664,7 @@ cudaError_t stable_x_run(const T* A, int64_t lda, int64_t m, int64_t n, const in
 // ------------------------------------------------------------ CUR middle factor
 struct CurPlan {
   QrScratch qc, qr;  // QR of C = A(:, J) (m x k) and of R^T = A(I, :)^T (n x k)
-  QtaPlan qta;           // M1 = Qc^T A
-  int m2splits = 1;
+  int m1splits = 1, m2splits = 1;
   size_t off_st, off_Fc, off_Qc, off_Fr, off_Qr, off_M1, off_M1P, off_M2, off_M2P, off_Y, off_Z, off_R, off_Ri,
       off_qc, off_qr, total;
 };
@@ -723,14 +683,14 @@ void cur_layout(int64_t m, int64_t n, int64_t k, int kind, CurPlan* p) {
   if (kind == 0) {
     qr_layout<T>(m, k, sms, &p->qc);
     qr_layout<T>(n, k, sms, &p->qr);
-    p->qta = qta_plan<T>(m, n, k, sms);
+    p->m1splits = qr_splits<T>(k, n, m, sms);
     p->m2splits = qr_splits<T>(k, k, n, sms);
     p->off_Fc = take((size_t)m * k * e);
     p->off_Qc = take((size_t)m * k * e);
     p->off_Fr = take((size_t)n * k * e);
     p->off_Qr = take((size_t)n * k * e);
     p->off_M1 = take((size_t)k * n * e);
-    p->off_M1P = take(p->qta.total);
+    p->off_M1P = take(p->m1splits > 1 ? (size_t)p->m1splits * k * n * e : 0);
   } else {  // QR of the square A(I, J)
     qr_layout<T>(k, k, sms, &p->qc);
     p->m2splits = qr_splits<T>(k, k, k, sms);
@@ -768,6 +728,7 @@ cudaError_t cur_run(const T* A, int64_t lda, int64_t m, int64_t n, const int64_t
     T* Fr = reinterpret_cast<T*>(ws + p.off_Fr);
     T* Qr = reinterpret_cast<T*>(ws + p.off_Qr);
     T* M1 = reinterpret_cast<T*>(ws + p.off_M1);
+    T* M1P = reinterpret_cast<T*>(ws + p.off_M1P);
     if (e == cudaSuccess) {
       k_gather2<T><<<grid1(m * k), 256, 0, s>>>(m, k, A, lda, m, n, nullptr, J, 0, Fc, m, st);  // C = A(:, J)
       k_gather2<T><<<grid1(n * k), 256, 0, s>>>(k, n, A, lda, m, n, I, nullptr, 1, Fr, n, st);  // R^T = A(I, :)^T
@@ -777,7 +738,7 @@ cudaError_t cur_run(const T* A, int64_t lda, int64_t m, int64_t n, const int64_t
     if (e == cudaSuccess) e = qr_form_q<T>(m, k, Fc, m, Qc, m, p.qc, ws + p.off_qc, s);
     if (e == cudaSuccess) e = qr_factor<T>(n, k, Fr, n, p.qr, ws + p.off_qr, st, s);
     if (e == cudaSuccess) e = qr_form_q<T>(n, k, Fr, n, Qr, n, p.qr, ws + p.off_qr, s);
-    if (e == cudaSuccess) e = qta<T>(m, n, k, Qc, m, A, lda, M1, p.qta, ws + p.off_M1P, st, s);  // M1 = Qc^T A (k x n)
+    if (e == cudaSuccess) e = gemm_tn<T>(k, n, m, Qc, m, A, lda, M1, n, M1P, p.m1splits, s);  // M1 = Qc^T A (k x n)
     if (e == cudaSuccess) {  // M2 = M1 Qr (k x k, row-major): rows of M1 against columns of Qr, both along n
       Operand<T> a{M1, n, nullptr, 0};
       Operand<T> b{Qr, n, nullptr, 0};

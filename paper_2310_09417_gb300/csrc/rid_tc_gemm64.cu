@@ -245,11 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       TOut* o = out + blockIdx.z * zstride + (int64_t)m * ldo;
 #pragma unroll
       for (int i = 0; i < kBN; ++i)
-        if (n0 + i < N) {
-          const int en = eb[n0 + i];
-          // an exponent above every finite number's: the row or column holds NaN or Inf
-          o[n0 + i] = em > 1024 || en > 1024 ? (TOut)NAN : (TOut)fixed_to_double(hi[i], lo[i], em + en + 2 - 64);
-        }
+        if (n0 + i < N) o[n0 + i] = (TOut)fixed_to_double(hi[i], lo[i], em + eb[n0 + i] + 2 - 64);
     }
   }
   fence_before_sync();
@@ -795,42 +791,6 @@ cudaError_t gemm_f64emu(int M, int N, int K, const double* A, int64_t lda, const
                         cudaStream_t s) {
   return tcg::gemm_emu_gather<double, 7>(M, N, K, A, lda, aidx, B, ldb, boff, bidx, adig, arows, aexp, bdig, brows,
                                          bexp, colmax, kmax, out, ldo, zstride, splits, st, done, s);
-}
-
-// A^T B for two matrices whose columns are contiguous (the QR's Q^T A): both operands'
-// columns are rows of length K to the slicer.
-size_t gemm_f64emu_tn_bytes(int64_t M, int64_t N, int64_t K) {
-  return (size_t)256 * 4 + gemm_f64emu_digit_bytes(M, K) + gemm_f64emu_digit_bytes(N, K) + (size_t)(M + N) * 4;
-}
-
-int gemm_f64emu_tn_splits(int64_t M, int64_t N, int64_t K, int sms) { return tcg::splits_for<7>(M, N, K, sms, 16); }
-
-cudaError_t gemm_f64emu_tn(int64_t M, int64_t N, int64_t K, const double* A, int64_t lda, const double* B, int64_t ldb,
-                           void* ws, double* out, int64_t ldo, int64_t zstride, int splits, DevState* st,
-                           cudaStream_t s) {
-  const int64_t Kp = gemm_f64emu_kpad(K);
-  unsigned char* w = static_cast<unsigned char*>(ws);
-  auto take = [&](size_t bytes) {
-    unsigned char* at = w;
-    w += (bytes + 255) / 256 * 256;
-    return at;
-  };
-  auto ad = reinterpret_cast<__nv_bfloat16*>(take(gemm_f64emu_digit_bytes(M, K)));
-  auto bd = reinterpret_cast<__nv_bfloat16*>(take(gemm_f64emu_digit_bytes(N, K)));
-  auto ae = reinterpret_cast<int32_t*>(take((size_t)M * 4)), be = reinterpret_cast<int32_t*>(take((size_t)N * 4));
-  auto slice = [&](int64_t rows, const double* src, int64_t ld, __nv_bfloat16* d, int32_t* e) {
-    int64_t g = (rows * 32 + 255) / 256;
-    if (g > 8192) g = 8192;
-    tcg::k_slice_rows<double, 7><<<(int)g, 256, 0, s>>>((int)rows, (int)K, (int)Kp, Kp, src, ld, nullptr, d, rows * Kp,
-                                                        e, nullptr);
-    return cudaGetLastError();
-  };
-  cudaError_t e = slice(M, A, lda, ad, ae);
-  if (e == cudaSuccess) e = slice(N, B, ldb, bd, be);
-  if (e == cudaSuccess)
-    e = tcg::launch<7, double>((int)M, (int)N, (int)K, Kp, ad, M, ae, bd, N, be, out, ldo, zstride, splits, st, nullptr,
-                               s);
-  return e;
 }
 
 // ---- FP32 sketch on the tensor cores (3 digits per operand)
