@@ -185,14 +185,15 @@ static __device__ __noinline__ double sq_add_f64(double acc, float x) { return a
 static __device__ __noinline__ double sq_fold(double acc, float hi, float lo) { return acc + ((double)hi + (double)lo); }
 
 // x^2 added to a float-float sum for an FP32 x: the square's rounding error comes
-// exactly from an FMA (TwoProduct) and the sum's from TwoSum; |x| outside
-// [2^-63, 2^54) (tiny, subnormal, huge) and zeros take the FP64 sum, NaN / Inf
+// from an FMA (TwoProduct, exact from |x| = 2^-51 on) and the sum's from TwoSum.  |x| in
+// [2^-49, 2^54) goes there, and anything smaller once the sum has reached 2^-96: what it
+// loses, at most 2^-148, is below 2^-52 of that sum.  Other values take the FP64 sum, NaN / Inf
 // clear `finite`.  A few dozen squares stay within about 2^-45 relative before
 // they are folded into FP64.
 __device__ __forceinline__ void sq_add_f32(float x, float& hi, float& lo, double& acc, bool& finite) {
   const uint32_t bits = __float_as_uint(x);
   const uint32_t ex = (bits >> 23) & 0xFFu;
-  if (ex - 64u <= 116u) {
+  if (ex - 78u <= 102u || (ex < 78u && hi >= 0x1.0p-96f)) {
     const float p = __fmul_rn(x, x);
     const float e = fmaf(x, x, -p);
     sq_twosum(p, hi, lo);

@@ -6,8 +6,9 @@
 // squares of FP32, BF16 and E4M3 values are summed in float-float (TwoSum of
 // D. Knuth; an FMA recovers an FP32 square's rounding error) on packed pairs --
 // one f32x2 instruction serves two elements -- and folded into FP64 once per 128
-// elements of a thread.  A vector with a value whose square is not a normal FP32
-// number well below overflow (zeros are fine) takes the FP64 sum instead.
+// elements of a thread.  A vector whose squares come near overflow, or whose sum of
+// squares lies so low that what FP32 cannot hold of it counts, takes the FP64 sum
+// instead (zeros are fine).
 // FP64 input has no way around one FP64 FMA per element.
 // Each thread keeps several 16-byte loads in flight: one load per thread and a
 // four-way branch per element left the pass latency-bound.
@@ -66,7 +67,7 @@ struct SqSum {
   __device__ __forceinline__ void add_square_exact(f32x2 x) { add(mul2(x, x)); }  // x with <= 12 significant bits
   __device__ __forceinline__ void add_square(f32x2 x) {
     const f32x2 p = mul2(x, x);
-    const f32x2 em = fma2(mul2(x, pack2(-1.f, -1.f)), x, p);  // p - x^2, exact
+    const f32x2 em = fma2(mul2(x, pack2(-1.f, -1.f)), x, p);  // p - x^2, exact from |x| = 2^-51 on
     add(p);
     lo = sub2(lo, em);
   }
@@ -82,9 +83,13 @@ struct SqSum {
 };
 constexpr int kGroup = 64;  // squares per packed half before a fold
 
-// Exponent window of values summed in float-float: |x| in [2^-63, 2^54), as FP32 bit
-// patterns; u - 1 of a zero wraps to the largest value and passes.
-constexpr uint32_t kLowF32 = (64u << 23) - 1u, kHighF32 = 181u << 23;
+// Windows of values summed in float-float, as FP32 bit patterns: below 2^54 in magnitude.
+// BF16 and E4M3: no value but zero below 2^-63, where its square (exact from then on)
+// leaves the normal range; u - 1 of a zero wraps to the largest value and passes.
+// FP32: the largest of a vector at least 2^-49 (or all zero).  A square is exact with its
+// FMA residual from 2^-51 on; what smaller entries lose, at most 2^-149 each, is then
+// below 2^-49 of the vector's sum.
+constexpr uint32_t kLowF32 = 78u << 23, kHighF32 = 181u << 23;
 
 __device__ __forceinline__ void put_part(double acc, bool finite, double* part, DevState* st) {
   if (!finite) atomicOr(&st->err, kErrNonFinite);
@@ -183,15 +188,11 @@ __global__ void __launch_bounds__(kNormThreads)
   unsigned col = 0u;  // largest magnitude of this thread's part of the column
   auto vec = [&](const float4& w) {
     const float x[4] = {w.x, w.y, w.z, w.w};
-    uint32_t mx = 0u, mn = 0xFFFFFFFFu;
+    uint32_t mx = 0u;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t u = __float_as_uint(x[q]) & 0x7FFFFFFFu;
-      mx = max(mx, u);
-      mn = min(mn, u - 1u);
-    }
+    for (int q = 0; q < 4; ++q) mx = max(mx, __float_as_uint(x[q]) & 0x7FFFFFFFu);
     col = max(col, mx);
-    if (mx < kHighF32 && mn >= kLowF32) {
+    if (mx - kLowF32 < kHighF32 - kLowF32 || mx == 0u) {
       sum.add_square(pack2(x[0], x[1]));
       sum.add_square(pack2(x[2], x[3]));
     } else {
