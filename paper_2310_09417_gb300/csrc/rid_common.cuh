@@ -248,6 +248,29 @@ __device__ __forceinline__ ArgMax block_argmax(ArgMax a) {
   return r;
 }
 
+// ------------------------------------------------------------------ quotients
+// a / b rounded to nearest given r = 1 / b rounded to nearest: q = a r is within one ulp
+// of the quotient, a - b q is exact in an FMA, and the corrected q is the rounded
+// quotient unless b's significand is all ones (P. W. Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990).  `ok`: b is such
+// and far from the ends of the exponent range; an a that is not, and zeros, take the
+// division itself.  On GB300 an FP64 division is a chain of a dozen instructions at
+// sixty-four clocks each, this one of three.  FP32 divides.
+__device__ __forceinline__ bool recip_usable(double b) {
+  const unsigned hi = (unsigned)__double2hiint(b), e = (hi >> 20) & 0x7FFu;
+  return e - 523u <= 1000u && !((hi & 0xFFFFFu) == 0xFFFFFu && __double2loint(b) == -1);
+}
+__device__ __forceinline__ double divide_by(double a, double b, double r, bool ok) {
+  const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7FFu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7FFu;
+  if (ok && ea - 523u <= 1000u && ea + 500u >= eb) {
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+  }
+  return a / b;
+}
+__device__ __forceinline__ bool recip_usable(float) { return false; }
+__device__ __forceinline__ float divide_by(float a, float b, float, bool) { return a / b; }
+
 // ------------------------------------------------------------------ Gaussian rows
 // Philox4x64-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two 64x64
 // -> 128-bit products whose high halves are xored into the other words and the

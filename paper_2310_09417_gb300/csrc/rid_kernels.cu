@@ -733,29 +733,6 @@ __device__ __forceinline__ unsigned long long tagged(unsigned data, unsigned tag
   return ((unsigned long long)tag << 32) | data;
 }
 
-// a / b rounded to nearest given r = 1 / b rounded to nearest: q = a r is within one ulp
-// of the quotient, a - b q is exact in an FMA, and the corrected q is the rounded
-// quotient unless b's significand is all ones (P. W. Markstein, "Computation of
-// elementary functions on the IBM RISC System/6000 processor", 1990).  `ok`: b is such
-// and far from the ends of the exponent range; an a that is not, and zeros, take the
-// division itself.  On GB300 an FP64 division is a chain of a dozen instructions at
-// sixty-four clocks each, this one of three; the reciprocal is computed by the block that
-// publishes the row, while the others wait for it.
-__device__ __forceinline__ bool recip_usable(double b) {
-  const unsigned hi = (unsigned)__double2hiint(b), e = (hi >> 20) & 0x7FFu;
-  return e - 523u <= 1000u && !((hi & 0xFFFFFu) == 0xFFFFFu && __double2loint(b) == -1);
-}
-__device__ __forceinline__ double divide_by(double a, double b, double r, bool ok) {
-  const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7FFu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7FFu;
-  if (ok && ea - 523u <= 1000u && ea + 500u >= eb) {
-    const double q = a * r;
-    return fma(fma(-q, b, a), r, q);
-  }
-  return a / b;
-}
-__device__ __forceinline__ bool recip_usable(float) { return false; }
-__device__ __forceinline__ float divide_by(float a, float b, float, bool) { return a / b; }
-
 // Block 0's record of a pivot (a call: its FP64 conversion is not to be predicated code
 // of every warp).
 template <typename T>
@@ -772,7 +749,7 @@ __global__ void __launch_bounds__(kPanelThreads)
   using PW = PanelWords<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T prow[2][kPanelMaxW];
-  __shared__ T s_rcp[2];  // FP64: the pivot's reciprocal
+  __shared__ T s_rcp[2];  // FP64: the pivot's reciprocal, by the block that publishes the row while the others wait
   __shared__ int s_piv[2];
   __shared__ unsigned long long s_mag[kPanelThreads / 32];
   __shared__ int s_row[kPanelThreads / 32];

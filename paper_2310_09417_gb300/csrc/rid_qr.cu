@@ -351,7 +351,9 @@ __global__ void k_transpose(int64_t rows, int64_t cols, const T* __restrict__ in
 // eighths of a block's columns and rows: the FP64 pipe of one SM bounds the inverse,
 // so a block's columns are spread over eight CTAs.  A warp per column c of
 // X = Rb^{-1}: once X(l, c) is known every lane adds its term to the rows above (two
-// rows per lane), a product and two FMAs per row of the chain.
+// rows per lane).  X(l, c) is the quotient by R(l, l), rounded once: the reciprocals are
+// taken once per CTA and corrected (divide_by), so a row of the chain is a product and
+// four FMAs.
 constexpr int kTriParts = 8;
 constexpr int kTriThreads = 32 * kTriB / kTriParts;
 template <typename T>
@@ -370,17 +372,15 @@ __global__ void __launch_bounds__(kTriThreads)
     Rb[i][c] = (i < bs && c < bs && c >= i) ? (double)F[(b0 + i) + (int64_t)(b0 + c) * ld] : 0.0;
   }
   __syncthreads();
-  if (threadIdx.x < kTriB) {
-    const double d = Rb[threadIdx.x][threadIdx.x];
-    s_inv[threadIdx.x] = d != 0.0 ? 1.0 / d : 0.0;
-  }
+  if (threadIdx.x < kTriB) s_inv[threadIdx.x] = 1.0 / Rb[threadIdx.x][threadIdx.x];
   __syncthreads();
   const int lane = threadIdx.x & 31, c = (threadIdx.x >> 5) * kTriParts + part;
   double x0 = 0.0, x1 = 0.0;  // X(lane, c), X(lane + 32, c)
   if (c < bs) {
     double s0 = lane == c ? 1.0 : 0.0, s1 = lane + 32 == c ? 1.0 : 0.0;
     for (int l = c; l >= 0; --l) {
-      const double x = __shfl_sync(0xffffffffu, l < 32 ? s0 : s1, l & 31) * s_inv[l];
+      const double s = __shfl_sync(0xffffffffu, l < 32 ? s0 : s1, l & 31), d = Rb[l][l];
+      const double x = d != 0.0 ? divide_by(s, d, s_inv[l], recip_usable(d)) : 0.0;
       if (lane == l) x0 = x;
       if (lane + 32 == l) x1 = x;
       if (lane < l) s0 -= Rb[lane][l] * x;
