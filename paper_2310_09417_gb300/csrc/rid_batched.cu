@@ -178,6 +178,63 @@ struct Squares {
     return acc;
   }
 };
+// The squares of A as the CTA GEMM loads it, for ||A||_F.  A thread's loads depend on the
+// tile height, which the tuner picks by time, but the result must not: the squares go into
+// 2048 sums keyed by (row mod 128, k mod 8, k / 8 mod 2), each in ascending order of row
+// and k, four of them in every thread whatever BM is, and those are added up by key.
+constexpr int kSqRows = 128, kSqSums = kSqRows * 16;
+template <typename T, int BM>
+struct RowSquares {
+  static constexpr int kRows = BM >= 64 ? BM / 64 : 1;  // rows of a tile that a thread loads
+  static constexpr int kHalves = BM >= 64 ? 2 : 1;      // values of k / 8 mod 2 among its loads of a row
+  static constexpr int kLive = kRows * kHalves;         // sums that one tile feeds: the first of acc
+  static_assert(kSqSums == 4 * kNT && 4 / kLive * BM == kSqRows, "four sums per thread");
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  float hi[kLive] = {}, lo[kLive] = {};
+  int cnt = 0;
+  bool finite = true;
+  __device__ __forceinline__ void add(int i, T v) {  // load i of a K step
+    const int u = (i % kRows) * kHalves + (i / kRows) % kHalves;
+    if constexpr (sizeof(T) == 4) {
+      sq_add_f32(v, hi[u], lo[u], acc[u], finite);
+    } else {
+      finite = finite && (__double2hiint(v) & 0x7FF00000) != 0x7FF00000;
+      acc[u] = fma(v, v, acc[u]);
+    }
+  }
+  __device__ __forceinline__ void fold() {
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int u = 0; u < kLive; ++u) {
+        acc[u] = sq_fold(acc[u], hi[u], lo[u]);
+        hi[u] = lo[u] = 0.f;
+      }
+      cnt = 0;
+    }
+  }
+  __device__ __forceinline__ void end_step() {  // a K step adds two squares to each sum
+    if (sizeof(T) == 4 && (cnt += 2) == 64) fold();
+  }
+  __device__ __forceinline__ void end_tile() {  // the next tile feeds the next kLive sums
+    fold();
+    double t[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) t[j] = acc[(j + kLive) % 4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = t[j];
+  }
+  // After `tiles` tiles: this thread's sums to out[key].
+  __device__ __forceinline__ void put(double* out, int tiles) const {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int s = (j + tiles * kLive) & 3, u = s % kLive;
+      const int row = s / kLive * BM + (warp + 16 * (u / kHalves)) % (BM / 4) * 4 + (lane >> 3);
+      const int half = kHalves == 2 ? u % 2 : warp >> 3;
+      out[(row * 8 + (lane & 7)) * 2 + half] = acc[j];
+    }
+  }
+};
 struct NoSquares {};
 
 // ------------------------------------------------------------------ CTA GEMM
@@ -250,7 +307,8 @@ __device__ __forceinline__ void cta_gemm(int M, int N, int K, const T* abase, in
         if constexpr (!std::is_same<Sq, NoSquares>::value) {
           if (n0 == 0) {
 #pragma unroll
-            for (int i = 0; i < NA; ++i) sq.add(ra[i]);
+            for (int i = 0; i < NA; ++i) sq.add(i, ra[i]);
+            sq.end_step();
           }
         }
       };
@@ -284,6 +342,9 @@ __device__ __forceinline__ void cta_gemm(int M, int N, int K, const T* abase, in
         }
         if (k0 + kTK < K) store(buf ^ 1);
         __syncthreads();
+      }
+      if constexpr (!std::is_same<Sq, NoSquares>::value) {
+        if (n0 == 0) sq.end_tile();
       }
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
@@ -465,15 +526,17 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
       __syncthreads();
       om = sl.omega;
     }
-    Squares<T> e2s;
     if (t == 0) {
       // the first sketch G (n x b) = (Omega A)^T is the panel; ||A||_F^2 and finiteness come
       // with its one read of A
-      Squares<T> sq;
+      RowSquares<T, BM> sq;
       cta_gemm<T, BM, true>(n, b, m, A, lda, nullptr, om, p.mmax, nullptr, sh, sq,
                             [&](int r, int c, T v) { R(r, c) = v; });
+      double* const sums = reinterpret_cast<double*>(sh.As);  // the tiles are not in use
+      static_assert(sizeof(sh.As) + sizeof(sh.Bs) >= kSqSums * sizeof(double), "room for the sums");
+      sq.put(sums, (n + BM - 1) / BM);
       const int bad = __syncthreads_or(!sq.finite);
-      const double n2 = block_sum(sq.sum());
+      const double n2 = block_sum((sums[tid] + sums[tid + kNT]) + (sums[tid + 2 * kNT] + sums[tid + 3 * kNT]));
       if (tid == 0) sh.red = n2;
       __syncthreads();
       norm2 = sh.red;
@@ -496,10 +559,15 @@ __device__ void run_problem(const Params& p, const Problem& pr, Result& res, Slo
       // Schur complement S = G(act) - T(act, 0:tb) G(perm) and its FP64 norm
       const int32_t* act = sl.act[cur];
       cta_gemm<T, BM, false>(na, b, tb, X, ldx, act, sl.G, b, sl.perm, sh, none, [&](int r, int c, T v) {
-        const T s = sl.G[(int64_t)act[r] * b + c] - v;
-        R(r, c) = s;
-        e2s.add(s);
+        R(r, c) = sl.G[(int64_t)act[r] * b + c] - v;
       });
+      __syncthreads();
+      // in an order of its own, not the tile's; lanes along the rows as in the panel
+      Squares<T> e2s;
+      for (int g = warp; 32 * g < na; g += kNT / 32)
+        if (32 * g + lane < na)
+#pragma unroll 4
+          for (int c = 0; c < b; ++c) e2s.add(R(32 * g + lane, c));
       double e2 = block_sum(e2s.finite || sizeof(T) == 8 ? e2s.sum() : (double)INFINITY);
       if (tid == 0) sh.red = e2;
       __syncthreads();
