@@ -22,6 +22,10 @@
  *     at least the size the matching *_workspace_size query returns, aligned to
  *     256 bytes.  The workspace may be reused between calls, not shared by calls
  *     that run concurrently.
+ *   - The library allocates no page-locked memory, but for two small state records
+ *     (under 256 bytes in all) per host thread that calls id_adaptive: allocated on the
+ *     thread's first such call, which may therefore synchronise the device, and freed
+ *     when the thread ends.
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  Every entry
  *     point enqueues its work on `stream` and returns after that work has
  *     finished (the adaptive driver needs the stop decision on the host), so

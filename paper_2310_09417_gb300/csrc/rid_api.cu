@@ -23,6 +23,7 @@
 
 #include "randid.h"
 #include "rid_internal.h"
+#include "rid_posted.h"
 
 using namespace rid;
 
@@ -323,25 +324,28 @@ int make_plan(const id_matrix* A, const id_opts* o, int64_t k, int64_t l, Plan* 
     if (rid_rc_ != 0) return rid_rc_; \
   } while (0)
 
-// Two page-locked DevStates of the calling thread, freed with it: a call uses them from
-// its first posted state to its last read one, and calls of one thread follow each other.
-DevState* pinned_states() {
-  struct Holder {
-    DevState* p = nullptr;
-    ~Holder() {
-      if (p != nullptr) cudaFreeHost(p);
-    }
-  };
-  static thread_local Holder h;
-  if (h.p == nullptr) {
-    void* q = nullptr;
-    if (cudaHostAlloc(&q, 2 * sizeof(DevState), cudaHostAllocPortable) == cudaSuccess)
-      h.p = static_cast<DevState*>(q);
-    else
-      cudaGetLastError();  // no page-locked memory: the caller waits for every round
+// The CUDA runtime as PostedStates uses it; a failed call leaves no error behind.
+struct CudaRt {
+  using Stream = cudaStream_t;
+  using Event = cudaEvent_t;
+  static bool ok(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess;
   }
-  return h.p;
-}
+  static void* alloc_pinned(size_t bytes) {
+    void* p = nullptr;
+    return ok(cudaHostAlloc(&p, bytes, cudaHostAllocPortable)) ? p : nullptr;
+  }
+  static void free_pinned(void* p) { cudaFreeHost(p); }
+  static bool create(Event* e) { return ok(cudaEventCreateWithFlags(e, cudaEventDisableTiming)); }
+  static void destroy(Event e) { cudaEventDestroy(e); }
+  static bool copy(void* dst, const void* src, size_t bytes, Stream s) {
+    return ok(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, s));
+  }
+  static bool record(Event e, Stream s) { return ok(cudaEventRecord(e, s)); }
+  static bool wait(Event e) { return ok(cudaEventSynchronize(e)); }
+  static void wait_stream(Stream s) { cudaStreamSynchronize(s); }
+};
 
 // One call's state and the steps of the method.
 template <typename T>
@@ -407,8 +411,6 @@ class Engine {
   }
   ~Engine() {
     for (cudaEvent_t e : events_) cudaEventDestroy(e);
-    for (cudaEvent_t e : posted_)
-      if (e != nullptr) cudaEventDestroy(e);
   }
 
   // Algorithm 1's loop, launched one round ahead of its stop test: while the host waits
@@ -421,7 +423,7 @@ class Engine {
     RID_TRY(start());
     int64_t tb = 0, na = p_.n, t = 0, sketched = 0, gstart = 0;
     const int64_t b = p_.b;
-    const bool ahead = !o_.profile && can_post();
+    const bool ahead = !o_.profile && posted_.open();
     bool full = false;
     for (;;) {
       if (t >= sketched) {
@@ -625,25 +627,15 @@ class Engine {
     return 0;
   }
 
-  // The state as of decision t, copied to page-locked memory in stream order; read_state
-  // waits for that copy only, not for what was queued after it.
-  bool can_post() {
-    pinned_ = pinned_states();
-    for (cudaEvent_t& e : posted_)
-      if (pinned_ != nullptr && e == nullptr && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess)
-        pinned_ = nullptr;
-    return pinned_ != nullptr;
-  }
+  // The state as of decision t, with the pass count and the active list of that round.
   int post_state(int64_t t) {
-    RID_TRY(cuda(cudaMemcpyAsync(&pinned_[t & 1], st_, sizeof(DevState), cudaMemcpyDeviceToHost, s_)));
-    RID_TRY(cuda(cudaEventRecord(posted_[t & 1], s_)));
+    if (!posted_.post(t, st_, s_)) return ID_ERR_CUDA;
     posted_passes_[t & 1] = passes_;
     posted_cur_[t & 1] = cur_;
     return 0;
   }
   int read_state(int64_t t) {
-    RID_TRY(cuda(cudaEventSynchronize(posted_[t & 1])));
-    h_ = pinned_[t & 1];
+    if (!posted_.read(t, &h_)) return ID_ERR_CUDA;
     if (h_.done) {  // what was queued past the stop did nothing
       passes_ = posted_passes_[t & 1];
       cur_ = posted_cur_[t & 1];
@@ -1030,8 +1022,7 @@ class Engine {
   int64_t phase_launches_[kNumPhases];
   std::vector<cudaEvent_t> events_;
   std::vector<int> pending_;
-  DevState* pinned_ = nullptr;  // two posted states (can_post)
-  cudaEvent_t posted_[2] = {nullptr, nullptr};
+  PostedStates<DevState, CudaRt> posted_;
   int32_t posted_passes_[2] = {0, 0};
   int posted_cur_[2] = {0, 0};
 };
