@@ -423,12 +423,13 @@ const char* id_status_string(int status);
 
 /* Self-test of the failure handling; the paper has no counterpart.  Every
    device-side wait of the library gives up after a bounded time (4 s of the
-   GPU's global timer).  That covers the grid barrier of the cooperative LUPP
-   panel and the mbarrier waits of the tensor-core kernels.  The wait records a
-   timeout and lets its kernel exit, so the call returns ID_ERR_TIMEOUT and the
-   CUDA context stays usable.  This entry runs, with the same device helpers,
-   one wait that nothing can satisfy: which = 0 the grid barrier, which = 1 an
-   mbarrier wait.
+   GPU's global timer).  That covers the grid barrier of the cooperative QR
+   panel, the LUPP panel's poll for the other blocks' candidates and the mbarrier
+   waits of the tensor-core kernels.  The wait records a timeout and lets its
+   kernel exit, so the call returns ID_ERR_TIMEOUT and the CUDA context stays
+   usable.  This entry runs, with the same device helpers, one wait that nothing
+   can satisfy: which = 0 the grid barrier, 1 an mbarrier wait, 2 the panel's
+   poll, 3 the mbarrier wait of a CTA pair.
    ws: DEVICE scratch of at least 256 bytes, 256-aligned, owned by the caller.
    Synchronises the stream and takes about 4 s.  Returns ID_ERR_TIMEOUT when
    the wait gave up as designed.  ID_OK would mean the wait was satisfied.

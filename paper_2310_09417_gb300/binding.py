@@ -558,9 +558,10 @@ def id_batched(As: list, tol: float, *, block: int = 32, relative: bool = True, 
 
 
 def selftest_timeout(which: int, device="cuda", stream=None) -> int:
-    """Run one device wait that nothing satisfies (0: the LUPP panel's grid
-    barrier, 1: an mbarrier wait of the tensor-core kernels) and return the
-    library's status: ERR_TIMEOUT when the bounded wait gave up as designed."""
+    """Run one device wait that nothing satisfies (0: the QR panel's grid barrier, 1: an
+    mbarrier wait of the tensor-core kernels, 2: the LUPP panel's poll, 3: the mbarrier
+    wait of a CTA pair) and return the library's status: ERR_TIMEOUT when the bounded
+    wait gave up as designed."""
     ws = torch.empty(256, dtype=torch.uint8, device=device)
     return _call(ws.device, "id_selftest_timeout", which, ws.data_ptr(), ws.numel(), _stream(stream, ws.device))
 

@@ -108,6 +108,30 @@ __device__ __forceinline__ bool grid_barrier(unsigned* ctr, unsigned target, Dev
   return s_ok != 0;
 }
 
+// The limit of a warp's poll on words that another block stores (no barrier object): after
+// kWaitLimitNs, or once another wait of the call has given up, every lane gets true.  The
+// kernels queued behind this one then return at once (done).
+struct PollLimit {
+  unsigned spins = 0;
+  uint64_t t0 = 0;
+  __device__ __forceinline__ bool gave_up(DevState* st) {
+    if ((++spins & 255u) != 0u) return false;
+    int bad = 0;
+    if ((threadIdx.x & 31) == 0) {
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      if (ld_acquire_u32(&st->err) & kErrTimeout) {
+        bad = 1;
+      } else if (now - t0 > kWaitLimitNs) {
+        atomicOr(&st->err, kErrTimeout);
+        st->done = 1;
+        bad = 1;
+      }
+    }
+    return __shfl_sync(0xffffffffu, bad, 0) != 0;
+  }
+};
+
 // ------------------------------------------------------------------ reductions
 // (value, index) argmax: larger |value| wins, ties go to the smaller index;
 // index < 0 means "no candidate".

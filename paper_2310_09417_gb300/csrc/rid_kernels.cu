@@ -754,7 +754,9 @@ __global__ void __launch_bounds__(kPanelThreads)
   __shared__ unsigned long long s_mag[kPanelThreads / 32];
   __shared__ int s_row[kPanelThreads / 32];
   const int nb = gridDim.x, bid = blockIdx.x, tid = threadIdx.x;
-  if (st->done) return;  // set before the launch or never during it: uniform over the grid
+  // set before the launch: uniform over the grid.  During it only a block whose wait ran
+  // out sets it, and then every block leaves without its results
+  if (st->done) return;
   const int lane = tid & 31, wid = tid >> 5;
   constexpr int nw = kPanelThreads / 32;
   const int r0 = bid * chunk;
@@ -842,24 +844,7 @@ __global__ void __launch_bounds__(kPanelThreads)
   auto collect = [&](int c) {
     const unsigned tag = tag0 + (unsigned)c;
     const unsigned long long* mw = xchg + (size_t)(c & 1) * nb * PW::kMag;
-    unsigned spins = 0;
-    uint64_t t0 = 0;
-    auto gave_up = [&]() {  // uniform over the warp
-      if ((++spins & 255u) != 0u) return false;
-      int bad = 0;
-      if (lane == 0) {
-        const uint64_t now = globaltimer_ns();
-        if (t0 == 0) t0 = now;
-        if (ld_acquire_u32(&st->err) & kErrTimeout) {
-          bad = 1;
-        } else if (now - t0 > kWaitLimitNs) {
-          atomicOr(&st->err, kErrTimeout);
-          st->done = 1;  // the kernels queued after this launch return at once
-          bad = 1;
-        }
-      }
-      return __shfl_sync(0xffffffffu, bad, 0) != 0;
-    };
+    PollLimit limit;
     // The row of block q: its words, and whether all of them are this step's.
     unsigned long long g = 0ull, ih = 0ull, il = 0ull, rh[kPanelMaxW / 32], rl[kPanelMaxW / 32];
     auto load_row = [&](int q) {
@@ -922,7 +907,7 @@ __global__ void __launch_bounds__(kPanelThreads)
       }
       const bool complete = __all_sync(0xffffffffu, all) != 0;
       if (!kGuess && !complete) {
-        if (gave_up()) {
+        if (limit.gave_up(st)) {
           if (lane == 0) s_piv[c & 1] = -2;
           return;
         }
@@ -940,7 +925,7 @@ __global__ void __launch_bounds__(kPanelThreads)
       while (complete && !kGuess && !there) {
         load_row(q);
         there = row_ready();
-        if (!there && gave_up()) {
+        if (!there && limit.gave_up(st)) {
           if (lane == 0) s_piv[c & 1] = -2;
           return;
         }
@@ -964,7 +949,7 @@ __global__ void __launch_bounds__(kPanelThreads)
         return;
       }
       guess = q;
-      if (gave_up()) {
+      if (limit.gave_up(st)) {
         if (lane == 0) s_piv[c & 1] = -2;
         return;
       }
