@@ -27,7 +27,7 @@ struct DevState {
   int32_t rounds;         // estimates computed
   uint32_t err;           // kErr* bits
   uint32_t zero_pivots;   // exactly zero pivot columns met
-  uint32_t bar[2];        // grid-barrier arrival counters, one per launch parity
+  uint32_t bar;           // arrival counter of the self-test's grid barrier
 };
 static_assert(sizeof(DevState) <= 256, "DevState must fit its 256-byte slot");
 
@@ -36,14 +36,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-__device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ unsigned atom_add_acqrel_u32(unsigned* p, unsigned v) {
-  unsigned old;
-  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
 }
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
@@ -133,65 +125,12 @@ struct PollLimit {
 };
 
 // ------------------------------------------------------------------ reductions
-// (value, index) argmax: larger |value| wins, ties go to the smaller index;
-// index < 0 means "no candidate".
-struct ArgMax {
-  double v;
-  int idx;
-};
-__device__ __forceinline__ ArgMax argmax_pick(ArgMax a, ArgMax b) {
-  if (b.idx < 0) return a;
-  if (a.idx < 0) return b;
-  if (b.v > a.v || (b.v == a.v && b.idx < a.idx)) return b;
-  return a;
-}
-__device__ __forceinline__ ArgMax warp_argmax(ArgMax a) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    ArgMax o;
-    o.v = __shfl_down_sync(0xffffffffu, a.v, off);
-    o.idx = __shfl_down_sync(0xffffffffu, a.idx, off);
-    a = argmax_pick(a, o);
-  }
-  return a;
-}
-
-// Block-wide maximum of 64-bit keys (0 = no candidate), by integer compares.
-__device__ __forceinline__ unsigned long long block_max_u64(unsigned long long k) {
-  __shared__ unsigned long long s_k[32];
-  __shared__ unsigned long long s_res64;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const unsigned long long o = __shfl_down_sync(0xffffffffu, k, off);
-    k = o > k ? o : k;
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) s_k[warp] = k;
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    unsigned long long b = lane < nw ? s_k[lane] : 0ull;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const unsigned long long o = __shfl_down_sync(0xffffffffu, b, off);
-      b = o > b ? o : b;
-    }
-    if (lane == 0) s_res64 = b;
-  }
-  __syncthreads();
-  const unsigned long long r = s_res64;
-  __syncthreads();
-  return r;
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
   return v;
 }
 
-// Block-wide sum of one double per thread (blockDim.x multiple of 32, <= 1024);
-// result valid in thread 0.
 // Sum of squares in float-float: t = x * x is exact in FP32 when x has at most 12
 // significant bits (BF16, E4M3) and its square is a normal FP32 number; TwoSum
 // (Knuth) keeps the rounding error of hi + t in lo, so a group of a few dozen
@@ -230,6 +169,8 @@ __device__ __forceinline__ void sq_add_f32(float x, float& hi, float& lo, double
   }
 }
 
+// Block-wide sum of one double per thread (blockDim.x multiple of 32, <= 1024);
+// result valid in thread 0.
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double s_part[32];
   v = warp_sum(v);
@@ -243,32 +184,6 @@ __device__ __forceinline__ double block_sum(double v) {
     r = lane < nw ? s_part[lane] : 0.0;
     r = warp_sum(r);
   }
-  return r;
-}
-
-// Block-wide argmax (every thread gets the result); blockDim.x multiple of 32.
-__device__ __forceinline__ ArgMax block_argmax(ArgMax a) {
-  __shared__ double s_v[32];
-  __shared__ int s_i[32];
-  __shared__ ArgMax s_res;
-  a = warp_argmax(a);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    s_v[warp] = a.v;
-    s_i[warp] = a.idx;
-  }
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = (blockDim.x + 31) >> 5;
-    ArgMax b;
-    b.v = lane < nw ? s_v[lane] : -1.0;
-    b.idx = lane < nw ? s_i[lane] : -1;
-    b = warp_argmax(b);
-    if (lane == 0) s_res = b;
-  }
-  __syncthreads();
-  const ArgMax r = s_res;
-  __syncthreads();
   return r;
 }
 

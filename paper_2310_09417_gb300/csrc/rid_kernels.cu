@@ -20,27 +20,6 @@
 
 namespace rid {
 
-// Element conversions (round to nearest) shared by the FP64/FP32/BF16 instantiations.
-template <typename T>
-__device__ __forceinline__ T from_double(double x) {
-  return static_cast<T>(x);
-}
-template <>
-__device__ __forceinline__ __nv_bfloat16 from_double<__nv_bfloat16>(double x) {
-  return __double2bfloat16(x);
-}
-template <>
-__device__ __forceinline__ __nv_fp8_e4m3 from_double<__nv_fp8_e4m3>(double x) {
-  __nv_fp8_e4m3 q;
-  q.__x = __nv_cvt_double_to_fp8(x, __NV_SATFINITE, __NV_E4M3);  // nearest even, saturating at +-448
-  return q;
-}
-template <typename T>
-__device__ __forceinline__ double to_double(T x) {
-  return static_cast<double>(x);
-}
-__device__ __forceinline__ double to_double(__nv_bfloat16 x) { return static_cast<double>(__bfloat162float(x)); }
-
 // ============================================================ Gaussian rows
 // FP32 / BF16 / E4M3 outputs are converted from the FP32 value directly (the same
 // rounding of the same value as through FP64, without FP64 instructions: GB300
@@ -77,7 +56,7 @@ __device__ __forceinline__ void gaussian_quad(uint64_t seed, int64_t row0, I e, 
     box_muller(x2, x3, z[2], z[3]);
 #pragma unroll
     for (int j = 0; j < 4; ++j)
-      if (j < lim) o[j] = from_double<T>(z[j]);
+      if (j < lim) o[j] = z[j];
   } else {
     float f[4];
     if constexpr (sizeof(T) <= 2) {  // BF16 / E4M3 output: Box-Muller in FP32 on 24-bit uniforms
@@ -1425,7 +1404,8 @@ cudaError_t make_n<double>(int na, int bt, const double* S, int64_t lds, const d
         na, bt, S, lds, Linv, pivmark, act, Nbuf, X, ldx, tb, piv, pivorig, done);
     return cudaGetLastError();
   };
-  if (warps1 >= 16 * (int64_t)sms) return run(std::integral_constant<int, 4>());  // four warps per scheduler's SM at least
+  // at four columns a warp still one warp per scheduler, four per SM
+  if (warps1 >= 16 * (int64_t)sms) return run(std::integral_constant<int, 4>());
   if (warps1 >= 8 * (int64_t)sms) return run(std::integral_constant<int, 2>());
   return run(std::integral_constant<int, 1>());
 }
@@ -1529,8 +1509,7 @@ __global__ void k_init_state(DevState* st, int32_t* act, int32_t* pivmark, int64
     st->rounds = 0;
     st->err = 0u;
     st->zero_pivots = 0u;
-    st->bar[0] = 0u;
-    st->bar[1] = 0u;
+    st->bar = 0u;
   }
   if (i < n) {
     act[i] = (int32_t)i;

@@ -20,7 +20,7 @@ namespace {
 
 // One block adds one arrival; the target asks for two, so the counter never
 // reaches it and the barrier can only time out.
-__global__ void k_unsatisfied_grid_barrier(DevState* st) { grid_barrier(&st->bar[0], 2u, st); }
+__global__ void k_unsatisfied_grid_barrier(DevState* st) { grid_barrier(&st->bar, 2u, st); }
 
 // An mbarrier that expects one arrival, which never comes: phase 0 never
 // completes and the wait can only time out.  Nothing asynchronous was issued
