@@ -436,8 +436,10 @@ const char* id_status_string(int status);
    Other returns: -1 for another `which`, ID_ERR_WORKSPACE, ID_ERR_CUDA. */
 int id_selftest_timeout(int which, void* ws, size_t ws_bytes, void* stream);
 
-/* Bytes of the library-owned device buffer behind id_fixed_rank_noalloc. */
-#define ID_NOALLOC_SCRATCH_BYTES ((size_t)64 << 20)
+/* Bytes of the library-owned device buffer behind id_fixed_rank_noalloc: 64 MiB for the
+   method's matrices and 1 MiB for the words through which the LUPP panel's blocks exchange
+   candidates (at most 0.7 MiB). */
+#define ID_NOALLOC_SCRATCH_BYTES ((size_t)65 << 20)
 
 /* id_fixed_rank for callers that cannot allocate device memory.  The paper has
    no counterpart: this is a deployment variant of id_fixed_rank.
