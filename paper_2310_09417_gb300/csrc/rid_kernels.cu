@@ -105,11 +105,10 @@ cudaError_t gaussian_rows(uint64_t seed, int64_t row0, int64_t rows, int64_t m, 
 // memory.  The bound is the FP64 pipe, about two FMAs per clock per SM: a warp
 // instruction occupies it for sixteen clocks, so shared memory and L2 are idle
 // whatever the tile, and the tile only has to give every SM the same share: 32 x 32
-// with many tiles, 16 x 16 with few (dgemm_small_tiles).  64 x 64 and 128 x 64 tiles
-// left most SMs without work where the products are small or narrow.  Measured: the
-// sketch of 600 x 400 with 56 rows 326 -> 34 us, of 4000 x 1000 with 64 rows 519 -> 401
-// (the rate of the FP64 pipe), the Schur product of 1000
-// rows and up to 384 pivots 271 -> 42, the QR's V^T C (4000 x 96 by 32) 570 -> 12.
+// with many tiles, 16 x 16 with few (dgemm_small_tiles).  Larger tiles leave most SMs
+// without work where a product is small or narrow.  Measured against 128 x 64 and 64 x 64
+// tiles: the sketch of 4000 x 1000 with 64 rows 519 -> 401 us (the rate of the FP64
+// pipe), of 600 x 400 with 56 rows 326 -> 34.
 // Every entry is summed over k in increasing order, one FMA per term, within its split:
 // the tile does not change a bit.
 constexpr int kDK = 16;

@@ -55,7 +55,7 @@ struct PanelRows {
 // block's own products, on the sum over blocks that every block repeats, and on the
 // update; kQrRows rows per block balance them.  Lanes run along the columns, so no
 // product is spent on shuffles.  32 columns of 4000 rows: 246 us with v formed and two
-// divisions per column, 233 us with one division and v left to the end.
+// divisions one after the other, 233 us with both in one instruction and v left to the end.
 constexpr int kQrRows = 64;
 
 // |x| in [2^-600, 2^600): 1 / x and its products with values up to 2^400 are normal.
@@ -352,7 +352,8 @@ __global__ void k_transpose(int64_t rows, int64_t cols, const T* __restrict__ in
 // X = Rb^{-1}: once X(l, c) is known every lane adds its term to the rows above (two
 // rows per lane).  X(l, c) is the quotient by R(l, l), rounded once: the reciprocals are
 // taken once per CTA and corrected (divide_by), so a row of the chain is a product and
-// four FMAs.
+// four FMAs.  k = 96: 139 us with a thread per column that divides, 28 here (19 with the
+// reciprocal alone, one rounding more).
 constexpr int kTriParts = 8;
 constexpr int kTriThreads = 32 * kTriB / kTriParts;
 template <typename T>

@@ -75,7 +75,8 @@ static_assert(kChunkSteps % kDual == 0, "a stage never straddles an exact chunk"
 // sums, hence their bits), so an item is only a few chunks long: as a CTA of its own it
 // paid for its start, its first loads and the conversion and store of its 8192 sums with
 // the tensor cores idle.  Here the loads and MMAs of the next item run meanwhile.
-// 128 rows of a 40000 x 10000 matrix (40 splits): 1.90 -> 1.56 ms.
+// 128 rows of a 40000 x 10000 matrix (40 splits): 1.90 -> 1.56 ms, and 1.50 since the
+// conversions at the ends of the exponent range are calls.
 __global__ void __launch_bounds__(kThreads, 1)
     k_sketch_f64emu(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_w,
                     const int32_t* __restrict__ colexp, int n, int rows, int K, int kchunk, int xtiles, int ytiles,

@@ -335,7 +335,12 @@ int tc_sketch_splits(int64_t m, int64_t n, int64_t rows, int sms) {
 cudaError_t tc_sketch_bf16(const void* A, int64_t lda, int64_t m, int64_t n, const void* W, int64_t ldw,
                            int64_t rows, float* out, int64_t out_ld, int64_t zstride, int splits, DevState* st,
                            const int32_t* done, cudaStream_t s) {
-  // more than one block of 64 rows: CTA pairs; one block: a CTA per tile, two CTAs per SM
+  // More than one block of 64 rows: CTA pairs; one block: a CTA per tile, two CTAs per SM.
+  // The pair's 256 rows pay from 192 on (512 rows of 100000 x 20000: 1.53 ms against
+  // 1.68).  Two blocks cost about the same either way, a call at 65 to 128 rows: 0.84 - 0.89
+  // ms with the pair and with the one-block kernel at 100000 x 20000; at 20000 x 4000 the
+  // one-block kernel is ahead (128 rows: 139 us against 154).  Passes of two blocks are
+  // what blocks_per_pass = 2 or blocks of 65 to 128 rows ask for, not a default.
   const bool pair = rows > tc::kBN1;
   CUtensorMap ma, mw;
   if (!tc::make_map_bf16(&ma, A, m, n, lda, tc::kBM)) return cudaErrorInvalidValue;
